@@ -388,8 +388,17 @@ static cudaError_t row_go(const Geom& g, const FftPlan& pz, const float2* tw, co
                         : row_go13<MODE, KC, MC, false>(g, pz, tw, maps, x, t, out, st);
 }
 
-cudaError_t launch_row(const Geom& g, RowMode mode, const FftPlan& pz, const float2* tw_z, const float2* maps,
+// Whether the passes of this shape keep t interleaved (k_col_il.cu): the size-specialised
+// passes of four basis images in their default column variant.
+bool t_interleaved(const Geom& g) {
+  const long long rows = (long long)g.S * g.C * std::max(g.ny, g.nz);
+  return g.K == 4 && g.colvar == 0 && g.nz % 4 == 0 && il_rb(g.ny) > 0 && row_il_supported(g) &&
+         rows + g.S * (long long)g.C <= 0x7fffffffLL && tma_encode_fn() != nullptr;
+}
+
+cudaError_t launch_row(const Geom& g, RowMode mode, bool il, const FftPlan& pz, const float2* tw_z, const float2* maps,
                        const float2* x, float2* t, float2* out, cudaStream_t st) {
+  if (il) return launch_row_il(g, mode, il_rb(g.ny), tw_z, maps, x, t, out, st);
   const cudaError_t ef = launch_row_fast(g, mode, tw_z, maps, x, t, out, st);
   if (ef != cudaErrorNotSupported) return ef;
   const bool k4 = g.K <= 4, m1 = g.M == 1;

@@ -62,6 +62,13 @@ enum RowMode : int {
   ROW_ADJ = 1   // out[m][k] = sum_c conj(S'_{c,m}) IDFT_z( t[c][k] )
 };
 
+// Column passes on the interleaved intermediate (k_col_il.cu)
+enum IlPass : int {
+  IL_NORMAL = 0,      // DFT_y, Psi, IDFT_y in place on t
+  IL_ADJ_PLANAR = 1,  // A^H y column pass from planar projected k-space [S][C][K][ny][nz]
+  IL_ADJ = 2          // the same from k-space in t's own layout (may be t itself)
+};
+
 struct FistaArgs {
   float mu;      // step
   float tau;     // mu * lambda
@@ -82,7 +89,9 @@ cudaError_t launch_psi_build(const Geom& g, const float* phi, const uint8_t* mas
                              unsigned* lam_psi_bits, cudaStream_t st);
 cudaError_t launch_project(const Geom& g, const float* phi, const uint8_t* mask, const float2* y_te,
                            float2* y_proj, cudaStream_t st);
-cudaError_t launch_row(const Geom& g, RowMode mode, const FftPlan& pz, const float2* tw_z, const float2* maps,
+// il: t has the interleaved layout of k_col_il.cu (only where t_interleaved(g))
+bool t_interleaved(const Geom& g);
+cudaError_t launch_row(const Geom& g, RowMode mode, bool il, const FftPlan& pz, const float2* tw_z, const float2* maps,
                        const float2* x, float2* t, float2* out, cudaStream_t st);
 cudaError_t launch_col(const Geom& g, ColMode mode, const FftPlan& py, const float2* tw_y, const float* psi,
                        const float* phi, const uint8_t* mask, const float2* tin, float2* tout, cudaStream_t st);
@@ -150,6 +159,14 @@ cudaError_t launch_wait_selftest(int* err, unsigned long long limit_ns, cudaStre
 cudaError_t launch_col_normal_pr(const Geom& g, const float2* tw_y, const float* psi, float2* t, cudaStream_t st);
 cudaError_t launch_col_normal_tc(const Geom& g, const float2* tw_y, const float* psi, float2* t, cudaStream_t st);
 cudaError_t launch_col_normal_tma(const Geom& g, const float2* tw_y, const float* psi, float2* t, cudaStream_t st);
+// the interleaved intermediate (layout: k_col_il.cu); il_rb: 0 where a column length has no such pass
+int il_rb(int ny);
+bool row_il_supported(const Geom& g);
+// trb: il_rb(ny)
+cudaError_t launch_row_il(const Geom& g, RowMode mode, int trb, const float2* tw_z, const float2* maps,
+                          const float2* x, float2* t, float2* out, cudaStream_t st);
+cudaError_t launch_col_il(const Geom& g, IlPass pass, const float2* tw_y, const float* psi, const float2* in, float2* t,
+                          cudaStream_t st);
 // A^H y column pass on TMA tiles (K <= 4, nz % 8 == 0, ny = 16 R1 <= 256; tin may equal tout)
 cudaError_t launch_col_adj_tma(const Geom& g, const float2* tw_y, const float2* tin, float2* tout, cudaStream_t st);
 

@@ -1,0 +1,40 @@
+"""Column and row passes over their whole range of lengths: every size-specialised column and row
+length with one and two map sets, enough tiles that a CTA's run crosses column tiles, against the
+FP64 oracle.  Tolerance 1e-5: a float32 2D DFT pair accumulates log2(ny nz) <= 18 roundings of
+6e-8 per stage, plus the K-term Psi and C-term coil sums, about 1e-6."""
+import numpy as np
+import pytest
+
+import oracle as O
+
+from t2sh_cases import crandn
+from test_gpu_parity import OP_TOL, T, c64, host, make_plan, nrmse, random_problem  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+LENGTHS = [
+    # S, ny, nz, C, M
+    (2, 48, 256, 3, 1),
+    (30, 64, 64, 7, 2),      # several column tiles per CTA, short lines
+    (3, 96, 192, 2, 1),
+    (2, 128, 96, 3, 2),
+    (40, 160, 48, 5, 1),     # runs that cross column tiles at 48-point rows
+    (1, 192, 160, 2, 2),
+    (1, 240, 64, 5, 1),
+    (9, 256, 128, 4, 1),
+    (5, 260, 240, 6, 1),     # two tensor-map boxes per column
+]
+
+
+@pytest.mark.parametrize("S,ny,nz,C,M", LENGTHS)
+def test_passes_of_four_images(T, S, ny, nz, C, M):  # noqa: F811
+    rng, phi, mask, maps = random_problem(ny + nz + C, S, ny, nz, C, 12, 4, M)
+    x, y = crandn(rng, S, M, 4, ny, nz), crandn(rng, S, C, 4, ny, nz)
+    with make_plan(T, phi, mask, maps, block=8) as p:
+        got_n, got_a = host(p.normal_op(c64(x))), host(p.adjoint(c64(y), T.KSPACE_PROJ))
+        p.sync()
+    psi = O.space_time_kernel(mask, phi)
+    xs, ys = (a.astype(np.complex64).astype(np.complex128) for a in (x, y))
+    for s in {0, S // 2, S - 1}:
+        assert nrmse(got_n[s], O.normal(xs[s], maps[s], psi)) < OP_TOL
+        assert nrmse(got_a[s], O.adjoint_projected(ys[s], maps[s])) < OP_TOL
