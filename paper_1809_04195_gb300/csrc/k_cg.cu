@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_dir(long long L, const float2
 
 // out[s] += sum_{c,t,n} P_t(n) |y_{s,c,t}(n)|^2 of T-form k-space y [S][C][T][N] (float64
 // per thread: a diagnostic reduction, not on the iteration path)
-__global__ void __launch_bounds__(kCgThreads) k_masked_energy(long long N, int C, int T, const uint8_t* __restrict__ mask,
+__global__ void __launch_bounds__(kCgThreads) k_masked_energy(long long N, int C, int T, const unsigned* __restrict__ bits,
                                                              const float2* __restrict__ y, double* out) {
   const int s = blockIdx.y;
   const long long L = (long long)C * T * N;
@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(kCgThreads) k_masked_energy(long long N, int C
   double acc = 0.0;
   for (long long n = (long long)blockIdx.x * kCgThreads + threadIdx.x; n < N; n += (long long)gridDim.x * kCgThreads)
     for (int t = 0; t < T; ++t)
-      if (mask[(long long)t * N + n])
+      if ((bits[(long long)(t >> 5) * N + n] >> (t & 31)) & 1u)
         for (int c = 0; c < C; ++c) {
           const float2 v = ys[((long long)c * T + t) * N + n];
           acc += (double)v.x * v.x + (double)v.y * v.y;
@@ -227,10 +227,10 @@ cudaError_t launch_cg_step(const Geom& g, float2* x, float2* r, const float2* p,
   return cudaGetLastError();
 }
 
-cudaError_t launch_masked_energy(const Geom& g, const uint8_t* mask, const float2* y, double* out, cudaStream_t st) {
+cudaError_t launch_masked_energy(const Geom& g, const unsigned* bits, const float2* y, double* out, cudaStream_t st) {
   const long long N = (long long)g.ny * g.nz;
   const unsigned gx = (unsigned)std::min<long long>((N + kCgThreads - 1) / kCgThreads, 64);
-  k_masked_energy<<<dim3(gx, (unsigned)g.S), kCgThreads, 0, st>>>(N, g.C, g.T, mask, y, out);
+  k_masked_energy<<<dim3(gx, (unsigned)g.S), kCgThreads, 0, st>>>(N, g.C, g.T, bits, y, out);
   return cudaGetLastError();
 }
 

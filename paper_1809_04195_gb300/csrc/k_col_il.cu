@@ -345,6 +345,109 @@ __global__ void __launch_bounds__(Il<N>::THREADS, 1)
   }
 }
 
+// Forward column pass of A: DFT_y of t, centring signs and scale.  PROJ: then Psi N, to planar
+// k-space `out` [S][C][K][ny][nz]; otherwise in place, row f of t holding frequency f (a tile is
+// read whole before it is written).
+template <int N, bool PROJ>
+__global__ void __launch_bounds__(Il<N>::THREADS, 1)
+    k_col_il_fwd(Geom g, const float2* __restrict__ tw_g, const float* __restrict__ psi, const float2* t, float2* out,
+                 long long ntiles, int ngroups) {
+  using L = Il<N>;
+  constexpr int RA = L::RA, RB = L::RB, GT = L::GT;
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  const int grp = threadIdx.x / GT, gt = threadIdx.x - grp * GT;
+  unsigned char* buf = smem_raw + (size_t)grp * L::TILE;
+  const int nz = g.nz;
+  const int rowlen = 4 * nz;
+  const IlItem it = il_item(gt);
+  const bool wa = (gt & ~31) / 8 < RB;
+  const bool on = it.j < RB;
+  const int ja = RA == RB || on ? it.j : 0;
+  unsigned char* pa[4];
+  unsigned char* pb[4];
+  int gs[4];
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    pa[m] = buf + ja * 128 + ((m + 2 * it.kp + ja) & 3) * 32 + it.w * 8;
+    pb[m] = buf + it.j * RB * 128 + ((m + 2 * it.kp + it.j) & 3) * 32 + it.w * 8;
+    gs[m] = ((m + 2 * it.kp + ja) & 3) * 4;
+  }
+  float2* tws = reinterpret_cast<float2*>(smem_raw + (size_t)ngroups * L::TILE);
+  for (int i = threadIdx.x; i < N; i += blockDim.x) tws[i] = tw_g[(i / RA) * (i % RA)];
+  const float2* tw = tws + it.j;
+  __syncthreads();
+  const int ntz = nz / 4;
+  const float scale = g.gsign * g.inv_sqrt_n * parity_sign(it.j + it.w);  // RA and 4 zt are even
+  const long long step = (long long)gridDim.x * ngroups;
+  for (long long tile = (long long)blockIdx.x * ngroups + grp; tile < ntiles; tile += step) {
+    const long long sc = tile / ntz;
+    const int zt = (int)(tile - sc * ntz);
+    if (wa) {
+      const float2* gp = t + (sc * N + ja) * rowlen + zt * 16 + it.w;
+      float2 a[2][RA];
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int q = 0; q < RA; ++q) a[k][q] = gp[(long long)(q * RB) * rowlen + gs[(k + q) & 3]];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        dft_r<RA, false>(a[k]);
+        if (on) {
+#pragma unroll
+          for (int q = 0; q < RA; ++q) sts2(pa[(k + q) & 3], q * RB * 128, a[k][q]);
+        }
+      }
+    }
+    group_sync<GT>(grp);
+    float2 b[2][RB];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+#pragma unroll
+      for (int j = 0; j < RB; ++j) b[k][j] = lds2(pb[(k + j) & 3], j * 128);
+#pragma unroll
+      for (int j = 1; j < RB; ++j) b[k][j] = twiddle_mul<false>(b[k][j], tw[j * RA]);
+      dft_r<RB, false>(b[k]);
+    }
+    group_sync<GT>(grp);  // the buffer is read: the next tile may be written
+#pragma unroll
+    for (int k2 = 0; k2 < RB; ++k2) {
+      const int f = it.j + RA * k2;
+      const float2 va = cscale(b[0][k2], scale), vb = cscale(b[1][k2], scale);
+      if constexpr (PROJ) {
+        float2 vc, vd;  // the other pair, from the lane that holds it
+        vc.x = __shfl_xor_sync(0xffffffffu, va.x, 4);
+        vc.y = __shfl_xor_sync(0xffffffffu, va.y, 4);
+        vd.x = __shfl_xor_sync(0xffffffffu, vb.x, 4);
+        vd.y = __shfl_xor_sync(0xffffffffu, vb.y, 4);
+        const float2 v[4] = {it.kp ? vc : va, it.kp ? vd : vb, it.kp ? va : vc, it.kp ? vb : vd};
+        const float* pp = psi + (long long)f * nz + zt * 4 + it.w;
+        const long long NN = (long long)N * nz;
+        // rows 2 kp and 2 kp + 1 of the upper triangle 00 01 02 03 11 12 13 22 23 33
+        const float n = (float)(N * nz);
+        const float p02 = pp[2 * NN] * n, p03 = pp[3 * NN] * n, p12 = pp[5 * NN] * n, p13 = pp[6 * NN] * n;
+        const float d0 = pp[(it.kp ? 7 : 0) * NN] * n, d1 = pp[(it.kp ? 8 : 1) * NN] * n,
+                    d2 = pp[(it.kp ? 9 : 4) * NN] * n;
+        const float r0[4] = {it.kp ? p02 : d0, it.kp ? p12 : d1, it.kp ? d0 : p02, it.kp ? d1 : p03};
+        const float r1[4] = {it.kp ? p03 : d1, it.kp ? p13 : d2, it.kp ? d1 : p12, it.kp ? d2 : p13};
+        float2 u0 = cscale(v[0], r0[0]), u1 = cscale(v[0], r1[0]);
+#pragma unroll
+        for (int l = 1; l < 4; ++l) {
+          u0 = make_float2(fmaf(r0[l], v[l].x, u0.x), fmaf(r0[l], v[l].y, u0.y));
+          u1 = make_float2(fmaf(r1[l], v[l].x, u1.x), fmaf(r1[l], v[l].y, u1.y));
+        }
+        float2* o = out + ((sc * 4 + 2 * it.kp) * N + f) * nz + zt * 4 + it.w;
+        o[0] = u0;
+        o[NN] = u1;
+      } else {
+        float2* o = out + (sc * N + f) * rowlen + zt * 16 + it.w;
+        const int rot = 2 * it.kp + f % RB + f / RB;
+        o[(rot & 3) * 4] = va;
+        o[((rot + 1) & 3) * 4] = vb;
+      }
+    }
+  }
+}
+
 // groups per CTA: all of them once the tiles fill the chip, fewer while SMs would stay idle
 template <int N>
 int il_groups(long long ntiles, int nsm) {
@@ -391,6 +494,20 @@ cudaError_t il_adj(const Geom& g, const float2* tw, const float2* in, float2* t,
   return cudaGetLastError();
 }
 
+template <int N, bool PROJ>
+cudaError_t il_fwd(const Geom& g, const float2* tw, const float* psi, const float2* t, float2* out, cudaStream_t st) {
+  using L = Il<N>;
+  const long long nsc = (long long)g.S * g.C, ntiles = nsc * (g.nz / 4);
+  int nsm = 0;
+  cudaError_t e = smem_optin((const void*)k_col_il_fwd<N, PROJ>, (int)L::smem_adj(L::G));
+  if (e == cudaSuccess) e = sm_count(&nsm);
+  if (e != cudaSuccess) return e;
+  const int ng = il_groups<N>(ntiles, nsm);
+  const int grid = (int)std::min<long long>(nsm, (ntiles + ng - 1) / ng);
+  k_col_il_fwd<N, PROJ><<<grid, ng * L::GT, L::smem_adj(ng), st>>>(g, tw, psi, t, out, ntiles, ng);
+  return cudaGetLastError();
+}
+
 template <int N>
 cudaError_t il_go(const Geom& g, IlPass pass, const float2* tw, const float* psi, const float2* in, float2* t,
                   cudaStream_t st) {
@@ -398,6 +515,8 @@ cudaError_t il_go(const Geom& g, IlPass pass, const float2* tw, const float* psi
     case IL_NORMAL: return il_normal<N>(g, tw, psi, t, st);
     case IL_ADJ_PLANAR: return il_adj<N, false>(g, tw, in, t, st);
     case IL_ADJ: return il_adj<N, true>(g, tw, in, t, st);
+    case IL_FWD_PROJ: return il_fwd<N, true>(g, tw, psi, in, t, st);
+    case IL_FWD_RAW: return il_fwd<N, false>(g, tw, psi, in, t, st);
   }
   return cudaErrorInvalidValue;
 }

@@ -243,12 +243,10 @@ __global__ void __launch_bounds__(kFftThreads, 1) k_col_normal(Geom g, FftPlan p
   cp_async_wait<0>();
 }
 
-// Column pass.  tin/tout are [S][C][K][ny][nz] (may alias); FWD_TE writes yout
-// [S][C][T][ny][nz] and FWD_PROJ writes yout [S][C][K][ny][nz].
+// Column pass.  tin/tout are [S][C][K][ny][nz] (may alias).
 template <int MODE, int KC, bool R13>
 __global__ void __launch_bounds__(kFftThreads) k_col(Geom g, FftPlan py, const float2* __restrict__ tw_g,
-                                                const float* __restrict__ psi, const float* __restrict__ phi,
-                                                const uint8_t* __restrict__ mask, const float2* tin, float2* tout,
+                                                const float* __restrict__ psi, const float2* tin, float2* tout,
                                                 int W) {
   extern __shared__ float2 smem[];
   const int ny = g.ny, nz = g.nz, N = ny * nz, K = g.K;
@@ -316,39 +314,17 @@ __global__ void __launch_bounds__(kFftThreads) k_col(Geom g, FftPlan py, const f
       __syncthreads();
       if (MODE == COL_FWD_PROJ) return;
       fft_lines<true, R13>(buf, ld, K * wc, py, tw);
-    } else {  // COL_FWD_TE
-      for (int q = threadIdx.x; q < npt; q += kFftThreads) {
-        const int w = q % wc, y = q / wc;
-        const long long n = (long long)y * nz + z0 + w;
-        const float sg = g.gsign * g.inv_sqrt_n * parity_sign(y + z0 + w);
-        float2 v[KC];
-#pragma unroll
-        for (int k = 0; k < KC; ++k) v[k] = (k < K) ? cscale(buf[(k * wc + w) * ld + y], sg) : make_float2(0.f, 0.f);
-        float2* yb = tout + ((long long)(s * g.C + c) * g.T) * N + n;
-        for (int tt = 0; tt < g.T; ++tt) {
-          float2 a = make_float2(0.f, 0.f);
-          if (mask[(long long)tt * N + n]) {
-#pragma unroll
-            for (int k = 0; k < KC; ++k)
-              if (k < K) {
-                const float ph = __ldg(phi + tt * K + k);
-                a.x = fmaf(ph, v[k].x, a.x);
-                a.y = fmaf(ph, v[k].y, a.y);
-              }
-          }
-          yb[(long long)tt * N] = a;
-        }
-      }
-      return;
     }
   }
-  // store the columns back (COL_NORMAL, COL_ADJ_DATA)
+  // store the columns back (COL_NORMAL, COL_ADJ_DATA, COL_FWD_RAW)
   float2* ob = tout + ((long long)(s * g.C + c) * K) * N + z0;
   for (int e = threadIdx.x; e < nel; e += kFftThreads) {
     const int w = e % wc;
     const int rest = e / wc;
     const int y = rest % ny, k = rest / ny;
-    ob[(long long)k * N + (long long)y * nz + w] = buf[(k * wc + w) * ld + y];
+    float2 v = buf[(k * wc + w) * ld + y];
+    if (MODE == COL_FWD_RAW) v = cscale(v, g.gsign * g.inv_sqrt_n * parity_sign(y + z0 + w));
+    ob[(long long)k * N + (long long)y * nz + w] = v;
   }
 }
 
@@ -415,8 +391,8 @@ cudaError_t launch_row(const Geom& g, RowMode mode, bool il, const FftPlan& pz, 
 }
 
 template <int MODE, int KC, bool R13>
-static cudaError_t col_go13(const Geom& g, const FftPlan& py, const float2* tw, const float* psi, const float* phi,
-                            const uint8_t* mask, const float2* tin, float2* tout, cudaStream_t st) {
+static cudaError_t col_go13(const Geom& g, const FftPlan& py, const float2* tw, const float* psi,
+                            const float2* tin, float2* tout, cudaStream_t st) {
   const int W = col_cols_per_cta(g);
   const size_t sm = sizeof(float2) * (((g.ny + 1) & ~1) + (size_t)g.K * W * (g.ny + 1));
   {
@@ -424,15 +400,15 @@ static cudaError_t col_go13(const Geom& g, const FftPlan& py, const float2* tw, 
     if (e != cudaSuccess) return e;
   }
   dim3 grid((g.nz + W - 1) / W, g.C, g.S);
-  k_col<MODE, KC, R13><<<grid, kFftThreads, sm, st>>>(g, py, tw, psi, phi, mask, tin, tout, W);
+  k_col<MODE, KC, R13><<<grid, kFftThreads, sm, st>>>(g, py, tw, psi, tin, tout, W);
   return cudaGetLastError();
 }
 
 template <int MODE, int KC>
-static cudaError_t col_go(const Geom& g, const FftPlan& py, const float2* tw, const float* psi, const float* phi,
-                          const uint8_t* mask, const float2* tin, float2* tout, cudaStream_t st) {
-  return plan_has13(py) ? col_go13<MODE, KC, true>(g, py, tw, psi, phi, mask, tin, tout, st)
-                        : col_go13<MODE, KC, false>(g, py, tw, psi, phi, mask, tin, tout, st);
+static cudaError_t col_go(const Geom& g, const FftPlan& py, const float2* tw, const float* psi,
+                          const float2* tin, float2* tout, cudaStream_t st) {
+  return plan_has13(py) ? col_go13<MODE, KC, true>(g, py, tw, psi, tin, tout, st)
+                        : col_go13<MODE, KC, false>(g, py, tw, psi, tin, tout, st);
 }
 
 template <int KC, bool R13>
@@ -464,7 +440,7 @@ static cudaError_t col_normal_go(const Geom& g, const FftPlan& py, const float2*
 }
 
 cudaError_t launch_col(const Geom& g, ColMode mode, const FftPlan& py, const float2* tw_y, const float* psi,
-                       const float* phi, const uint8_t* mask, const float2* tin, float2* tout, cudaStream_t st) {
+                       const float2* tin, float2* tout, cudaStream_t st) {
   const bool k4 = g.K <= 4;
   switch (mode) {
     case COL_NORMAL:
@@ -488,14 +464,14 @@ cudaError_t launch_col(const Geom& g, ColMode mode, const FftPlan& py, const flo
       const cudaError_t et = launch_col_adj_tma(g, tw_y, tin, tout, st);
       if (et != cudaErrorNotSupported) return et;
     }
-      return k4 ? col_go<COL_ADJ_DATA, 4>(g, py, tw_y, psi, phi, mask, tin, tout, st)
-                : col_go<COL_ADJ_DATA, 8>(g, py, tw_y, psi, phi, mask, tin, tout, st);
+      return k4 ? col_go<COL_ADJ_DATA, 4>(g, py, tw_y, psi, tin, tout, st)
+                : col_go<COL_ADJ_DATA, 8>(g, py, tw_y, psi, tin, tout, st);
     case COL_FWD_PROJ:
-      return k4 ? col_go<COL_FWD_PROJ, 4>(g, py, tw_y, psi, phi, mask, tin, tout, st)
-                : col_go<COL_FWD_PROJ, 8>(g, py, tw_y, psi, phi, mask, tin, tout, st);
-    case COL_FWD_TE:
-      return k4 ? col_go<COL_FWD_TE, 4>(g, py, tw_y, psi, phi, mask, tin, tout, st)
-                : col_go<COL_FWD_TE, 8>(g, py, tw_y, psi, phi, mask, tin, tout, st);
+      return k4 ? col_go<COL_FWD_PROJ, 4>(g, py, tw_y, psi, tin, tout, st)
+                : col_go<COL_FWD_PROJ, 8>(g, py, tw_y, psi, tin, tout, st);
+    case COL_FWD_RAW:
+      return k4 ? col_go<COL_FWD_RAW, 4>(g, py, tw_y, psi, tin, tout, st)
+                : col_go<COL_FWD_RAW, 8>(g, py, tw_y, psi, tin, tout, st);
   }
   return cudaErrorInvalidValue;
 }

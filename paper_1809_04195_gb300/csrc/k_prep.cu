@@ -4,6 +4,8 @@
 
 namespace t2sh {
 
+constexpr int kPsiThreads = 64;  // many small CTAs: these kernels are bound by latency
+
 // S'_{c,m}(y, z) = (-1)^(y+z) S_{c,m}(y, z): the image-side half of the FFT centring
 // (FFTmod, Sec. IV.A) folded into the maps once.  Also the per-pixel largest
 // eigenvalue of S(p)^H S(p) (C x M), max-reduced over all pixels into *lam_bits
@@ -44,13 +46,92 @@ __global__ void __launch_bounds__(kThreads) k_maps_prep(Geom g, const float2* in
   if ((threadIdx.x & 31) == 0 && lam > 0.0f) atomicMax(lam_bits, __float_as_uint(lam));
 }
 
+// Largest eigenvalue of the real symmetric K x K matrix acc (upper triangle): its eigenvector v in
+// float32 (Jacobi on the matrix scaled by its trace, so the pivots are in the normal range), then
+// in float64 w = A v and w.w / v.w.  That quotient errs by the square of v's error (1e-13 of the
+// trace; where the two largest eigenvalues agree to 1e-6, by less than a float32 rounding), and a
+// full float64 Jacobi per point costs 20 times the rest of the kernel on a chip whose float64 rate
+// is 1/60 of float32: 64x48, T = 32: 263 -> 22 us; 256x160, T = 80: 527 -> 41 us.
+template <int KC>
+__device__ __forceinline__ float sym_lam_max(const double (&acc)[KC][KC]) {
+  double tr = 0.0;
+#pragma unroll
+  for (int k = 0; k < KC; ++k) tr += acc[k][k];
+  if (!(tr > 0.0)) return 0.f;
+  const double inv = 1.0 / tr;
+  float ar[KC][KC], ai[KC][KC], vr[KC][KC], vi[KC][KC];
+#pragma unroll
+  for (int k = 0; k < KC; ++k)
+#pragma unroll
+    for (int l = k; l < KC; ++l) {
+      ar[k][l] = ar[l][k] = (float)(acc[k][l] * inv);
+      ai[k][l] = ai[l][k] = 0.f;
+    }
+  herm_jacobi_rounds<float, KC>(ar, ai, vr, vi, KC == 4 ? 6 : 9);
+  float m = ar[0][0], v[KC];
+#pragma unroll
+  for (int k = 0; k < KC; ++k) v[k] = vr[k][0];
+#pragma unroll
+  for (int i = 1; i < KC; ++i) {
+    const bool up = ar[i][i] > m;
+    m = up ? ar[i][i] : m;
+#pragma unroll
+    for (int k = 0; k < KC; ++k) v[k] = up ? vr[k][i] : v[k];
+  }
+  double ww = 0.0, vw = 0.0;
+#pragma unroll
+  for (int k = 0; k < KC; ++k) {
+    double w = 0.0;
+#pragma unroll
+    for (int l = 0; l < KC; ++l) w += (k <= l ? acc[k][l] : acc[l][k]) * (double)v[l];
+    ww += w * w;
+    vw += (double)v[k] * w;
+  }
+  return vw > 0.0 ? (float)(ww / vw) : 0.f;
+}
+
+__device__ __forceinline__ void warp_max_bits(float lam, unsigned* bits) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) lam = fmaxf(lam, __shfl_xor_sync(0xffffffffu, lam, o));
+  if ((threadIdx.x & 31) == 0 && lam > 0.0f) atomicMax(bits, __float_as_uint(lam));
+}
+
+// acc += the outer products of the basis rows in `word` (bit i: echo t0 + i), in float64
+template <int KC>
+__device__ __forceinline__ void psi_add(double (&acc)[KC][KC], const float* sphi, int K, int t0, unsigned word) {
+  while (word) {
+    const float* ph = sphi + (t0 + __ffs(word) - 1) * K;
+    word &= word - 1;
+    double d[KC];
+#pragma unroll
+    for (int k = 0; k < KC; ++k) d[k] = k < K ? (double)ph[k] : 0.0;
+#pragma unroll
+    for (int k = 0; k < KC; ++k)
+#pragma unroll
+      for (int l = k; l < KC; ++l)
+        if (l < K) acc[k][l] += d[k] * d[l];
+  }
+}
+
+// the 32 echoes t0 .. t0 + 31 of point n as a bit word
+__device__ __forceinline__ unsigned mask_word(const uint8_t* __restrict__ mask, int T, int N, int t0, int n) {
+  unsigned word = 0;
+  const int m = min(32, T - t0);
+#pragma unroll 16
+  for (int i = 0; i < m; ++i) word |= (mask[(long long)(t0 + i) * N + n] ? 1u : 0u) << i;
+  return word;
+}
+
 // Psi(n)_{kl} = sum_t Phi_{tk} P_t(n) Phi_{tl} in float64, stored as float32 upper
 // triangle (p = 0.. for k <= l, row by row) scaled by 1/N so the unnormalised
-// DFT pair needs no other scaling, SoA [P][ny][nz].  Also lambda_max(Psi(n)) max-reduced.
+// DFT pair needs no other scaling, SoA [P][ny][nz].  Also the sampling pattern as bit words
+// bits[T / 32][n] (nullable) and lambda_max(Psi(n)) max-reduced into *lam_bits.
+// A thread adds only its own samples: a warp takes as many steps as its densest point has
+// samples, not T.
 template <int KC>
-__global__ void __launch_bounds__(kThreads) k_psi_build(Geom g, const float* __restrict__ phi,
+__global__ void __launch_bounds__(kPsiThreads) k_psi_build(Geom g, const float* __restrict__ phi,
                                                       const uint8_t* __restrict__ mask, float* __restrict__ psi,
-                                                      unsigned* lam_bits) {
+                                                      unsigned* __restrict__ bits, unsigned* lam_bits) {
   extern __shared__ float sphi[];  // [T][K]
   for (int i = threadIdx.x; i < g.T * g.K; i += blockDim.x) sphi[i] = phi[i];
   __syncthreads();
@@ -63,15 +144,10 @@ __global__ void __launch_bounds__(kThreads) k_psi_build(Geom g, const float* __r
     for (int k = 0; k < KC; ++k)
 #pragma unroll
       for (int l = 0; l < KC; ++l) acc[k][l] = 0.0;
-    for (int t = 0; t < g.T; ++t) {
-      if (mask[(long long)t * N + n]) {
-        const float* ph = sphi + t * g.K;
-#pragma unroll
-        for (int k = 0; k < KC; ++k)
-#pragma unroll
-          for (int l = k; l < KC; ++l)
-            if (l < g.K) acc[k][l] += (double)ph[k] * (double)ph[l];
-      }
+    for (int t0 = 0; t0 < g.T; t0 += 32) {
+      const unsigned word = mask_word(mask, g.T, N, t0, n);
+      if (bits) bits[(long long)(t0 >> 5) * N + n] = word;
+      psi_add<KC>(acc, sphi, g.K, t0, word);
     }
     const double inv_n = 1.0 / (double)N;
     int p = 0;
@@ -83,57 +159,164 @@ __global__ void __launch_bounds__(kThreads) k_psi_build(Geom g, const float* __r
           psi[(long long)p * N + n] = (float)(acc[k][l] * inv_n);
           ++p;
         }
-    double ar[KC][KC], ai[KC][KC], vr[KC][KC], vi[KC][KC];
-#pragma unroll
-    for (int k = 0; k < KC; ++k)
-#pragma unroll
-      for (int l = 0; l < KC; ++l) {
-        const bool in = (k < g.K && l < g.K);
-        ar[k][l] = in ? (k <= l ? acc[k][l] : acc[l][k]) : 0.0;
-        ai[k][l] = 0.0;
-      }
-    herm_jacobi<double, KC>(ar, ai, vr, vi, 12);
-    double m = 0.0;
-#pragma unroll
-    for (int k = 0; k < KC; ++k) m = fmax(m, ar[k][k]);
-    lam = (float)m;
+    lam = sym_lam_max<KC>(acc);
   }
-  for (int o = 16; o > 0; o >>= 1) lam = fmaxf(lam, __shfl_xor_sync(0xffffffffu, lam, o));
-  if ((threadIdx.x & 31) == 0 && lam > 0.0f) atomicMax(lam_bits, __float_as_uint(lam));
+  warp_max_bits(lam, lam_bits);
 }
 
-// ytil[s][c][k][n] = sum_t Phi_{tk} P_t(n) y[s][c][t][n]
-template <int KC>
-__global__ void __launch_bounds__(kThreads) k_project(Geom g, const float* __restrict__ phi,
-                                                    const uint8_t* __restrict__ mask,
+// Place of (image k, point n = y nz + z) of per-coil data: planar [K][ny][nz], or t's interleaved
+// layout (k_col_il.cu) where trb > 0
+struct TePlace {
+  long long base;
+  int step;  // image stride (planar)
+  int rot;   // slot of image 0 (interleaved)
+  bool il;
+  __device__ __forceinline__ TePlace(const Geom& g, int trb, long long sc, int n) {
+    il = trb > 0;
+    const int N = g.ny * g.nz;
+    if (il) {
+      const int y = n / g.nz, z = n - y * g.nz;
+      base = (sc * g.ny + y) * (4LL * g.nz) + (z >> 2) * 16 + (z & 3);
+      rot = y % trb + y / trb;
+      step = 0;
+    } else {
+      base = sc * g.K * (long long)N + n;
+      step = N;
+      rot = 0;
+    }
+  }
+  __device__ __forceinline__ long long at(int k) const {
+    return base + (il ? (long long)(((k + rot) & 3) * 4) : (long long)k * step);
+  }
+};
+
+__device__ __forceinline__ float2 ld_sample(const float2* p) {
+  float2 v;
+  asm("ld.global.nc.L1::no_allocate.L2::64B.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
+
+// ytil[s][c][k][n] = sum_t Phi_{tk} P_t(n) y[s][c][t][n], planar or interleaved.  A thread walks
+// the set bits of its point only, NS samples of NP (slice, coil) planes at a time, so eight
+// independent loads are in flight instead of one behind one mask byte.  The samples are
+// scattered 8-byte values (5 % of the plane), so the kernel is bound by what DRAM fetches for them:
+// with the default 128-byte fetches 54 % of the whole array (2.0 GB of 3.8, 342 us), with 64-byte
+// ones 281 us.  240x128, C = 8, T = 80 at 5 %, 24 slices: 785 us before.
+template <int KC, int NP, int NS>
+__global__ void __launch_bounds__(kThreads) k_project(Geom g, int trb, const float* __restrict__ phi,
+                                                    const unsigned* __restrict__ bits,
                                                     const float2* __restrict__ y, float2* __restrict__ out) {
   extern __shared__ float sphi[];
   for (int i = threadIdx.x; i < g.T * g.K; i += blockDim.x) sphi[i] = phi[i];
   __syncthreads();
   const int N = g.ny * g.nz;
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  const int sc = blockIdx.y;  // s * C + c
   if (n >= N) return;
-  float2 acc[KC];
+  const long long nsc = (long long)g.S * g.C, plane = (long long)g.T * N;
+  for (long long sc0 = (long long)blockIdx.y * NP; sc0 < nsc; sc0 += (long long)gridDim.y * NP) {
+    const int np = (int)min((long long)NP, nsc - sc0);
+    float2 acc[NP][KC];
 #pragma unroll
-  for (int k = 0; k < KC; ++k) acc[k] = make_float2(0.f, 0.f);
-  const float2* yb = y + (long long)sc * g.T * N + n;
-  for (int t = 0; t < g.T; ++t) {
-    if (mask[(long long)t * N + n]) {
-      const float2 v = yb[(long long)t * N];
-      const float* ph = sphi + t * g.K;
+    for (int i = 0; i < NP; ++i)
 #pragma unroll
-      for (int k = 0; k < KC; ++k)
-        if (k < g.K) {
-          acc[k].x = fmaf(ph[k], v.x, acc[k].x);
-          acc[k].y = fmaf(ph[k], v.y, acc[k].y);
+      for (int k = 0; k < KC; ++k) acc[i][k] = make_float2(0.f, 0.f);
+    const float2* yb = y + sc0 * plane + n;
+    for (int t0 = 0; t0 < g.T; t0 += 32) {
+      unsigned word = bits[(long long)(t0 >> 5) * N + n];
+      while (word) {
+        int t[NS];
+        float2 v[NS][NP];
+#pragma unroll
+        for (int u = 0; u < NS; ++u) {
+          t[u] = word ? t0 + __ffs(word) - 1 : -1;
+          word &= word - 1;
+#pragma unroll
+          for (int i = 0; i < NP; ++i)
+            v[u][i] = t[u] >= 0 && i < np ? ld_sample(yb + i * plane + (long long)t[u] * N) : make_float2(0.f, 0.f);
         }
+#pragma unroll
+        for (int u = 0; u < NS; ++u) {
+          if (t[u] >= 0) {
+            const float* ph = sphi + t[u] * g.K;
+#pragma unroll
+            for (int k = 0; k < KC; ++k)
+              if (k < g.K) {
+                const float f = ph[k];
+#pragma unroll
+                for (int i = 0; i < NP; ++i) {
+                  acc[i][k].x = fmaf(f, v[u][i].x, acc[i][k].x);
+                  acc[i][k].y = fmaf(f, v[u][i].y, acc[i][k].y);
+                }
+              }
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      if (i < np) {
+        const TePlace pl(g, trb, sc0 + i, n);
+#pragma unroll
+        for (int k = 0; k < KC; ++k)
+          if (k < g.K) out[pl.at(k)] = acc[i][k];
+      }
     }
   }
-  float2* ob = out + (long long)sc * g.K * N + n;
+}
+
+// y[s][c][t][n] = P_t(n) sum_k Phi_{tk} v_k(n) for every echo, v (planar or interleaved) the
+// transformed and scaled coefficients of the coil.  A pure streaming write (the T echoes are K / T
+// times the input): one thread owns two neighbouring points and writes 16 bytes per echo, whole
+// 512-byte runs per warp, so it is bound by HBM writes.  256x160, C = 12, T = 80, 8 slices
+// (2.5 GB): 400 us, 0.93 of the measured copy bandwidth; 745 us when the column pass wrote the
+// echoes itself in 64-byte runs, 445 us with the column pass now.
+template <int KC>
+__global__ void __launch_bounds__(kThreads) k_expand_te(Geom g, int trb, const float* __restrict__ phi,
+                                                      const unsigned* __restrict__ bits,
+                                                      const float2* __restrict__ v, float2* __restrict__ y) {
+  extern __shared__ float sphi[];
+  for (int i = threadIdx.x; i < g.T * g.K; i += blockDim.x) sphi[i] = phi[i];
+  __syncthreads();
+  const int N = g.ny * g.nz;
+  const int n = 2 * (blockIdx.x * blockDim.x + threadIdx.x);  // nz is even: both points share a row
+  if (n >= N) return;
+  const long long nsc = (long long)g.S * g.C;
+  for (long long sc = blockIdx.y; sc < nsc; sc += gridDim.y) {
+    const TePlace pl(g, trb, sc, n);
+    float4 a[KC];
 #pragma unroll
-  for (int k = 0; k < KC; ++k)
-    if (k < g.K) ob[(long long)k * N] = acc[k];
+    for (int k = 0; k < KC; ++k)
+      a[k] = k < g.K ? *reinterpret_cast<const float4*>(v + pl.at(k)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    float4* yb = reinterpret_cast<float4*>(y + sc * g.T * (long long)N + n);
+    const long long step = N / 2;
+    for (int t0 = 0; t0 < g.T; t0 += 32) {
+      uint2 b = *reinterpret_cast<const uint2*>(bits + (long long)(t0 >> 5) * N + n);
+      const int m = min(32, g.T - t0);
+#pragma unroll 4
+      for (int i = 0; i < m; ++i) {
+        float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float* ph = sphi + (t0 + i) * g.K;
+        if ((b.x >> i) & 1u) {
+#pragma unroll
+          for (int k = 0; k < KC; ++k)
+            if (k < g.K) {
+              o.x = fmaf(ph[k], a[k].x, o.x);
+              o.y = fmaf(ph[k], a[k].y, o.y);
+            }
+        }
+        if ((b.y >> i) & 1u) {
+#pragma unroll
+          for (int k = 0; k < KC; ++k)
+            if (k < g.K) {
+              o.z = fmaf(ph[k], a[k].z, o.z);
+              o.w = fmaf(ph[k], a[k].w, o.w);
+            }
+        }
+        __stcs(yb, o);
+        yb += step;
+      }
+    }
+  }
 }
 
 cudaError_t launch_maps_prep(const Geom& g, const float2* maps_in, float2* maps_out, unsigned* lam_bits,
@@ -144,23 +327,52 @@ cudaError_t launch_maps_prep(const Geom& g, const float2* maps_in, float2* maps_
   return cudaGetLastError();
 }
 
-cudaError_t launch_psi_build(const Geom& g, const float* phi, const uint8_t* mask, float* psi,
+cudaError_t launch_psi_build(const Geom& g, const float* phi, const uint8_t* mask, float* psi, unsigned* bits,
                              unsigned* lam_bits, cudaStream_t st) {
   const int N = g.ny * g.nz;
-  const unsigned grid = (unsigned)((N + kThreads - 1) / kThreads);
+  const unsigned grid = (unsigned)((N + kPsiThreads - 1) / kPsiThreads);
   const size_t sm = sizeof(float) * g.T * g.K;
-  if (g.K <= 4) k_psi_build<4><<<grid, kThreads, sm, st>>>(g, phi, mask, psi, lam_bits);
-  else k_psi_build<8><<<grid, kThreads, sm, st>>>(g, phi, mask, psi, lam_bits);
+  if (g.K <= 4) k_psi_build<4><<<grid, kPsiThreads, sm, st>>>(g, phi, mask, psi, bits, lam_bits);
+  else k_psi_build<8><<<grid, kPsiThreads, sm, st>>>(g, phi, mask, psi, bits, lam_bits);
   return cudaGetLastError();
 }
 
-cudaError_t launch_project(const Geom& g, const float* phi, const uint8_t* mask, const float2* y_te,
-                           float2* y_proj, cudaStream_t st) {
+template <int KC, int NP, int NS>
+static cudaError_t project_go(const Geom& g, int trb, const float* phi, const unsigned* bits, const float2* y,
+                              float2* out, cudaStream_t st) {
   const int N = g.ny * g.nz;
-  dim3 grid((N + kThreads - 1) / kThreads, g.S * g.C);
+  const long long planes = ((long long)g.S * g.C + NP - 1) / NP;
+  dim3 grid((N + kThreads - 1) / kThreads, (unsigned)(planes < 65535 ? planes : 65535));
+  k_project<KC, NP, NS><<<grid, kThreads, sizeof(float) * g.T * g.K, st>>>(g, trb, phi, bits, y, out);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_project(const Geom& g, bool il, const float* phi, const unsigned* bits, const float2* y_te,
+                           float2* y_proj, cudaStream_t st) {
+  const int trb = il ? il_rb(g.ny) : 0;
+  int nsm = 0;
+  const cudaError_t e = sm_count(&nsm);
+  if (e != cudaSuccess) return e;
+  // four planes per thread read the bit words once for four; where that leaves SMs without a few
+  // CTAs each, the k-space centre (every echo sampled) is the critical path: one plane per thread
+  // and eight samples at a time
+  const long long ctas = (long long)((g.ny * g.nz + kThreads - 1) / kThreads) * (((long long)g.S * g.C + 3) / 4);
+  if (ctas >= 6LL * nsm)
+    return g.K <= 4 ? project_go<4, 4, 2>(g, trb, phi, bits, y_te, y_proj, st)
+                    : project_go<8, 4, 2>(g, trb, phi, bits, y_te, y_proj, st);
+  return g.K <= 4 ? project_go<4, 1, 8>(g, trb, phi, bits, y_te, y_proj, st)
+                  : project_go<8, 1, 8>(g, trb, phi, bits, y_te, y_proj, st);
+}
+
+cudaError_t launch_expand_te(const Geom& g, bool il, const float* phi, const unsigned* bits, const float2* v,
+                             float2* y_te, cudaStream_t st) {
+  const int N2 = g.ny * g.nz / 2;
+  const long long nsc = (long long)g.S * g.C;
+  dim3 grid((N2 + kThreads - 1) / kThreads, (unsigned)(nsc < 65535 ? nsc : 65535));
   const size_t sm = sizeof(float) * g.T * g.K;
-  if (g.K <= 4) k_project<4><<<grid, kThreads, sm, st>>>(g, phi, mask, y_te, y_proj);
-  else k_project<8><<<grid, kThreads, sm, st>>>(g, phi, mask, y_te, y_proj);
+  const int trb = il ? il_rb(g.ny) : 0;
+  if (g.K <= 4) k_expand_te<4><<<grid, kThreads, sm, st>>>(g, trb, phi, bits, v, y_te);
+  else k_expand_te<8><<<grid, kThreads, sm, st>>>(g, trb, phi, bits, v, y_te);
   return cudaGetLastError();
 }
 

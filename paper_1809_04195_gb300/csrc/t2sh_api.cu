@@ -242,7 +242,7 @@ struct t2sh_plan_s {
   float2* tw_y = nullptr;
   float2* tw_z = nullptr;
   float* phi = nullptr;
-  uint8_t* mask = nullptr;
+  unsigned* bits = nullptr;  // sampling pattern as bit words [ceil(T / 32)][ny][nz]
   float* psi = nullptr;
   float2* maps = nullptr;
   float2* x = nullptr;
@@ -368,7 +368,7 @@ t2sh_status normal_op(t2sh_plan_t p, const float2* x, float2* y) {
   {
     KTimer k(p, KC_COL);
     T2SH_CK(il ? launch_col_il(p->g, IL_NORMAL, p->tw_y, p->psi, nullptr, p->t, p->st)
-               : launch_col(p->g, COL_NORMAL, p->py, p->tw_y, p->psi, p->phi, p->mask, p->t, p->t, p->st));
+               : launch_col(p->g, COL_NORMAL, p->py, p->tw_y, p->psi, p->t, p->t, p->st));
   }
   { KTimer k(p, KC_ROW_ADJ); T2SH_CK(launch_row(p->g, ROW_ADJ, il, p->pz, p->tw_z, p->maps, nullptr, p->t, y, p->st)); }
   return T2SH_OK;
@@ -377,18 +377,19 @@ t2sh_status normal_op(t2sh_plan_t p, const float2* x, float2* y) {
 // A^H y for device k-space in either form, result in x.
 t2sh_status adjoint_data(t2sh_plan_t p, const void* y, int32_t kform, float2* x) {
   const float2* proj = static_cast<const float2*>(y);
-  // per-echo data are projected into t (planar), which an interleaved column pass could not
-  // read and write at once
-  const bool il = t_interleaved(p->g) && kform == T2SH_KSPACE_PROJ;
+  const bool il = t_interleaved(p->g);
+  // per-echo data are projected into t itself, in the layout the column pass takes in place
+  IlPass pass = IL_ADJ_PLANAR;
   if (kform == T2SH_KSPACE_TE) {
     KTimer k(p, KC_PROJ);
-    T2SH_CK(launch_project(p->g, p->phi, p->mask, static_cast<const float2*>(y), p->t, p->st));
+    T2SH_CK(launch_project(p->g, il, p->phi, p->bits, static_cast<const float2*>(y), p->t, p->st));
     proj = p->t;
+    pass = IL_ADJ;
   }
   {
     KTimer k(p, KC_COL);
-    T2SH_CK(il ? launch_col_il(p->g, IL_ADJ_PLANAR, p->tw_y, nullptr, proj, p->t, p->st)
-               : launch_col(p->g, COL_ADJ_DATA, p->py, p->tw_y, p->psi, p->phi, p->mask, proj, p->t, p->st));
+    T2SH_CK(il ? launch_col_il(p->g, pass, p->tw_y, nullptr, proj, p->t, p->st)
+               : launch_col(p->g, COL_ADJ_DATA, p->py, p->tw_y, p->psi, proj, p->t, p->st));
   }
   { KTimer k(p, KC_ROW_ADJ); T2SH_CK(launch_row(p->g, ROW_ADJ, il, p->pz, p->tw_z, p->maps, nullptr, p->t, x, p->st)); }
   return T2SH_OK;
@@ -465,7 +466,8 @@ t2sh_status t2sh_plan(const t2sh_dims* dims, const float* phi, const uint8_t* ma
   ALLOC(p->maps, f.maps);
   ALLOC(p->psi, f.psi);
   ALLOC(p->phi, f.phi);
-  ALLOC(p->mask, f.mask);
+  const size_t word_bytes = (size_t)((d.nechoes + 31) / 32) * 4 * d.ny * d.nz;
+  ALLOC(p->bits, word_bytes);
   ALLOC(p->x, f.vec);
   ALLOC(p->z, f.vec);
   ALLOC(p->aty, f.vec);
@@ -501,15 +503,29 @@ t2sh_status t2sh_plan(const t2sh_dims* dims, const float* phi, const uint8_t* ma
   FAIL_CK(cudaMemcpyAsync(p->tw_z, tw.data(), cbytes(d.nz), cudaMemcpyHostToDevice, p->st));
   const cudaMemcpyKind kind = p->host_io ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
   FAIL_CK(cudaMemcpyAsync(p->phi, phi, f.phi, kind, p->st));
-  FAIL_CK(cudaMemcpyAsync(p->mask, mask, f.mask, kind, p->st));
   const float2* maps_src = static_cast<const float2*>(maps);
   if (p->host_io) {
     FAIL_CK(cudaMemcpyAsync(p->maps, maps, f.maps, kind, p->st));
     maps_src = p->maps;
   }
+  const uint8_t* mask_src = mask;
+  if (p->host_io) {  // staged in t, which nothing has used yet (t holds at least 8 C K bytes a point)
+    uint8_t* stage = nullptr;
+    if (f.mask <= f.t) {
+      stage = reinterpret_cast<uint8_t*>(p->t);
+    } else {
+      const t2sh_status a_ = p->alloc(&stage, f.mask);
+      if (a_ != T2SH_OK) {
+        delete p;
+        return a_;
+      }
+    }
+    FAIL_CK(cudaMemcpyAsync(stage, mask, f.mask, kind, p->st));
+    mask_src = stage;
+  }
   FAIL_CK(cudaMemsetAsync(p->red, 0, 64, p->st));
   FAIL_CK(launch_maps_prep(g, maps_src, p->maps, p->red, p->st));
-  FAIL_CK(launch_psi_build(g, p->phi, p->mask, p->psi, p->red + 1, p->st));
+  FAIL_CK(launch_psi_build(g, p->phi, mask_src, p->psi, p->bits, p->red + 1, p->st));
   unsigned bits[2];
   FAIL_CK(cudaMemcpyAsync(bits, p->red, sizeof(bits), cudaMemcpyDeviceToHost, p->st));
   FAIL_CK(cudaStreamSynchronize(p->st));
@@ -609,9 +625,20 @@ t2sh_status t2sh_get_step(t2sh_plan_t p, float* step) {
 t2sh_status t2sh_forward(t2sh_plan_t p, const void* x, void* y, int32_t kform) {
   T2SH_REQ(p && x && y, "NULL argument");
   T2SH_REQ(kform == T2SH_KSPACE_TE || kform == T2SH_KSPACE_PROJ, "bad kform %d", kform);
-  { KTimer k(p, KC_ROW_FWD); T2SH_CK(launch_row(p->g, ROW_FWD, false, p->pz, p->tw_z, p->maps, static_cast<const float2*>(x), p->t, nullptr, p->st)); }
-  { KTimer k(p, KC_COL); T2SH_CK(launch_col(p->g, kform == T2SH_KSPACE_TE ? COL_FWD_TE : COL_FWD_PROJ, p->py, p->tw_y, p->psi, p->phi,
-                     p->mask, p->t, static_cast<float2*>(y), p->st)); }
+  const bool il = t_interleaved(p->g), te = kform == T2SH_KSPACE_TE;
+  float2* yo = static_cast<float2*>(y);
+  { KTimer k(p, KC_ROW_FWD); T2SH_CK(launch_row(p->g, ROW_FWD, il, p->pz, p->tw_z, p->maps, static_cast<const float2*>(x), p->t, nullptr, p->st)); }
+  {
+    KTimer k(p, KC_COL);
+    if (il)
+      T2SH_CK(launch_col_il(p->g, te ? IL_FWD_RAW : IL_FWD_PROJ, p->tw_y, p->psi, p->t, te ? p->t : yo, p->st));
+    else
+      T2SH_CK(launch_col(p->g, te ? COL_FWD_RAW : COL_FWD_PROJ, p->py, p->tw_y, p->psi, p->t, te ? p->t : yo, p->st));
+  }
+  if (te) {
+    KTimer k(p, KC_PROJ);
+    T2SH_CK(launch_expand_te(p->g, il, p->phi, p->bits, p->t, yo, p->st));
+  }
   return T2SH_OK;
 }
 
@@ -717,7 +744,7 @@ t2sh_status iteration(t2sh_plan_t p) {
     // LLR, momentum and DFT_z(S z_{k+1}) for the next iteration (z_0 = 0: no A^H A z_0)
     if (it > 0) {
       KTimer k(p, KC_COL);
-      T2SH_CK(launch_col(p->g, COL_NORMAL, p->py, p->tw_y, p->psi, p->phi, p->mask, p->t, p->t, p->st));
+      T2SH_CK(launch_col(p->g, COL_NORMAL, p->py, p->tw_y, p->psi, p->t, p->t, p->st));
     }
     KTimer k(p, KC_BAND);
     T2SH_CK(launch_band_fused(p->g, a, p->tw_z, p->maps, p->t, p->x, p->z, p->aty, p->st));
@@ -1240,7 +1267,7 @@ t2sh_status t2sh_objective(t2sh_plan_t p, const void* kspace, int32_t kform, con
   if (s != T2SH_OK) return s;
   T2SH_CK(launch_cg_dot(p->g, xd, p->grad, 0.f, xa, p->st));
   if (kform == T2SH_KSPACE_TE)
-    T2SH_CK(launch_masked_energy(p->g, p->mask, static_cast<const float2*>(ky), yy, p->st));
+    T2SH_CK(launch_masked_energy(p->g, p->bits, static_cast<const float2*>(ky), yy, p->st));
   std::vector<double> h(3 * (size_t)S);
   T2SH_CK(cudaMemcpyAsync(h.data(), p->obj, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, p->st));
   T2SH_CK(cudaStreamSynchronize(p->st));

@@ -53,7 +53,7 @@ enum ColMode : int {
   COL_NORMAL = 0,    // DFT_y, Psi (pre-scaled by 1/N), IDFT_y                 (normal operator)
   COL_ADJ_DATA = 1,  // multiply by gsign (-1)^(ky+kz) / sqrt(N), IDFT_y          (A^H y)
   COL_FWD_PROJ = 2,  // DFT_y, multiply by gsign (-1)^(ky+kz) / sqrt(N), Psi * N  (Phi^T P A x)
-  COL_FWD_TE = 3     // DFT_y, multiply by gsign (-1)^(ky+kz) / sqrt(N), P_t Phi  (A x, per echo)
+  COL_FWD_RAW = 3    // DFT_y, multiply by gsign (-1)^(ky+kz) / sqrt(N), in place  (A x before P_t Phi)
 };
 
 // Row-pass (kz direction) modes.
@@ -66,7 +66,9 @@ enum RowMode : int {
 enum IlPass : int {
   IL_NORMAL = 0,      // DFT_y, Psi, IDFT_y in place on t
   IL_ADJ_PLANAR = 1,  // A^H y column pass from planar projected k-space [S][C][K][ny][nz]
-  IL_ADJ = 2          // the same from k-space in t's own layout (may be t itself)
+  IL_ADJ = 2,         // the same from k-space in t's own layout (may be t itself)
+  IL_FWD_PROJ = 3,    // DFT_y of t, centring and scale, Psi N, to planar k-space [S][C][K][ny][nz]
+  IL_FWD_RAW = 4      // DFT_y of t, centring and scale, in place
 };
 
 struct FistaArgs {
@@ -85,16 +87,21 @@ struct FistaArgs {
 // All return the cudaGetLastError() of their launch.
 cudaError_t launch_maps_prep(const Geom& g, const float2* maps_in, float2* maps_out, unsigned* lam_s_bits,
                              cudaStream_t st);
-cudaError_t launch_psi_build(const Geom& g, const float* phi, const uint8_t* mask, float* psi,
-                             unsigned* lam_psi_bits, cudaStream_t st);
-cudaError_t launch_project(const Geom& g, const float* phi, const uint8_t* mask, const float2* y_te,
+// bits (nullable): the sampling pattern as bit words [ceil(T / 32)][ny][nz], bit i of word w for
+// echo 32 w + i; lam_bits: zero on entry
+cudaError_t launch_psi_build(const Geom& g, const float* phi, const uint8_t* mask, float* psi, unsigned* bits,
+                             unsigned* lam_bits, cudaStream_t st);
+// per-echo k-space and its projection / synthesis; il: the projected side has t's interleaved layout
+cudaError_t launch_project(const Geom& g, bool il, const float* phi, const unsigned* bits, const float2* y_te,
                            float2* y_proj, cudaStream_t st);
+cudaError_t launch_expand_te(const Geom& g, bool il, const float* phi, const unsigned* bits, const float2* v,
+                             float2* y_te, cudaStream_t st);
 // il: t has the interleaved layout of k_col_il.cu (only where t_interleaved(g))
 bool t_interleaved(const Geom& g);
 cudaError_t launch_row(const Geom& g, RowMode mode, bool il, const FftPlan& pz, const float2* tw_z, const float2* maps,
                        const float2* x, float2* t, float2* out, cudaStream_t st);
 cudaError_t launch_col(const Geom& g, ColMode mode, const FftPlan& py, const float2* tw_y, const float* psi,
-                       const float* phi, const uint8_t* mask, const float2* tin, float2* tout, cudaStream_t st);
+                       const float2* tin, float2* tout, cudaStream_t st);
 // TE images: back-projection at echoes te[0..nte), coil images, homodyne along z with
 // band half-width w, root sum of squares -> out [S][nte][ny][nz] float
 size_t post_smem_bytes(const Geom& g, int nte);
@@ -120,7 +127,7 @@ cudaError_t launch_cg_init(const Geom& g, const float2* x, const float2* w, cons
                            const float2* u, float rho, float2* r, float2* p, double* rr, cudaStream_t st);
 cudaError_t launch_cg_dot(const Geom& g, const float2* p, const float2* w, float rho, double* pq, cudaStream_t st);
 // out[s] += sum of P_t(n) |y|^2 over T-form k-space y [S][C][T][ny][nz]
-cudaError_t launch_masked_energy(const Geom& g, const uint8_t* mask, const float2* y, double* out, cudaStream_t st);
+cudaError_t launch_masked_energy(const Geom& g, const unsigned* bits, const float2* y, double* out, cudaStream_t st);
 cudaError_t launch_cg_step(const Geom& g, float2* x, float2* r, const float2* p, const float2* w, float rho,
                            const double* rr, const double* pq, double* rr_new, cudaStream_t st);
 cudaError_t launch_cg_dir(const Geom& g, const float2* r, float2* p, const double* rr, const double* rr_new,

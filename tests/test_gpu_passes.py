@@ -38,3 +38,30 @@ def test_passes_of_four_images(T, S, ny, nz, C, M):  # noqa: F811
     for s in {0, S // 2, S - 1}:
         assert nrmse(got_n[s], O.normal(xs[s], maps[s], psi)) < OP_TOL
         assert nrmse(got_a[s], O.adjoint_projected(ys[s], maps[s])) < OP_TOL
+
+
+@pytest.mark.parametrize("S,ny,nz,C,Tn,K,M", [
+    (2, 64, 64, 3, 32, 4, 1),     # exactly one word of echoes
+    (1, 256, 48, 5, 33, 4, 2),    # one echo in the second word; planes not a multiple of four
+    (3, 260, 160, 3, 70, 4, 1),
+    (1, 192, 240, 2, 4, 4, 1),    # as few echoes as images
+    (2, 60, 36, 3, 40, 3, 1),     # planar intermediate, K < 4
+    (1, 30, 50, 2, 65, 6, 2),     # K > 4
+])
+def test_per_echo_and_projected_forms(T, S, ny, nz, C, Tn, K, M):  # noqa: F811
+    rng, phi, mask, maps = random_problem(ny + nz + Tn, S, ny, nz, C, Tn, K, M)
+    mask[:, ny // 2, nz // 2] = 1   # a point with every echo
+    mask[:, 0, :2] = 0              # points with none
+    x, y = crandn(rng, S, M, K, ny, nz), crandn(rng, S, C, Tn, ny, nz)
+    with make_plan(T, phi, mask, maps) as p:
+        te, pr = host(p.forward(c64(x), T.KSPACE_TE)), host(p.forward(c64(x), T.KSPACE_PROJ))
+        ad, mu = host(p.adjoint(c64(y), T.KSPACE_TE)), p.step
+    xs, ys = (a.astype(np.complex64).astype(np.complex128) for a in (x, y))
+    psi = O.space_time_kernel(mask, phi)
+    L = max(O.lipschitz(maps[s], psi) for s in range(S))
+    assert abs(mu - 1.0 / L) <= 1e-5 / L
+    for s in {0, S - 1}:
+        ref = O.forward(xs[s], maps[s], mask, phi)
+        assert nrmse(te[s], ref) < OP_TOL and np.all(te[s][:, mask == 0] == 0)
+        assert nrmse(pr[s], O.project(ref, mask, phi)) < OP_TOL
+        assert nrmse(ad[s], O.adjoint(ys[s], maps[s], mask, phi)) < OP_TOL
