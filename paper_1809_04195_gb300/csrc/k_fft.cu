@@ -364,17 +364,38 @@ static cudaError_t row_go(const Geom& g, const FftPlan& pz, const float2* tw, co
                         : row_go13<MODE, KC, MC, false>(g, pz, tw, maps, x, t, out, st);
 }
 
-// Whether the passes of this shape keep t interleaved (k_col_il.cu): the size-specialised
-// passes of four basis images in their default column variant.
-bool t_interleaved(const Geom& g) {
-  const long long rows = (long long)g.S * g.C * std::max(g.ny, g.nz);
-  return g.K == 4 && g.colvar == 0 && g.nz % 4 == 0 && il_rb(g.ny) > 0 && row_il_supported(g) &&
-         rows + g.S * (long long)g.C <= 0x7fffffffLL && tma_encode_fn() != nullptr;
+// Chunked layouts serve the default column variant: the size-specialised passes of four basis
+// images where both lengths have them, the passes of k_any.cu for what they cover otherwise (the
+// two share a layout at K = 4, so one side may be specialised).  Planar: the other column
+// variants and lengths that need three radix stages.
+TLayout t_layout(const Geom& g) {
+  TLayout lt{};
+  if (g.colvar != 0) return lt;
+  const long long nsc = (long long)g.S * g.C;
+  const bool four = g.K == 4 && g.nz % 4 == 0;
+  // fewer images on lengths that the planar size-specialised passes have: those are 1.1 to 1.7
+  // times faster than the two-radix ones (256x160, C = 12, 16 slices, K = 3: 244 against 403 us)
+  if (g.K < 4 && g.nz % 8 == 0 && il_rb(g.ny) > 0 && row_fast_supported(g)) return lt;
+  lt.col_il = four && il_rb(g.ny) > 0 && nsc * (std::max(g.ny, g.nz) + 1) <= 0x7fffffffLL && tma_encode_fn() != nullptr;
+  lt.row_il = four && row_il_supported(g);
+  if ((lt.col_il || any_col_supported(g)) && (lt.row_il || any_row_supported(g))) {
+    lt.W = g.nz % 4 ? 2 : 4;
+    lt.trb = lt.col_il ? il_rb(g.ny) : 0;
+  }
+  return lt;
 }
 
-cudaError_t launch_row(const Geom& g, RowMode mode, bool il, const FftPlan& pz, const float2* tw_z, const float2* maps,
-                       const float2* x, float2* t, float2* out, cudaStream_t st) {
-  if (il) return launch_row_il(g, mode, il_rb(g.ny), tw_z, maps, x, t, out, st);
+cudaError_t launch_col_t(const Geom& g, const TLayout& lt, IlPass pass, const float2* tw_y, const float* psi,
+                         const float2* in, float2* out, cudaStream_t st) {
+  return lt.col_il ? launch_col_il(g, pass, tw_y, psi, in, out, st)
+                   : launch_col_any(g, lt.W, pass, tw_y, psi, in, out, st);
+}
+
+cudaError_t launch_row(const Geom& g, RowMode mode, const TLayout& lt, const FftPlan& pz, const float2* tw_z,
+                       const float2* maps, const float2* x, float2* t, float2* out, cudaStream_t st) {
+  if (lt.W)
+    return lt.row_il ? launch_row_il(g, mode, lt.trb, tw_z, maps, x, t, out, st)
+                     : launch_row_any(g, mode, lt.W, lt.trb, tw_z, maps, x, t, out, st);
   const cudaError_t ef = launch_row_fast(g, mode, tw_z, maps, x, t, out, st);
   if (ef != cudaErrorNotSupported) return ef;
   const bool k4 = g.K <= 4, m1 = g.M == 1;

@@ -422,6 +422,12 @@ static cudaError_t row_fast_n(const Geom& g, RowMode mode, const float2* tw, con
                   : row_fast_go<N, ROW_ADJ, 2>(g, tw, maps, x, t, out, st);
 }
 
+bool row_fast_supported(const Geom& g) {
+  for (int n : {48, 64, 96, 128, 160, 192, 240, 256})
+    if (g.nz == n) return g.K <= 4 && g.M <= 2;
+  return false;
+}
+
 cudaError_t launch_row_fast(const Geom& g, RowMode mode, const float2* tw_z, const float2* maps, const float2* x,
                             float2* t, float2* out, cudaStream_t st) {
   if (g.K > 4 || g.M > 2) return cudaErrorNotSupported;

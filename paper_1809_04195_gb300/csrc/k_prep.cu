@@ -164,29 +164,26 @@ __global__ void __launch_bounds__(kPsiThreads) k_psi_build(Geom g, const float* 
   warp_max_bits(lam, lam_bits);
 }
 
-// Place of (image k, point n = y nz + z) of per-coil data: planar [K][ny][nz], or t's interleaved
-// layout (k_col_il.cu) where trb > 0
+// Place of (image k, point n = y nz + z) of per-coil data in a layout of t
 struct TePlace {
   long long base;
-  int step;  // image stride (planar)
-  int rot;   // slot of image 0 (interleaved)
-  bool il;
-  __device__ __forceinline__ TePlace(const Geom& g, int trb, long long sc, int n) {
-    il = trb > 0;
+  int step;  // image stride
+  int rot;   // slot of image 0 (with slot rotation, K = 4), or -1
+  __device__ __forceinline__ TePlace(const Geom& g, const TLayout& lt, long long sc, int n) {
     const int N = g.ny * g.nz;
-    if (il) {
+    rot = -1;
+    if (lt.W) {
       const int y = n / g.nz, z = n - y * g.nz;
-      base = (sc * g.ny + y) * (4LL * g.nz) + (z >> 2) * 16 + (z & 3);
-      rot = y % trb + y / trb;
-      step = 0;
+      base = (sc * N + (long long)y * g.nz) * g.K + (z / lt.W) * (g.K * lt.W) + z % lt.W;
+      step = lt.W;
+      if (lt.trb) rot = y % lt.trb + y / lt.trb;
     } else {
       base = sc * g.K * (long long)N + n;
       step = N;
-      rot = 0;
     }
   }
   __device__ __forceinline__ long long at(int k) const {
-    return base + (il ? (long long)(((k + rot) & 3) * 4) : (long long)k * step);
+    return base + (long long)(rot >= 0 ? (k + rot) & 3 : k) * step;
   }
 };
 
@@ -196,14 +193,14 @@ __device__ __forceinline__ float2 ld_sample(const float2* p) {
   return v;
 }
 
-// ytil[s][c][k][n] = sum_t Phi_{tk} P_t(n) y[s][c][t][n], planar or interleaved.  A thread walks
+// ytil[s][c][k][n] = sum_t Phi_{tk} P_t(n) y[s][c][t][n], in any layout of t.  A thread walks
 // the set bits of its point only, NS samples of NP (slice, coil) planes at a time, so eight
 // independent loads are in flight instead of one behind one mask byte.  The samples are
 // scattered 8-byte values (5 % of the plane), so the kernel is bound by what DRAM fetches for them:
 // with the default 128-byte fetches 54 % of the whole array (2.0 GB of 3.8, 342 us), with 64-byte
 // ones 281 us.  240x128, C = 8, T = 80 at 5 %, 24 slices: 785 us before.
 template <int KC, int NP, int NS>
-__global__ void __launch_bounds__(kThreads) k_project(Geom g, int trb, const float* __restrict__ phi,
+__global__ void __launch_bounds__(kThreads) k_project(Geom g, TLayout lt, const float* __restrict__ phi,
                                                     const unsigned* __restrict__ bits,
                                                     const float2* __restrict__ y, float2* __restrict__ out) {
   extern __shared__ float sphi[];
@@ -255,7 +252,7 @@ __global__ void __launch_bounds__(kThreads) k_project(Geom g, int trb, const flo
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
       if (i < np) {
-        const TePlace pl(g, trb, sc0 + i, n);
+        const TePlace pl(g, lt, sc0 + i, n);
 #pragma unroll
         for (int k = 0; k < KC; ++k)
           if (k < g.K) out[pl.at(k)] = acc[i][k];
@@ -264,14 +261,14 @@ __global__ void __launch_bounds__(kThreads) k_project(Geom g, int trb, const flo
   }
 }
 
-// y[s][c][t][n] = P_t(n) sum_k Phi_{tk} v_k(n) for every echo, v (planar or interleaved) the
+// y[s][c][t][n] = P_t(n) sum_k Phi_{tk} v_k(n) for every echo, v (in any layout of t) the
 // transformed and scaled coefficients of the coil.  A pure streaming write (the T echoes are K / T
 // times the input): one thread owns two neighbouring points and writes 16 bytes per echo, whole
 // 512-byte runs per warp, so it is bound by HBM writes.  256x160, C = 12, T = 80, 8 slices
 // (2.5 GB): 400 us, 0.93 of the measured copy bandwidth; 745 us when the column pass wrote the
 // echoes itself in 64-byte runs, 445 us with the column pass now.
 template <int KC>
-__global__ void __launch_bounds__(kThreads) k_expand_te(Geom g, int trb, const float* __restrict__ phi,
+__global__ void __launch_bounds__(kThreads) k_expand_te(Geom g, TLayout lt, const float* __restrict__ phi,
                                                       const unsigned* __restrict__ bits,
                                                       const float2* __restrict__ v, float2* __restrict__ y) {
   extern __shared__ float sphi[];
@@ -282,7 +279,7 @@ __global__ void __launch_bounds__(kThreads) k_expand_te(Geom g, int trb, const f
   if (n >= N) return;
   const long long nsc = (long long)g.S * g.C;
   for (long long sc = blockIdx.y; sc < nsc; sc += gridDim.y) {
-    const TePlace pl(g, trb, sc, n);
+    const TePlace pl(g, lt, sc, n);
     float4 a[KC];
 #pragma unroll
     for (int k = 0; k < KC; ++k)
@@ -338,18 +335,17 @@ cudaError_t launch_psi_build(const Geom& g, const float* phi, const uint8_t* mas
 }
 
 template <int KC, int NP, int NS>
-static cudaError_t project_go(const Geom& g, int trb, const float* phi, const unsigned* bits, const float2* y,
+static cudaError_t project_go(const Geom& g, const TLayout& lt, const float* phi, const unsigned* bits, const float2* y,
                               float2* out, cudaStream_t st) {
   const int N = g.ny * g.nz;
   const long long planes = ((long long)g.S * g.C + NP - 1) / NP;
   dim3 grid((N + kThreads - 1) / kThreads, (unsigned)(planes < 65535 ? planes : 65535));
-  k_project<KC, NP, NS><<<grid, kThreads, sizeof(float) * g.T * g.K, st>>>(g, trb, phi, bits, y, out);
+  k_project<KC, NP, NS><<<grid, kThreads, sizeof(float) * g.T * g.K, st>>>(g, lt, phi, bits, y, out);
   return cudaGetLastError();
 }
 
-cudaError_t launch_project(const Geom& g, bool il, const float* phi, const unsigned* bits, const float2* y_te,
+cudaError_t launch_project(const Geom& g, const TLayout& lt, const float* phi, const unsigned* bits, const float2* y_te,
                            float2* y_proj, cudaStream_t st) {
-  const int trb = il ? il_rb(g.ny) : 0;
   int nsm = 0;
   const cudaError_t e = sm_count(&nsm);
   if (e != cudaSuccess) return e;
@@ -358,21 +354,20 @@ cudaError_t launch_project(const Geom& g, bool il, const float* phi, const unsig
   // and eight samples at a time
   const long long ctas = (long long)((g.ny * g.nz + kThreads - 1) / kThreads) * (((long long)g.S * g.C + 3) / 4);
   if (ctas >= 6LL * nsm)
-    return g.K <= 4 ? project_go<4, 4, 2>(g, trb, phi, bits, y_te, y_proj, st)
-                    : project_go<8, 4, 2>(g, trb, phi, bits, y_te, y_proj, st);
-  return g.K <= 4 ? project_go<4, 1, 8>(g, trb, phi, bits, y_te, y_proj, st)
-                  : project_go<8, 1, 8>(g, trb, phi, bits, y_te, y_proj, st);
+    return g.K <= 4 ? project_go<4, 4, 2>(g, lt, phi, bits, y_te, y_proj, st)
+                    : project_go<8, 4, 2>(g, lt, phi, bits, y_te, y_proj, st);
+  return g.K <= 4 ? project_go<4, 1, 8>(g, lt, phi, bits, y_te, y_proj, st)
+                  : project_go<8, 1, 8>(g, lt, phi, bits, y_te, y_proj, st);
 }
 
-cudaError_t launch_expand_te(const Geom& g, bool il, const float* phi, const unsigned* bits, const float2* v,
+cudaError_t launch_expand_te(const Geom& g, const TLayout& lt, const float* phi, const unsigned* bits, const float2* v,
                              float2* y_te, cudaStream_t st) {
   const int N2 = g.ny * g.nz / 2;
   const long long nsc = (long long)g.S * g.C;
   dim3 grid((N2 + kThreads - 1) / kThreads, (unsigned)(nsc < 65535 ? nsc : 65535));
   const size_t sm = sizeof(float) * g.T * g.K;
-  const int trb = il ? il_rb(g.ny) : 0;
-  if (g.K <= 4) k_expand_te<4><<<grid, kThreads, sm, st>>>(g, trb, phi, bits, v, y_te);
-  else k_expand_te<8><<<grid, kThreads, sm, st>>>(g, trb, phi, bits, v, y_te);
+  if (g.K <= 4) k_expand_te<4><<<grid, kThreads, sm, st>>>(g, lt, phi, bits, v, y_te);
+  else k_expand_te<8><<<grid, kThreads, sm, st>>>(g, lt, phi, bits, v, y_te);
   return cudaGetLastError();
 }
 

@@ -1,0 +1,255 @@
+// Row (kz) passes on the interleaved per-coil intermediate t[s][c][y][z / 4][slot][z % 4] of
+// k_col_il.cuh (four basis images), for the line lengths of T2SH_ROW_LENGTHS: N = RI RT.
+//
+// CTA = (slice, band of RB rows), the coil loop inside (Algorithm 1 puts it
+// outermost): the image rows stay in registers and only t goes to memory.  A line is transformed
+// in two register stages with one shared-memory exchange, RI items of radix RT on the side of t
+// and RT items of radix RI on the image side:
+//   forward  A: item j < RT forms S x at z = j + RT r (r < RI), DFT_RI
+//            B: item j < RI: twiddle, DFT_RT                       -> t at z = j + RI k
+//   adjoint  A: item j < RI: IDFT_RT of t at z = j + RI r
+//            B: item j < RT: twiddle, IDFT_RI, conj(S) and the sum over coils at z = j + RT k
+// The basis image is the fastest thread index in every stage: a half-warp is four columns of all
+// four images, so on the side of t it touches exactly one 128-byte line per access (t is bound by
+// the number of lines a load touches as much as by bytes), the map values of the image side are
+// broadcast, and with the four lines' exchange windows starting four (mod 16) apart no stage has
+// bank conflicts.  The adjoint requests the next coil's t one coil ahead.
+//
+// Bound by HBM (maps and t once each, image rows once).  Knee scan (320 slices of 256x160, C = 12,
+// 6.71 GB per launch): forward 1.11 -> 0.99 ms, adjoint 1.15 -> 1.01 ms against the planar passes,
+// 0.98 of the measured copy bandwidth; Table I (M = 2, 7.19 GB): 1.39 -> 1.04 and 1.48 -> 1.22 ms.
+// Reading t with half-warps of one image (four lines per load instead of one) took 1.43 ms, and
+// storing it as runs of R1 columns (partial sectors) 1.30 ms.
+#pragma once
+
+#include <algorithm>
+
+// packed two-lane complex additions in the butterflies: fewer issue slots
+#define T2SH_PACKED_ADD 1
+#include "t2sh_device.cuh"
+
+namespace t2sh {
+
+namespace {
+
+// length, RI, RT: multiples of four from 48 to 320 that are two radices of at most 20, RI a multiple
+// of four so that a half-warp's columns on the side of t are one aligned chunk
+#define T2SH_ROW_LENGTHS(X)                                                                                        \
+  X(48, 16, 3) X(52, 4, 13) X(60, 12, 5) X(64, 16, 4) X(72, 8, 9) X(80, 16, 5) X(96, 16, 6) X(100, 20, 5) X(104, 8, 13) \
+  X(108, 12, 9) X(120, 12, 10) X(128, 16, 8) X(144, 12, 12) X(156, 12, 13) X(160, 16, 10) X(180, 12, 15)               \
+  X(192, 16, 12) X(200, 20, 10) X(208, 16, 13) X(216, 12, 18) X(240, 16, 15) X(256, 16, 16) X(260, 20, 13)           \
+  X(288, 16, 18) X(300, 20, 15) X(320, 16, 20)
+
+template <int N, int RI_, int RT_, int MODE, int MC>
+struct RowIl {
+  static constexpr int RI = RI_, RT = RT_;
+  static_assert(RI * RT == N && RI % 4 == 0, "N = RI RT");
+  // exchange [RT items][RI] (forward) or [RI items][RT] (adjoint), the inner run padded to odd
+  static constexpr int S = (MODE == ROW_FWD ? RI : RT) | 1;
+  static constexpr int L0 = (MODE == ROW_FWD ? RT : RI) * S;
+  static constexpr int LINE = L0 + ((4 - L0 % 16) + 16) % 16;
+  static constexpr int J = RI > RT ? RI : RT;
+  // One-row bands where the items of the smaller side fill their warps or lines are short, two-row
+  // bands otherwise: adjoint at N = 160 1.02 ms with two rows, 1.09 with one (40
+  // items leave the second warp three quarters empty); forward with two map sets at N = 240
+  // 1.04 ms with one row, 1.09 with two.  MINB holds the registers to 80 (forward), 96 or 128.
+  static constexpr int RB = (MODE == ROW_FWD || N <= 64 || RT == 8 || RT >= 15) ? 1 : 2;
+  static constexpr int THREADS = (4 * J * RB + 31) / 32 * 32;
+  static constexpr int REGS = MC == 2 ? (RI > 16 ? 168 : 128) : MODE == ROW_FWD ? (RI > 16 || RT > 16 ? 96 : 80)
+                                                                               : RT <= 10 && RI <= 16 ? 96 : 128;
+  static constexpr int MINB = 65536 / (REGS * THREADS) > 0 ? 65536 / (REGS * THREADS) : 1;
+  static constexpr size_t smem = sizeof(float2) * ((size_t)N + 4 * RB * LINE + 2 * (size_t)MC * RB * N);
+};
+
+template <int N, int RI, int RT, int MODE, int MC>
+__global__ void __launch_bounds__(RowIl<N, RI, RT, MODE, MC>::THREADS, RowIl<N, RI, RT, MODE, MC>::MINB)
+    k_row_il(Geom g, int trb, const float2* __restrict__ tw_g, const float2* __restrict__ maps,
+             const float2* __restrict__ x, float2* __restrict__ t, float2* __restrict__ out) {
+  using R = RowIl<N, RI, RT, MODE, MC>;
+  constexpr int LINE = R::LINE, S = R::S, RB = R::RB;
+  extern __shared__ float2 smem[];
+  const int NN = g.ny * N;
+  const int s = blockIdx.y, y0 = blockIdx.x * RB;
+  const int rb = min(RB, g.ny - y0);
+  // basis image k, item i of the band: t-side items (jt < RI, row rt), image-side items (ji < RT, row ri)
+  const int k = threadIdx.x & 3, i = threadIdx.x >> 2;
+  const int rt = i / RI, jt = i - rt * RI;
+  const int ri = i / RT, ji = i - ri * RT;
+  constexpr bool ALL_T = 4 * RI * RB == R::THREADS;  // every thread has an item on the side of t
+  const bool in_t = ALL_T || rt < RB, on_t = rt < rb, on_i = ri < rb;
+  float2* tw = smem;
+  float2* ex = tw + N;               // [RB][4][LINE]
+  float2* mst = ex + 4 * RB * LINE;  // map rows x2 [MC][RB][N]
+  for (int e = threadIdx.x; e < N; e += R::THREADS) tw[e] = tw_g[e];
+
+  auto issue = [&](int c, int buf) {
+    constexpr int H = N / 2;  // 16-byte copies per row
+    const float2* mp = maps + (long long)(s * g.C + c) * MC * NN + (long long)y0 * N;
+    float2* md = mst + buf * MC * RB * N;
+    for (int e = threadIdx.x; e < MC * RB * H; e += R::THREADS) {
+      const int line = e / H, col = 2 * (e - line * H);
+      const int m = line / RB, row = line - m * RB;
+      if (row < rb) cp_async16(md + line * N + col, mp + (long long)m * NN + row * N + col);
+    }
+  };
+  issue(0, 0);
+  cp_async_commit();
+
+  // t-side address of coil 0: row, slot and the thread's column within its line of t
+  const int yt = y0 + (in_t ? rt : 0);
+  const int slot = trb ? (k + yt % trb + yt / trb) & 3 : k;
+  float2* tp = t + ((long long)s * g.C * g.ny + yt) * (4 * N) + slot * 4 + (jt >> 2) * 16 + (jt & 3);
+  const long long tcoil = 4LL * NN;
+  const float2* exi = ex + ((ri < RB ? ri : 0) * 4 + k) * LINE;
+  float2* ext = ex + ((in_t ? rt : 0) * 4 + k) * LINE;
+  const long long img = (long long)s * MC * 4 * NN + (long long)k * NN + (long long)(y0 + ri) * N + ji;
+
+  if constexpr (MODE == ROW_FWD) {
+    float2 xr[MC][RI];
+#pragma unroll
+    for (int m = 0; m < MC; ++m)
+#pragma unroll
+      for (int q = 0; q < RI; ++q)
+        xr[m][q] = on_i ? x[img + (long long)m * 4 * NN + RT * q] : make_float2(0.f, 0.f);
+    float2* exw = const_cast<float2*>(exi) + ji * S;
+    for (int c = 0; c < g.C; ++c) {
+      const int buf = c & 1;
+      cp_async_wait<0>();
+      __syncthreads();  // coil c's maps are here, and nobody is in the previous coil any more
+      if (c + 1 < g.C) issue(c + 1, buf ^ 1);
+      cp_async_commit();
+      if (ri < RB) {
+        const float2* mrow = mst + (buf * MC * RB + ri) * N + ji;
+        float2 a[RI];
+#pragma unroll
+        for (int q = 0; q < RI; ++q) {
+          float2 v = make_float2(0.f, 0.f);
+#pragma unroll
+          for (int m = 0; m < MC; ++m) cfma(v, mrow[m * RB * N + RT * q], xr[m][q]);
+          a[q] = v;
+        }
+        dft_r<RI, false>(a);
+#pragma unroll
+        for (int q = 0; q < RI; ++q) exw[q] = a[q];
+      }
+      __syncthreads();
+      if (in_t) {
+        float2 b[RT];
+#pragma unroll
+        for (int q = 0; q < RT; ++q) b[q] = ext[q * S + jt];
+#pragma unroll
+        for (int q = 1; q < RT; ++q) b[q] = twiddle_mul<false>(b[q], tw[q * jt]);
+        dft_r<RT, false>(b);
+        if (on_t) {
+#pragma unroll
+          for (int q = 0; q < RT; ++q) tp[q * (4 * RI)] = b[q];
+        }
+      }
+      tp += tcoil;
+    }
+  } else {
+    float2 acc[MC][RI];
+#pragma unroll
+    for (int m = 0; m < MC; ++m)
+#pragma unroll
+      for (int q = 0; q < RI; ++q) acc[m][q] = make_float2(0.f, 0.f);
+    float2 tn[RT];
+#pragma unroll
+    for (int q = 0; q < RT; ++q) tn[q] = on_t ? tp[q * (4 * RI)] : make_float2(0.f, 0.f);
+    for (int c = 0; c < g.C; ++c) {
+      const int buf = c & 1;
+      cp_async_wait<0>();
+      __syncthreads();  // coil c's maps are here, and nobody is in the previous coil any more
+      if (c + 1 < g.C) issue(c + 1, buf ^ 1);
+      cp_async_commit();
+      float2 a[RT];
+#pragma unroll
+      for (int q = 0; q < RT; ++q) a[q] = tn[q];
+      tp += tcoil;
+      if (c + 1 < g.C) {
+#pragma unroll
+        for (int q = 0; q < RT; ++q) tn[q] = on_t ? tp[q * (4 * RI)] : make_float2(0.f, 0.f);
+      }
+      if (in_t) {
+        dft_r<RT, true>(a);
+#pragma unroll
+        for (int q = 0; q < RT; ++q) ext[jt * S + q] = a[q];
+      }
+      __syncthreads();
+      if (ri < RB) {
+        float2 b[RI];
+#pragma unroll
+        for (int q = 0; q < RI; ++q) b[q] = exi[q * S + ji];
+#pragma unroll
+        for (int q = 1; q < RI; ++q) b[q] = twiddle_mul<true>(b[q], tw[q * ji]);
+        dft_r<RI, true>(b);
+        const float2* mrow = mst + (buf * MC * RB + ri) * N + ji;
+#pragma unroll
+        for (int m = 0; m < MC; ++m)
+#pragma unroll
+          for (int q = 0; q < RI; ++q) cfmac(acc[m][q], mrow[m * RB * N + RT * q], b[q]);
+      }
+    }
+    if (on_i) {
+#pragma unroll
+      for (int m = 0; m < MC; ++m)
+#pragma unroll
+        for (int q = 0; q < RI; ++q) out[img + (long long)m * 4 * NN + RT * q] = acc[m][q];
+    }
+  }
+  cp_async_wait<0>();
+}
+
+template <int N, int RI, int RT, int MODE, int MC>
+cudaError_t row_il_go(const Geom& g, int trb, const float2* tw, const float2* maps, const float2* x, float2* t,
+                      float2* out, cudaStream_t st) {
+  using R = RowIl<N, RI, RT, MODE, MC>;
+  const cudaError_t e = smem_optin((const void*)k_row_il<N, RI, RT, MODE, MC>, (int)R::smem);
+  if (e != cudaSuccess) return e;
+  dim3 grid((g.ny + R::RB - 1) / R::RB, g.S);
+  k_row_il<N, RI, RT, MODE, MC><<<grid, R::THREADS, R::smem, st>>>(g, trb, tw, maps, x, t, out);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+// compiled once per direction (T2SH_ROW_MODE), so that the unrolled kernels build in parallel
+#define T2SH_ROW_NAME2(m) launch_row_il_##m
+#define T2SH_ROW_NAME(m) T2SH_ROW_NAME2(m)
+cudaError_t T2SH_ROW_NAME(T2SH_ROW_MODE)(const Geom& g, int trb, const float2* tw, const float2* maps, const float2* x,
+                                         float2* t, float2* out, cudaStream_t st) {
+  switch (g.nz) {
+#define X(n, ri, rt)                                                                                     \
+  case n:                                                                                                \
+    return g.M == 1 ? row_il_go<n, ri, rt, T2SH_ROW_MODE, 1>(g, trb, tw, maps, x, t, out, st)            \
+                    : row_il_go<n, ri, rt, T2SH_ROW_MODE, 2>(g, trb, tw, maps, x, t, out, st);
+    T2SH_ROW_LENGTHS(X)
+#undef X
+    default: return cudaErrorNotSupported;
+  }
+}
+
+#if T2SH_ROW_FIRST
+cudaError_t launch_row_il_ROW_ADJ(const Geom& g, int trb, const float2* tw, const float2* maps, const float2* x,
+                                  float2* t, float2* out, cudaStream_t st);
+
+bool row_il_supported(const Geom& g) {
+  if (g.K != 4 || g.M > 2) return false;
+  switch (g.nz) {
+#define X(n, ri, rt) case n:
+    T2SH_ROW_LENGTHS(X)
+#undef X
+    return true;
+    default: return false;
+  }
+}
+
+cudaError_t launch_row_il(const Geom& g, RowMode mode, int trb, const float2* tw_z, const float2* maps,
+                          const float2* x, float2* t, float2* out, cudaStream_t st) {
+  if (!row_il_supported(g)) return cudaErrorNotSupported;
+  return mode == ROW_FWD ? launch_row_il_ROW_FWD(g, trb, tw_z, maps, x, t, out, st)
+                         : launch_row_il_ROW_ADJ(g, trb, tw_z, maps, x, t, out, st);
+}
+#endif
+
+}  // namespace t2sh

@@ -363,35 +363,35 @@ enum { KC_ROW_FWD = 0, KC_ROW_ADJ = 1, KC_COL = 2, KC_LLR = 3, KC_PLAN = 4, KC_P
 namespace {
 
 t2sh_status normal_op(t2sh_plan_t p, const float2* x, float2* y) {
-  const bool il = t_interleaved(p->g);
-  { KTimer k(p, KC_ROW_FWD); T2SH_CK(launch_row(p->g, ROW_FWD, il, p->pz, p->tw_z, p->maps, x, p->t, nullptr, p->st)); }
+  const TLayout lt = t_layout(p->g);
+  { KTimer k(p, KC_ROW_FWD); T2SH_CK(launch_row(p->g, ROW_FWD, lt, p->pz, p->tw_z, p->maps, x, p->t, nullptr, p->st)); }
   {
     KTimer k(p, KC_COL);
-    T2SH_CK(il ? launch_col_il(p->g, IL_NORMAL, p->tw_y, p->psi, nullptr, p->t, p->st)
+    T2SH_CK(lt.W ? launch_col_t(p->g, lt, IL_NORMAL, p->tw_y, p->psi, p->t, p->t, p->st)
                : launch_col(p->g, COL_NORMAL, p->py, p->tw_y, p->psi, p->t, p->t, p->st));
   }
-  { KTimer k(p, KC_ROW_ADJ); T2SH_CK(launch_row(p->g, ROW_ADJ, il, p->pz, p->tw_z, p->maps, nullptr, p->t, y, p->st)); }
+  { KTimer k(p, KC_ROW_ADJ); T2SH_CK(launch_row(p->g, ROW_ADJ, lt, p->pz, p->tw_z, p->maps, nullptr, p->t, y, p->st)); }
   return T2SH_OK;
 }
 
 // A^H y for device k-space in either form, result in x.
 t2sh_status adjoint_data(t2sh_plan_t p, const void* y, int32_t kform, float2* x) {
   const float2* proj = static_cast<const float2*>(y);
-  const bool il = t_interleaved(p->g);
+  const TLayout lt = t_layout(p->g);
   // per-echo data are projected into t itself, in the layout the column pass takes in place
   IlPass pass = IL_ADJ_PLANAR;
   if (kform == T2SH_KSPACE_TE) {
     KTimer k(p, KC_PROJ);
-    T2SH_CK(launch_project(p->g, il, p->phi, p->bits, static_cast<const float2*>(y), p->t, p->st));
+    T2SH_CK(launch_project(p->g, lt, p->phi, p->bits, static_cast<const float2*>(y), p->t, p->st));
     proj = p->t;
     pass = IL_ADJ;
   }
   {
     KTimer k(p, KC_COL);
-    T2SH_CK(il ? launch_col_il(p->g, pass, p->tw_y, nullptr, proj, p->t, p->st)
+    T2SH_CK(lt.W ? launch_col_t(p->g, lt, pass, p->tw_y, nullptr, proj, p->t, p->st)
                : launch_col(p->g, COL_ADJ_DATA, p->py, p->tw_y, p->psi, proj, p->t, p->st));
   }
-  { KTimer k(p, KC_ROW_ADJ); T2SH_CK(launch_row(p->g, ROW_ADJ, il, p->pz, p->tw_z, p->maps, nullptr, p->t, x, p->st)); }
+  { KTimer k(p, KC_ROW_ADJ); T2SH_CK(launch_row(p->g, ROW_ADJ, lt, p->pz, p->tw_z, p->maps, nullptr, p->t, x, p->st)); }
   return T2SH_OK;
 }
 
@@ -625,19 +625,20 @@ t2sh_status t2sh_get_step(t2sh_plan_t p, float* step) {
 t2sh_status t2sh_forward(t2sh_plan_t p, const void* x, void* y, int32_t kform) {
   T2SH_REQ(p && x && y, "NULL argument");
   T2SH_REQ(kform == T2SH_KSPACE_TE || kform == T2SH_KSPACE_PROJ, "bad kform %d", kform);
-  const bool il = t_interleaved(p->g), te = kform == T2SH_KSPACE_TE;
+  const TLayout lt = t_layout(p->g);
+  const bool te = kform == T2SH_KSPACE_TE;
   float2* yo = static_cast<float2*>(y);
-  { KTimer k(p, KC_ROW_FWD); T2SH_CK(launch_row(p->g, ROW_FWD, il, p->pz, p->tw_z, p->maps, static_cast<const float2*>(x), p->t, nullptr, p->st)); }
+  { KTimer k(p, KC_ROW_FWD); T2SH_CK(launch_row(p->g, ROW_FWD, lt, p->pz, p->tw_z, p->maps, static_cast<const float2*>(x), p->t, nullptr, p->st)); }
   {
     KTimer k(p, KC_COL);
-    if (il)
-      T2SH_CK(launch_col_il(p->g, te ? IL_FWD_RAW : IL_FWD_PROJ, p->tw_y, p->psi, p->t, te ? p->t : yo, p->st));
+    if (lt.W)
+      T2SH_CK(launch_col_t(p->g, lt, te ? IL_FWD_RAW : IL_FWD_PROJ, p->tw_y, p->psi, p->t, te ? p->t : yo, p->st));
     else
       T2SH_CK(launch_col(p->g, te ? COL_FWD_RAW : COL_FWD_PROJ, p->py, p->tw_y, p->psi, p->t, te ? p->t : yo, p->st));
   }
   if (te) {
     KTimer k(p, KC_PROJ);
-    T2SH_CK(launch_expand_te(p->g, il, p->phi, p->bits, p->t, yo, p->st));
+    T2SH_CK(launch_expand_te(p->g, lt, p->phi, p->bits, p->t, yo, p->st));
   }
   return T2SH_OK;
 }

@@ -249,6 +249,68 @@ __device__ __forceinline__ void dft_pfa(float2* v) {
   }
 }
 
+// cos and sin of 2 pi m / n by their power series in double, at compile time (0 <= m < n, the
+// angle brought into [-pi, pi] first; 30 terms leave nothing above rounding)
+constexpr double ct_angle(int m, int n) {
+  return 2.0 * 3.14159265358979323846 * (2 * m > n ? (double)(m - n) / n : (double)m / n);
+}
+constexpr double ct_cos(int m, int n) {
+  const double x = ct_angle(m, n);
+  double t = 1.0, s = 1.0;
+  for (int i = 1; i < 30; ++i) {
+    t *= -x * x / ((2.0 * i - 1.0) * (2.0 * i));
+    s += t;
+  }
+  return s;
+}
+constexpr double ct_sin(int m, int n) {
+  const double x = ct_angle(m, n);
+  double t = x, s = x;
+  for (int i = 1; i < 30; ++i) {
+    t *= -x * x / ((2.0 * i) * (2.0 * i + 1.0));
+    s += t;
+  }
+  return s;
+}
+template <int M, int N>
+struct CtTwiddle {  // exp(-2 pi i M / N)
+  static constexpr float c = (float)ct_cos(M, N), s = (float)-ct_sin(M, N);
+};
+
+// A x A Cooley-Tukey DFT (A = 3, 5): DFT_A over n1 of v[A n1 + n2], twiddles w^(n2 k1), DFT_A over
+// n2 -> X[k1 + A k2]
+template <int A, bool INV, int I>
+__device__ __forceinline__ void ct_twiddles(float2 (&a)[A][A]) {
+  if constexpr (I < A * A) {
+    constexpr int n2 = I / A, k1 = I % A;
+    if constexpr (n2 > 0 && k1 > 0) {
+      using W = CtTwiddle<n2 * k1, A * A>;
+      a[n2][k1] = twiddle_mul<INV>(a[n2][k1], make_float2(W::c, W::s));
+    }
+    ct_twiddles<A, INV, I + 1>(a);
+  }
+}
+template <int A, bool INV>
+__device__ __forceinline__ void dft_square(float2* v) {
+  float2 a[A][A];
+#pragma unroll
+  for (int n2 = 0; n2 < A; ++n2) {
+#pragma unroll
+    for (int n1 = 0; n1 < A; ++n1) a[n2][n1] = v[A * n1 + n2];
+    dft_r<A, INV>(a[n2]);
+  }
+  ct_twiddles<A, INV, 0>(a);
+#pragma unroll
+  for (int k1 = 0; k1 < A; ++k1) {
+    float2 b[A];
+#pragma unroll
+    for (int n2 = 0; n2 < A; ++n2) b[n2] = a[n2][k1];
+    dft_r<A, INV>(b);
+#pragma unroll
+    for (int k2 = 0; k2 < A; ++k2) v[k1 + A * k2] = b[k2];
+  }
+}
+
 template <int R, bool INV>
 __device__ __forceinline__ void dft_r(float2* v) {
   if constexpr (R == 1) {
@@ -258,12 +320,15 @@ __device__ __forceinline__ void dft_r(float2* v) {
   else if constexpr (R == 5) dft5<INV>(v);
   else if constexpr (R == 6) dft_pfa<2, 3, INV>(v);
   else if constexpr (R == 8) dft8<INV>(v);
+  else if constexpr (R == 9) dft_square<3, INV>(v);
   else if constexpr (R == 10) dft_pfa<2, 5, INV>(v);
   else if constexpr (R == 12) dft_pfa<4, 3, INV>(v);
   else if constexpr (R == 13) dft13<INV>(v);
   else if constexpr (R == 15) dft_pfa<3, 5, INV>(v);
   else if constexpr (R == 16) dft16<INV>(v);
+  else if constexpr (R == 18) dft_pfa<2, 9, INV>(v);
   else if constexpr (R == 20) dft_pfa<4, 5, INV>(v);
+  else if constexpr (R == 25) dft_square<5, INV>(v);
   else static_assert(R == 2, "unsupported radix");
 }
 

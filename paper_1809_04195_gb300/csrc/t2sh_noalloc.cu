@@ -143,12 +143,12 @@ extern "C" t2sh_status t2sh_normal_op_noalloc(const t2sh_dims* dims, const float
   if (e == cudaSuccess) e = cudaMemsetAsync(red, 0, kHeader - kRedOff, st);
   if (e == cudaSuccess) e = launch_maps_prep(g, static_cast<const float2*>(maps), maps_s, red, st);
   if (e == cudaSuccess) e = launch_psi_build(g, phi, mask, psi, nullptr, red + 1, st);
-  const bool il = t_interleaved(g);
-  if (e == cudaSuccess) e = launch_row(g, ROW_FWD, il, pz, tw_z, maps_s, static_cast<const float2*>(x), t, nullptr, st);
+  const TLayout lt = t_layout(g);
+  if (e == cudaSuccess) e = launch_row(g, ROW_FWD, lt, pz, tw_z, maps_s, static_cast<const float2*>(x), t, nullptr, st);
   if (e == cudaSuccess)
-    e = il ? launch_col_il(g, IL_NORMAL, tw_y, psi, nullptr, t, st)
+    e = lt.W ? launch_col_t(g, lt, IL_NORMAL, tw_y, psi, t, t, st)
            : launch_col(g, COL_NORMAL, py, tw_y, psi, t, t, st);
-  if (e == cudaSuccess) e = launch_row(g, ROW_ADJ, il, pz, tw_z, maps_s, nullptr, t, static_cast<float2*>(y), st);
+  if (e == cudaSuccess) e = launch_row(g, ROW_ADJ, lt, pz, tw_z, maps_s, nullptr, t, static_cast<float2*>(y), st);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return fail(T2SH_ECUDA, cudaGetErrorString(e));

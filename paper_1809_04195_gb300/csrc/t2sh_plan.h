@@ -62,7 +62,7 @@ enum RowMode : int {
   ROW_ADJ = 1   // out[m][k] = sum_c conj(S'_{c,m}) IDFT_z( t[c][k] )
 };
 
-// Column passes on the interleaved intermediate (k_col_il.cu)
+// Column passes on the interleaved intermediate (k_col_il.cuh)
 enum IlPass : int {
   IL_NORMAL = 0,      // DFT_y, Psi, IDFT_y in place on t
   IL_ADJ_PLANAR = 1,  // A^H y column pass from planar projected k-space [S][C][K][ny][nz]
@@ -87,19 +87,27 @@ struct FistaArgs {
 // All return the cudaGetLastError() of their launch.
 cudaError_t launch_maps_prep(const Geom& g, const float2* maps_in, float2* maps_out, unsigned* lam_s_bits,
                              cudaStream_t st);
+// Layout of the per-coil intermediate t and of projected k-space kept in it
+struct TLayout {
+  int W;                // columns per chunk: t[s][c][y][z / W][slot][z % W]; 0: planar [s][c][k][y][z]
+  int trb;              // slot of image k in row y: (k + y % trb + y / trb) % 4 (k_col_il.cuh); 0: k
+  bool col_il, row_il;  // the size-specialised column / row passes serve it, else those of k_any.cu
+};
+TLayout t_layout(const Geom& g);
 // bits (nullable): the sampling pattern as bit words [ceil(T / 32)][ny][nz], bit i of word w for
 // echo 32 w + i; lam_bits: zero on entry
 cudaError_t launch_psi_build(const Geom& g, const float* phi, const uint8_t* mask, float* psi, unsigned* bits,
                              unsigned* lam_bits, cudaStream_t st);
-// per-echo k-space and its projection / synthesis; il: the projected side has t's interleaved layout
-cudaError_t launch_project(const Geom& g, bool il, const float* phi, const unsigned* bits, const float2* y_te,
+// per-echo k-space and its projection / synthesis; the projected side has layout lt
+cudaError_t launch_project(const Geom& g, const TLayout& lt, const float* phi, const unsigned* bits, const float2* y_te,
                            float2* y_proj, cudaStream_t st);
-cudaError_t launch_expand_te(const Geom& g, bool il, const float* phi, const unsigned* bits, const float2* v,
+cudaError_t launch_expand_te(const Geom& g, const TLayout& lt, const float* phi, const unsigned* bits, const float2* v,
                              float2* y_te, cudaStream_t st);
-// il: t has the interleaved layout of k_col_il.cu (only where t_interleaved(g))
-bool t_interleaved(const Geom& g);
-cudaError_t launch_row(const Geom& g, RowMode mode, bool il, const FftPlan& pz, const float2* tw_z, const float2* maps,
-                       const float2* x, float2* t, float2* out, cudaStream_t st);
+cudaError_t launch_row(const Geom& g, RowMode mode, const TLayout& lt, const FftPlan& pz, const float2* tw_z,
+                       const float2* maps, const float2* x, float2* t, float2* out, cudaStream_t st);
+// column pass on a chunked layout (lt.W > 0)
+cudaError_t launch_col_t(const Geom& g, const TLayout& lt, IlPass pass, const float2* tw_y, const float* psi,
+                         const float2* in, float2* out, cudaStream_t st);
 cudaError_t launch_col(const Geom& g, ColMode mode, const FftPlan& py, const float2* tw_y, const float* psi,
                        const float2* tin, float2* tout, cudaStream_t st);
 // TE images: back-projection at echoes te[0..nte), coil images, homodyne along z with
@@ -154,6 +162,7 @@ cudaError_t launch_llr_list(const LlrJob* jobs, int njobs, int units, bool kc8, 
                             cudaStream_t st);
 
 // size-specialised passes (k_fft_fast.cu); cudaErrorNotSupported when the shape has none
+bool row_fast_supported(const Geom& g);
 cudaError_t launch_row_fast(const Geom& g, RowMode mode, const float2* tw_z, const float2* maps, const float2* x,
                             float2* t, float2* out, cudaStream_t st);
 cudaError_t launch_col_normal_fast(const Geom& g, const float2* tw_y, const float* psi, float2* t, cudaStream_t st);
@@ -166,14 +175,21 @@ cudaError_t launch_wait_selftest(int* err, unsigned long long limit_ns, cudaStre
 cudaError_t launch_col_normal_pr(const Geom& g, const float2* tw_y, const float* psi, float2* t, cudaStream_t st);
 cudaError_t launch_col_normal_tc(const Geom& g, const float2* tw_y, const float* psi, float2* t, cudaStream_t st);
 cudaError_t launch_col_normal_tma(const Geom& g, const float2* tw_y, const float* psi, float2* t, cudaStream_t st);
-// the interleaved intermediate (layout: k_col_il.cu); il_rb: 0 where a column length has no such pass
+// the interleaved intermediate (layout: k_col_il.cuh); il_rb: 0 where a column length has no such pass
 int il_rb(int ny);
 bool row_il_supported(const Geom& g);
-// trb: il_rb(ny)
+// trb: TLayout::trb
 cudaError_t launch_row_il(const Geom& g, RowMode mode, int trb, const float2* tw_z, const float2* maps,
                           const float2* x, float2* t, float2* out, cudaStream_t st);
 cudaError_t launch_col_il(const Geom& g, IlPass pass, const float2* tw_y, const float* psi, const float2* in, float2* t,
                           cudaStream_t st);
+// passes of any two-radix length (k_any.cu)
+bool any_col_supported(const Geom& g);
+bool any_row_supported(const Geom& g);
+cudaError_t launch_col_any(const Geom& g, int W, IlPass pass, const float2* tw_y, const float* psi, const float2* in,
+                           float2* out, cudaStream_t st);
+cudaError_t launch_row_any(const Geom& g, RowMode mode, int W, int trb, const float2* tw_z, const float2* maps,
+                           const float2* x, float2* t, float2* out, cudaStream_t st);
 // A^H y column pass on TMA tiles (K <= 4, nz % 8 == 0, ny = 16 R1 <= 256; tin may equal tout)
 cudaError_t launch_col_adj_tma(const Geom& g, const float2* tw_y, const float2* tin, float2* tout, cudaStream_t st);
 

@@ -65,3 +65,62 @@ def test_per_echo_and_projected_forms(T, S, ny, nz, C, Tn, K, M):  # noqa: F811
         assert nrmse(te[s], ref) < OP_TOL and np.all(te[s][:, mask == 0] == 0)
         assert nrmse(pr[s], O.project(ref, mask, phi)) < OP_TOL
         assert nrmse(ad[s], O.adjoint(ys[s], maps[s], mask, phi)) < OP_TOL
+
+
+@pytest.mark.parametrize("S,ny,nz,C,K,M", [
+    # every radix of the two-radix passes, chunks of four and of two columns, one to eight images
+    (2, 50, 54, 3, 4, 1), (1, 52, 60, 4, 3, 2), (2, 72, 78, 3, 4, 2), (1, 80, 90, 3, 6, 1),
+    (3, 100, 104, 2, 2, 1), (1, 108, 120, 5, 4, 1), (1, 130, 144, 2, 5, 2), (2, 150, 156, 2, 4, 1),
+    (1, 162, 180, 3, 4, 2), (1, 200, 208, 2, 1, 1), (1, 216, 234, 2, 4, 1), (1, 250, 270, 2, 4, 1),
+    (2, 288, 160, 2, 4, 2),   # specialised rows, two-radix columns
+    (2, 256, 180, 3, 4, 1),   # specialised columns (rotated slots), two-radix rows
+    (1, 128, 100, 3, 4, 2),
+    (2, 8, 10, 2, 8, 1), (1, 26, 12, 3, 7, 2),
+    (40, 36, 40, 9, 4, 1),    # runs of tiles across column chunks
+    (1, 300, 250, 2, 8, 1),   # eight images of 250-point rows: the three-stage passes
+    (1, 512, 400, 1, 4, 1),
+])
+def test_two_radix_passes(T, S, ny, nz, C, K, M):  # noqa: F811
+    rng, phi, mask, maps = random_problem(ny * nz + K, S, ny, nz, C, 12, K, M)
+    x, y = crandn(rng, S, M, K, ny, nz), crandn(rng, S, C, K, ny, nz)
+    yt = crandn(rng, S, C, 12, ny, nz)
+    with make_plan(T, phi, mask, maps, block=4) as p:
+        got_n, got_a = host(p.normal_op(c64(x))), host(p.adjoint(c64(y), T.KSPACE_PROJ))
+        got_f, got_t = host(p.forward(c64(x), T.KSPACE_PROJ)), host(p.adjoint(c64(yt), T.KSPACE_TE))
+        got_e = host(p.forward(c64(x), T.KSPACE_TE))
+    psi = O.space_time_kernel(mask, phi)
+    xs, ys, ts = (a.astype(np.complex64).astype(np.complex128) for a in (x, y, yt))
+    for s in {0, S // 2, S - 1}:
+        ref = O.forward(xs[s], maps[s], mask, phi)
+        assert nrmse(got_n[s], O.normal(xs[s], maps[s], psi)) < OP_TOL
+        assert nrmse(got_a[s], O.adjoint_projected(ys[s], maps[s])) < OP_TOL
+        assert nrmse(got_f[s], O.project(ref, mask, phi)) < OP_TOL
+        assert nrmse(got_e[s], ref) < OP_TOL
+        assert nrmse(got_t[s], O.adjoint(ts[s], maps[s], mask, phi)) < OP_TOL
+
+
+COLUMN_LENGTHS = [48, 50, 52, 54, 60, 64, 72, 78, 80, 90, 96, 100, 104, 108, 120, 128, 130, 144, 150, 156, 160, 162,
+                  180, 192, 200, 208, 216, 234, 240, 256, 260, 270, 288, 300, 320]
+
+
+@pytest.mark.parametrize("n", COLUMN_LENGTHS)
+def test_every_specialised_length(T, n):  # noqa: F811
+    """Four images on every column length, and on every row length that has specialised rows (the
+    multiples of four), with one and two map sets, in every direction and form."""
+    for ny, nz, M, S, C in [(n, 52, 1, 3, 5), (n, 60, 2, 1, 2)] + ([(54, n, 1, 2, 3), (48, n, 2, 1, 2)] if n % 4 == 0 else []):
+        rng, phi, mask, maps = random_problem(ny * nz + M, S, ny, nz, C, 8, 4, M)
+        x, y = crandn(rng, S, M, 4, ny, nz), crandn(rng, S, C, 4, ny, nz)
+        yt = crandn(rng, S, C, 8, ny, nz)
+        with make_plan(T, phi, mask, maps, block=4) as p:
+            got_n, got_a = host(p.normal_op(c64(x))), host(p.adjoint(c64(y), T.KSPACE_PROJ))
+            got_f, got_t = host(p.forward(c64(x), T.KSPACE_PROJ)), host(p.adjoint(c64(yt), T.KSPACE_TE))
+            got_e = host(p.forward(c64(x), T.KSPACE_TE))
+        psi = O.space_time_kernel(mask, phi)
+        xs, ys, ts = (a.astype(np.complex64).astype(np.complex128) for a in (x, y, yt))
+        for s in {0, S - 1}:
+            ref = O.forward(xs[s], maps[s], mask, phi)
+            assert nrmse(got_n[s], O.normal(xs[s], maps[s], psi)) < OP_TOL
+            assert nrmse(got_a[s], O.adjoint_projected(ys[s], maps[s])) < OP_TOL
+            assert nrmse(got_f[s], O.project(ref, mask, phi)) < OP_TOL
+            assert nrmse(got_e[s], ref) < OP_TOL
+            assert nrmse(got_t[s], O.adjoint(ts[s], maps[s], mask, phi)) < OP_TOL
