@@ -20,12 +20,6 @@ namespace {
 constexpr int kPostThreads = 256;
 constexpr int kPostRB = 4;
 
-struct PostArgs {
-  int te[kMaxPostTe];
-  int nte;
-  int w;  // half-width of the two-sided band
-};
-
 template <int MC, bool R13>
 __global__ void __launch_bounds__(kPostThreads) k_post(Geom g, FftPlan pz, const float2* __restrict__ tw_g,
                                                      const float2* __restrict__ maps, const float* __restrict__ phi,
@@ -125,6 +119,11 @@ cudaError_t launch_post(const Geom& g, const FftPlan& pz, const float2* tw_z, co
   for (int i = 0; i < nte; ++i) pa.te[i] = te[i];
   pa.nte = nte;
   pa.w = w;
+  // lengths with specialised line transforms; the kernel above is for the others
+  for (auto launch : {launch_post_il_a, launch_post_il_b, launch_post_il_c}) {
+    const cudaError_t e = launch(g, tw_z, maps, phi, alpha, pa, out, st);
+    if (e != cudaErrorNotSupported) return e;
+  }
   const size_t sm = post_smem_bytes(g, nte);
   dim3 grid((g.ny + kPostRB - 1) / kPostRB, g.S);
   const bool r13 = plan_has13(pz);

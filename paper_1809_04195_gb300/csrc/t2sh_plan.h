@@ -110,11 +110,23 @@ cudaError_t launch_col_t(const Geom& g, const TLayout& lt, IlPass pass, const fl
                          const float2* in, float2* out, cudaStream_t st);
 cudaError_t launch_col(const Geom& g, ColMode mode, const FftPlan& py, const float2* tw_y, const float* psi,
                        const float2* tin, float2* tout, cudaStream_t st);
+struct PostArgs {
+  int te[kMaxPostTe];
+  int nte;
+  int w;  // half-width of the two-sided band
+};
 // TE images: back-projection at echoes te[0..nte), coil images, homodyne along z with
 // band half-width w, root sum of squares -> out [S][nte][ny][nz] float
 size_t post_smem_bytes(const Geom& g, int nte);
 cudaError_t launch_post(const Geom& g, const FftPlan& pz, const float2* tw_z, const float2* maps, const float* phi,
                         const float2* alpha, const int* te, int nte, int w, float* out, cudaStream_t st);
+// the same on size-specialised line transforms; cudaErrorNotSupported where nz has none
+cudaError_t launch_post_il_a(const Geom& g, const float2* tw, const float2* maps, const float* phi, const float2* alpha,
+                             const PostArgs& pa, float* out, cudaStream_t st);
+cudaError_t launch_post_il_b(const Geom& g, const float2* tw, const float2* maps, const float* phi, const float2* alpha,
+                             const PostArgs& pa, float* out, cudaStream_t st);
+cudaError_t launch_post_il_c(const Geom& g, const float2* tw, const float2* maps, const float* phi, const float2* alpha,
+                             const PostArgs& pa, float* out, cudaStream_t st);
 // pre-processing from sparse readout lines (k_preproc.cu)
 cudaError_t launch_calib(const float2* lines, int ctot, int nx, const int* order, const int* seg_off, const int* wseg,
                          int nwseg, int win, float2* X, cudaStream_t st);

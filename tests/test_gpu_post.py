@@ -67,3 +67,17 @@ def test_postprocess_rejects_bad_arguments(T):
         for te, pf in [([8], 0.65), ([-1], 0.65), ([0], 0.5), ([0], 1.01), (list(range(8)) + [0], 0.7)]:
             with pytest.raises(T.T2shError):
                 p.postprocess(a, te, pf=pf)
+
+
+@pytest.mark.parametrize("nz", [48, 50, 52, 54, 60, 64, 72, 78, 80, 90, 96, 100, 104, 108, 120, 128, 130, 144, 150, 156,
+                                160, 162, 180, 192, 200, 208, 216, 234, 240, 250, 256, 260, 270, 288, 300, 320])
+def test_postprocess_every_specialised_length(T, nz):
+    """Every specialised line length (and 250, which has none), one and two map sets, rows that do
+    not fill a band, several echoes after one another."""
+    for ny, M, te in ((10, 1, [0, 5, 2]), (26, 2, [7])):
+        rng, phi, mask, maps = random_problem(nz + M, 2, ny, nz, 3, 8, 3, M)
+        alpha = crandn(rng, 2, M, 3, ny, nz)
+        with make_plan(T, phi, mask, maps, block=4) as p:
+            got = p.postprocess(c64(alpha), te, pf=0.65).cpu().numpy().astype(np.float64)
+        ref = O.postprocess(alpha.astype(np.complex64).astype(np.complex128)[1], maps[1], phi, te, float(np.float32(0.65)))
+        assert nrmse(got[1], ref) < POST_TOL
