@@ -8,7 +8,8 @@
 // coefficient with low/high pattern (ex, ey, ez) at the cube point (dx, dy, dz) = (ex, ey, ez):
 // the approximation lands on the cube origin, the next level's lattice.  Details are
 // thresholded as they are formed; the coarsest level's inverse runs in the same pass and
-// the finer inverses follow level by level.  The 2-point Haar pair (a + b, a - b) / sqrt(2)
+// the finer inverses follow level by level.  Pyramids of two or three levels run in one
+// pass (k_haar_tile); the passes per level serve one level and the deeper pyramids.  The 2-point Haar pair (a + b, a - b) / sqrt(2)
 // is its own inverse, so the inverse passes apply the same butterflies.  One thread per
 // cube; at level 1 the z pairs are 16-byte loads of consecutive threads (coalesced).
 #include <algorithm>
@@ -109,6 +110,103 @@ __global__ void k_haar(float2* a, int S, int MK, int ny, int nz, int s, float ta
   }
 }
 
+// Two or three levels of the pyramid in one pass over the volume: a CTA owns a tile of 2^L slices x
+// 2^L rows x 32 columns of one coefficient image, whose cubes are independent of all others.
+// Level 1 cubes live in registers (one per thread); the approximations of a level go to shared
+// memory, where the next level's fewer threads take theirs; the inverse walks back the same way.
+// Details never leave their thread.  Every value is read and written once: three levels of the
+// knee volume (0.42 GB) 341 -> 199 us (floor 124) against one pass per level and direction.
+// Warps whose columns lie past nz (nz a multiple of 2^L, not of 32) only take part in barriers.
+template <int L>
+__global__ void __launch_bounds__(16 << (2 * (L - 1))) k_haar_tile(float2* a, int MK, int ny, int nz, float tau) {
+  constexpr int E = 1 << (L - 1);  // cubes of the tile along x and y
+  __shared__ float2 s1[E * E * 16], s2[L > 2 ? 4 * 8 : 1];
+  const int l = threadIdx.x & 15, j = (threadIdx.x >> 4) & (E - 1), i = threadIdx.x >> (4 + L - 1);
+  const long long sx = (long long)MK * ny * nz;
+  const int ntz = (nz + 31) / 32, tz = blockIdx.x % ntz, ty = blockIdx.x / ntz;
+  const int z = tz * 32 + 2 * l, y = (ty * E + j) * 2;
+  float2* base = a + ((long long)blockIdx.z * E + i) * 2 * sx + (long long)blockIdx.y * ny * nz + (long long)y * nz + z;
+  const bool on = z < nz;
+  float2 v[2][2][2];
+#pragma unroll
+  for (int dx = 0; dx < 2; ++dx)
+#pragma unroll
+    for (int dy = 0; dy < 2; ++dy) {
+      const float4 w = on ? *reinterpret_cast<const float4*>(base + dx * sx + dy * nz) : make_float4(0.f, 0.f, 0.f, 0.f);
+      v[dx][dy][0] = make_float2(w.x, w.y);
+      v[dx][dy][1] = make_float2(w.z, w.w);
+    }
+  haar_cube(v);
+#pragma unroll
+  for (int e = 1; e < 8; ++e) {
+    float2& c = v[e >> 2][(e >> 1) & 1][e & 1];
+    c = soft_threshold(c, tau);
+  }
+  {
+    s1[threadIdx.x] = v[0][0][0];  // [i][j][l]
+    __syncthreads();
+    // level 2: cubes (E / 2)^2 x 8; level 3: one x one x 4
+    constexpr int E2 = E / 2;
+    if ((int)threadIdx.x < E2 * E2 * 8) {
+      const int l2 = threadIdx.x & 7, j2 = (threadIdx.x >> 3) & (E2 - 1), i2 = threadIdx.x >> (3 + (L > 2 ? 1 : 0));
+      float2* p = s1 + ((2 * i2) * E + 2 * j2) * 16 + 2 * l2;
+      float2 u[2][2][2];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) u[e >> 2][(e >> 1) & 1][e & 1] = p[(e >> 2) * E * 16 + ((e >> 1) & 1) * 16 + (e & 1)];
+      haar_cube(u);
+#pragma unroll
+      for (int e = 1; e < 8; ++e) {
+        float2& c = u[e >> 2][(e >> 1) & 1][e & 1];
+        c = soft_threshold(c, tau);
+      }
+      if constexpr (L > 2) {
+        s2[threadIdx.x] = u[0][0][0];  // [i2][j2][l2], all in one warp
+        __syncwarp();
+        if (threadIdx.x < 4) {
+          float2* r = s2 + 2 * threadIdx.x;
+          float2 t[2][2][2];
+#pragma unroll
+          for (int e = 0; e < 8; ++e) t[e >> 2][(e >> 1) & 1][e & 1] = r[(e >> 2) * 16 + ((e >> 1) & 1) * 8 + (e & 1)];
+          haar_cube(t);
+#pragma unroll
+          for (int e = 1; e < 8; ++e) {
+            float2& c = t[e >> 2][(e >> 1) & 1][e & 1];
+            c = soft_threshold(c, tau);
+          }
+          haar_cube(t);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) r[(e >> 2) * 16 + ((e >> 1) & 1) * 8 + (e & 1)] = t[e >> 2][(e >> 1) & 1][e & 1];
+        }
+        __syncwarp();
+        u[0][0][0] = s2[threadIdx.x];
+      }
+      haar_cube(u);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) p[(e >> 2) * E * 16 + ((e >> 1) & 1) * 16 + (e & 1)] = u[e >> 2][(e >> 1) & 1][e & 1];
+    }
+    __syncthreads();
+    v[0][0][0] = s1[threadIdx.x];
+  }
+  haar_cube(v);
+  if (on) {
+#pragma unroll
+    for (int dx = 0; dx < 2; ++dx)
+#pragma unroll
+      for (int dy = 0; dy < 2; ++dy)
+        *reinterpret_cast<float4*>(base + dx * sx + dy * nz) =
+            make_float4(v[dx][dy][0].x, v[dx][dy][0].y, v[dx][dy][1].x, v[dx][dy][1].y);
+  }
+}
+
+template <int L>
+cudaError_t haar_tile_go(const Geom& g, float2* a, float tau, cudaStream_t st) {
+  const int f = 1 << L;
+  const long long gx = (long long)((g.nz + 31) / 32) * (g.ny / f);
+  k_haar_tile<L><<<dim3((unsigned)gx, (unsigned)(g.M * g.K), (unsigned)(g.S / f)), 16 << (2 * (L - 1)), 0, st>>>(
+      a, g.M * g.K, g.ny, g.nz, tau);
+  return cudaGetLastError();
+}
+
 template <int MODE>
 cudaError_t haar_go(float2* a, int S, int MK, int ny, int nz, int s, float tau, cudaStream_t st) {
   const long long ncube = (long long)(S / (2 * s)) * MK * (ny / (2 * s)) * (nz / (2 * s));
@@ -125,6 +223,8 @@ cudaError_t haar_go(float2* a, int S, int MK, int ny, int nz, int s, float tau, 
 
 cudaError_t launch_wavelet_denoise(const Geom& g, float2* alpha, float tau, int levels, cudaStream_t st) {
   const int MK = g.M * g.K;
+  if (levels == 2) return haar_tile_go<2>(g, alpha, tau, st);
+  if (levels == 3) return haar_tile_go<3>(g, alpha, tau, st);
   cudaError_t e = cudaSuccess;
   for (int l = 1; l < levels && e == cudaSuccess; ++l)
     e = haar_go<WV_FWD>(alpha, g.S, MK, g.ny, g.nz, 1 << (l - 1), tau, st);

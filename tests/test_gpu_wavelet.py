@@ -127,3 +127,18 @@ def test_wavelet_denoise_rejects_bad_arguments(T):
         with pytest.raises(T.T2shError) as ei:
             p.wavelet_denoise(torch.zeros((6, 1, 2, 16, 24), dtype=torch.complex64, device="cuda"), 0.1, 1)
         assert ei.value.status == T.EUNSUPPORTED
+
+
+@pytest.mark.parametrize("S,M,K,ny,nz,levels", [(8, 2, 3, 24, 40, 3), (16, 1, 1, 8, 104, 3), (4, 1, 2, 12, 52, 2),
+                                                 (12, 2, 1, 8, 32, 2)])
+def test_wavelet_tiles(T, S, M, K, ny, nz, levels):
+    """One-pass pyramids whose column count does not fill the last tile."""
+    rng, phi, mask, maps = random_problem(950 + S + nz, S, ny, nz, 2, 8, K, M)
+    a32 = crandn(rng, S, M, K, ny, nz).astype(np.complex64)
+    tau = 0.7
+    with make_plan(T, phi, mask, maps, block=4) as p:
+        x = c64(a32)
+        p.wavelet_denoise(x, tau, levels)
+        got = host(x)
+    ref = O.wavelet_denoise(a32.astype(np.complex128), float(np.float32(tau)), levels)
+    assert np.linalg.norm(got - ref) <= 1e-6 * np.linalg.norm(ref)
