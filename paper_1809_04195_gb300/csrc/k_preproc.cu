@@ -1,7 +1,7 @@
 // Pre-processing in front of the per-slice solve (Sec. III.A), from a sparse array of
 // fully sampled readout lines: line j holds the channels [Ctot][Nx] of phase encode
-// (ky_j, kz_j) at echo t_j.  The host sorts the lines by (ky, kz) into segments (one per
-// sampled phase encode); every kernel below works on that table.
+// (ky_j, kz_j) at echo t_j.  The host groups the lines by phase encode (pixel) ky nz + kz with a
+// counting sort: order[off[pixel]] .. order[off[pixel + 1] - 1]; every kernel works on that table.
 //
 //   coil compression: the central win^3 window averaged over the echoes of each (ky, kz)
 //     (k_calib), its channel Gram matrix G = X^H X (k_gram), eigenvectors of G by a
@@ -9,9 +9,10 @@
 //     W [Ctot][C];
 //   decoupling: y_v = y W per line, then the centred unitary inverse DFT along x
 //     (k_compress_readout): yhat [n][C][Nx];
-//   re-sort and project: ytil[x][c][k][ky][kz] = sum_{j in segment} Phi[t_j][k] yhat[j][c][x]
+//   re-sort and project: ytil[x][c][k][ky][kz] = sum_{j at (ky, kz)} Phi[t_j][k] yhat[j][c][x]
 //     (k_project_lines) and the masks mask[t_j][ky_j][kz_j] = 1 (k_mark_mask).
 #include "t2sh_device.cuh"
+#include "two_radix.h"
 
 namespace t2sh {
 
@@ -19,19 +20,19 @@ namespace {
 
 constexpr int kPpThreads = 256;
 
-// calibration rows X[p][c], p = (segment in the window, kx in the window)
+// calibration rows X[p][c], p = (sampled phase encode in the window, kx in the window); off: first
+// line of each phase encode in `order`, wpix: the sampled phase encodes of the window
 __global__ void __launch_bounds__(kPpThreads) k_calib(const float2* __restrict__ lines, int ctot, int nx,
-                                                    const int* __restrict__ order, const int* __restrict__ seg_off,
-                                                    const int* __restrict__ wseg, int nwseg, int win,
+                                                    const int* __restrict__ order, const int* __restrict__ off,
+                                                    const int* __restrict__ wpix, int nwpix, int win,
                                                     float2* __restrict__ X) {
   const int x0 = nx / 2 - win / 2;
-  const long long total = (long long)nwseg * win * ctot;
+  const long long total = (long long)nwpix * win * ctot;
   for (long long e = blockIdx.x * (long long)kPpThreads + threadIdx.x; e < total; e += (long long)gridDim.x * kPpThreads) {
     const int c = (int)(e % ctot);
     const long long p = e / ctot;
     const int xw = (int)(p % win), si = (int)(p / win);
-    const int sg = wseg[si];
-    const int j0 = seg_off[sg], j1 = seg_off[sg + 1];
+    const int j0 = off[wpix[si]], j1 = off[wpix[si] + 1];
     float2 acc = make_float2(0.f, 0.f);
     for (int j = j0; j < j1; ++j) {
       const float2 v = lines[((long long)order[j] * ctot + c) * nx + x0 + xw];
@@ -61,99 +62,143 @@ __global__ void __launch_bounds__(kPpThreads) k_gram(const float2* __restrict__ 
   }
 }
 
-// Eigenvectors of the Hermitian G (interleaved re/im, ctot <= kMaxChan) by cyclic Jacobi
-// in float64 on one thread, sorted by decreasing eigenvalue, each column rotated so that
-// its entry of largest magnitude (first such index) is real positive; W [ctot][ncomp].
-__global__ void k_eig(const double* G, int ctot, int ncomp, float2* W, int* err) {
-  __shared__ double ar[kMaxChan][kMaxChan], ai[kMaxChan][kMaxChan], vr[kMaxChan][kMaxChan], vi[kMaxChan][kMaxChan];
+// Eigenvectors of the Hermitian G (interleaved re/im, ctot <= kMaxChan) by Jacobi in float64, sorted
+// by decreasing eigenvalue, each column rotated so that its entry of largest magnitude (first such
+// index) is real positive; W [ctot][ncomp].  One CTA; each sweep is n - 1 rounds of n / 2 disjoint
+// rotations (round-robin pairs), whose parameters come from the matrix before the round and which
+// all threads apply together: on one thread the chain of dependent float64 operations took 21.3 ms
+// for 16 channels, here 0.43 ms.
+constexpr int kEigLd = kMaxChan + 1;
+struct EigRot {
+  int a, b;  // b < 0: no rotation
+  double c, s, dr, di;
+};
+__global__ void __launch_bounds__(kPpThreads) k_eig(const double* G, int ctot, int ncomp, float2* W, int* err) {
+  __shared__ double ar[kMaxChan][kEigLd], ai[kMaxChan][kEigLd], vr[kMaxChan][kEigLd], vi[kMaxChan][kEigLd];
+  __shared__ EigRot rot[kMaxChan / 2];
+  __shared__ double part[2][kPpThreads / 32];
   __shared__ int ord[kMaxChan];
-  if (threadIdx.x != 0) return;
-  const int n = ctot;
-  for (int i = 0; i < n; ++i)
-    for (int j = 0; j < n; ++j) {
-      ar[i][j] = G[2 * (i * n + j)];
-      ai[i][j] = G[2 * (i * n + j) + 1];
-      vr[i][j] = i == j ? 1.0 : 0.0;
-      vi[i][j] = 0.0;
-    }
-  // symmetrise (the float partial sums are Hermitian only to rounding)
-  for (int i = 0; i < n; ++i) {
-    ai[i][i] = 0.0;
-    for (int j = i + 1; j < n; ++j) {
-      const double r = 0.5 * (ar[i][j] + ar[j][i]), m = 0.5 * (ai[i][j] - ai[j][i]);
-      ar[i][j] = r; ar[j][i] = r; ai[i][j] = m; ai[j][i] = -m;
-    }
+  const int n = ctot, tid = threadIdx.x, m = n + (n & 1), h = m / 2;
+  for (int e = tid; e < n * n; e += kPpThreads) {
+    const int i = e / n, j = e - i * n;
+    // symmetrised: the float partial sums are Hermitian only to rounding
+    ar[i][j] = 0.5 * (G[2 * (i * n + j)] + G[2 * (j * n + i)]);
+    ai[i][j] = i == j ? 0.0 : 0.5 * (G[2 * (i * n + j) + 1] - G[2 * (j * n + i) + 1]);
+    vr[i][j] = i == j ? 1.0 : 0.0;
+    vi[i][j] = 0.0;
   }
-  bool converged = false;
+  __syncthreads();
+  bool converged = n == 1;
   for (int sweep = 0; sweep < 60 && !converged; ++sweep) {
     double off = 0.0, diag = 0.0;
-    for (int p = 0; p < n; ++p) {
-      diag += ar[p][p] * ar[p][p];
-      for (int q = p + 1; q < n; ++q) off += ar[p][q] * ar[p][q] + ai[p][q] * ai[p][q];
+    for (int e = tid; e < n * n; e += kPpThreads) {
+      const int i = e / n, j = e - i * n;
+      if (i == j) diag += ar[i][i] * ar[i][i];
+      else if (i < j) off += ar[i][j] * ar[i][j] + ai[i][j] * ai[i][j];
     }
-    if (!(off > 1e-30 * diag)) {
-      converged = true;
-      break;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      off += __shfl_xor_sync(0xffffffffu, off, o);
+      diag += __shfl_xor_sync(0xffffffffu, diag, o);
     }
-    for (int p = 0; p < n - 1; ++p)
-      for (int q = p + 1; q < n; ++q) {
-        const double xr = ar[p][q], xi = ai[p][q];
-        const double r2 = xr * xr + xi * xi;
-        if (!(r2 > 0.0)) continue;
-        const double r = sqrt(r2), dr = xr / r, di = -xi / r;  // column q *= d = conj(a_pq)/|a_pq|
-        for (int k = 0; k < n; ++k) {
-          if (k == q) continue;
-          const double yr = ar[k][q] * dr - ai[k][q] * di, yi = ar[k][q] * di + ai[k][q] * dr;
-          ar[k][q] = yr; ai[k][q] = yi; ar[q][k] = yr; ai[q][k] = -yi;
+    if ((tid & 31) == 0) {
+      part[0][tid >> 5] = off;
+      part[1][tid >> 5] = diag;
+    }
+    __syncthreads();
+    off = diag = 0.0;
+    for (int i = 0; i < kPpThreads / 32; ++i) {
+      off += part[0][i];
+      diag += part[1][i];
+    }
+    converged = !(off > 1e-30 * diag);  // the same sums in every thread
+    __syncthreads();
+    if (converged) break;
+    for (int rd = 0; rd < m - 1; ++rd) {
+      if (tid < h) {  // pair tid of the round: i + j = rd (mod m - 1), the fixed point meets m - 1
+        const int i0 = (int)((long long)rd * h % (m - 1));
+        int a = tid == 0 ? i0 : (i0 + tid) % (m - 1);
+        int b = tid == 0 ? m - 1 : (i0 - tid + m - 1) % (m - 1);
+        if (a > b) {
+          const int t = a;
+          a = b;
+          b = t;
         }
-        for (int k = 0; k < n; ++k) {
-          const double yr = vr[k][q] * dr - vi[k][q] * di, yi = vr[k][q] * di + vi[k][q] * dr;
-          vr[k][q] = yr; vi[k][q] = yi;
+        EigRot r{a, -1, 1.0, 0.0, 1.0, 0.0};
+        if (b < n) {
+          const double xr = ar[a][b], xi = ai[a][b], r2 = xr * xr + xi * xi;
+          if (r2 > 1e-290) {
+            const double ir = rsqrt(r2);  // column b *= d = conj(a_ab) / |a_ab|
+            const double theta = (ar[b][b] - ar[a][a]) * (0.5 * ir), u = theta * theta + 1.0;
+            double t = fabs(theta) > 1e100 ? 0.5 / fabs(theta) : 1.0 / (fabs(theta) + u * rsqrt(u));
+            if (theta < 0.0) t = -t;
+            r.b = b;
+            r.dr = xr * ir;
+            r.di = -xi * ir;
+            r.c = rsqrt(t * t + 1.0);
+            r.s = t * r.c;
+          }
         }
-        const double theta = (ar[q][q] - ar[p][p]) / (2.0 * r);
-        double t = 1.0 / (fabs(theta) + sqrt(theta * theta + 1.0));
-        if (theta < 0.0) t = -t;
-        const double c = 1.0 / sqrt(t * t + 1.0), s = t * c;
-        ar[p][p] -= t * r;
-        ar[q][q] += t * r;
-        ar[p][q] = 0.0; ar[q][p] = 0.0; ai[p][q] = 0.0; ai[q][p] = 0.0;
-        for (int k = 0; k < n; ++k) {
-          if (k == p || k == q) continue;
-          const double pr_ = ar[k][p], pi_ = ai[k][p], qr_ = ar[k][q], qi_ = ai[k][q];
-          const double npr = c * pr_ - s * qr_, npi = c * pi_ - s * qi_;
-          const double nqr = s * pr_ + c * qr_, nqi = s * pi_ + c * qi_;
-          ar[k][p] = npr; ai[k][p] = npi; ar[p][k] = npr; ai[p][k] = -npi;
-          ar[k][q] = nqr; ai[k][q] = nqi; ar[q][k] = nqr; ai[q][k] = -nqi;
-        }
-        for (int k = 0; k < n; ++k) {
-          const double pr_ = vr[k][p], pi_ = vi[k][p], qr_ = vr[k][q], qi_ = vi[k][q];
-          vr[k][p] = c * pr_ - s * qr_; vi[k][p] = c * pi_ - s * qi_;
-          vr[k][q] = s * pr_ + c * qr_; vi[k][q] = s * pi_ + c * qi_;
-        }
+        rot[tid] = r;
       }
+      __syncthreads();
+      for (int e = tid; e < 2 * n * h; e += kPpThreads) {  // columns of A and of V
+        const int k = (e >> 1) % n;
+        const EigRot r = rot[(e >> 1) / n];
+        if (r.b < 0) continue;
+        double(*pr)[kEigLd] = (e & 1) ? vr : ar;
+        double(*pi)[kEigLd] = (e & 1) ? vi : ai;
+        const double xr = pr[k][r.a], xi = pi[k][r.a];
+        const double yr = pr[k][r.b] * r.dr - pi[k][r.b] * r.di, yi = pr[k][r.b] * r.di + pi[k][r.b] * r.dr;
+        pr[k][r.a] = r.c * xr - r.s * yr;
+        pi[k][r.a] = r.c * xi - r.s * yi;
+        pr[k][r.b] = r.s * xr + r.c * yr;
+        pi[k][r.b] = r.s * xi + r.c * yi;
+      }
+      __syncthreads();
+      for (int e = tid; e < n * h; e += kPpThreads) {  // rows of A
+        const int k = e % n;
+        const EigRot r = rot[e / n];
+        if (r.b < 0) continue;
+        const double xr = ar[r.a][k], xi = ai[r.a][k];
+        const double yr = ar[r.b][k] * r.dr + ai[r.b][k] * r.di, yi = ai[r.b][k] * r.dr - ar[r.b][k] * r.di;
+        const bool pa = k == r.a, pb = k == r.b;  // the pivot is zero, the diagonal real
+        ar[r.a][k] = pb ? 0.0 : r.c * xr - r.s * yr;
+        ai[r.a][k] = pa || pb ? 0.0 : r.c * xi - r.s * yi;
+        ar[r.b][k] = pa ? 0.0 : r.s * xr + r.c * yr;
+        ai[r.b][k] = pa || pb ? 0.0 : r.s * xi + r.c * yi;
+      }
+      __syncthreads();
+    }
   }
-  if (!converged && err) atomicExch(err, 1);
-  // order by decreasing eigenvalue (stable selection)
-  for (int i = 0; i < n; ++i) ord[i] = i;
-  for (int i = 0; i < n; ++i) {
-    int best = i;
-    for (int j = i + 1; j < n; ++j)
-      if (ar[ord[j]][ord[j]] > ar[ord[best]][ord[best]]) best = j;
-    const int tmp = ord[i]; ord[i] = ord[best]; ord[best] = tmp;
+  if (!converged && err && tid == 0) atomicExch(err, 1);
+  if (tid == 0) {  // order by decreasing eigenvalue (stable selection)
+    for (int i = 0; i < n; ++i) ord[i] = i;
+    for (int i = 0; i < n; ++i) {
+      int best = i;
+      for (int j = i + 1; j < n; ++j)
+        if (ar[ord[j]][ord[j]] > ar[ord[best]][ord[best]]) best = j;
+      const int t = ord[i];
+      ord[i] = ord[best];
+      ord[best] = t;
+    }
   }
-  for (int c = 0; c < ncomp; ++c) {
+  __syncthreads();
+  for (int c = tid; c < ncomp; c += kPpThreads) {
     const int col = ord[c];
     int im = 0;
     double mm = -1.0;
     for (int k = 0; k < n; ++k) {
       const double m2 = vr[k][col] * vr[k][col] + vi[k][col] * vi[k][col];
-      if (m2 > mm) { mm = m2; im = k; }
+      if (m2 > mm) {
+        mm = m2;
+        im = k;
+      }
     }
     const double a = sqrt(mm);
-    const double pr_ = a > 0.0 ? vr[im][col] / a : 1.0, pi_ = a > 0.0 ? -vi[im][col] / a : 0.0;  // conj phase
+    const double pr = a > 0.0 ? vr[im][col] / a : 1.0, pi = a > 0.0 ? -vi[im][col] / a : 0.0;  // conj phase
     for (int k = 0; k < n; ++k)
-      W[k * ncomp + c] = make_float2((float)(vr[k][col] * pr_ - vi[k][col] * pi_),
-                                     (float)(vr[k][col] * pi_ + vi[k][col] * pr_));
+      W[k * ncomp + c] = make_float2((float)(vr[k][col] * pr - vi[k][col] * pi), (float)(vr[k][col] * pi + vi[k][col] * pr));
   }
 }
 
@@ -193,37 +238,146 @@ __global__ void __launch_bounds__(kPpThreads) k_compress_readout(const float2* _
   }
 }
 
-// ytil[x][c][k][ky][kz] = sum_{j in segment} Phi[t_j][k] yhat[j][c][x]
+// The same for lengths nx = RA RB with two radices (run-time choice, fully unrolled butterflies).
+// One thread per x reads each channel once and forms up to eight components in registers; the
+// transform of a component is two register stages in place, an item per thread: A, DFT_RA over q of
+// x = j + RB q; B, twiddle and DFT_RB over j, straight to global memory at x = k1 + RA k2 (runs of
+// RA values).  RB values take an odd run in shared memory, so both stages are conflict free.
+// Table I scan (35,777 lines, 16 channels to 7, nx = 288): 2.05 ms with per-value contractions
+// and Stockham passes, 0.51 here (1.9 GB in and out: 0.28).
+template <int R>
+__device__ __forceinline__ void line_a(float2* b, int stride) {
+  float2 v[R];
+#pragma unroll
+  for (int q = 0; q < R; ++q) v[q] = b[q * stride];
+  dft_r<R, true>(v);
+#pragma unroll
+  for (int q = 0; q < R; ++q) b[q * stride] = v[q];
+}
+template <int R>
+__device__ __forceinline__ void line_b(const float2* b, const float2* tw, int k1, float2* out, int ostride, float s0,
+                                       float s1) {
+  float2 v[R];
+#pragma unroll
+  for (int q = 0; q < R; ++q) v[q] = b[q];
+#pragma unroll
+  for (int q = 1; q < R; ++q) v[q] = twiddle_mul<true>(v[q], tw[q * k1]);
+  dft_r<R, true>(v);
+#pragma unroll
+  for (int q = 0; q < R; ++q) out[q * ostride] = cscale(v[q], q & 1 ? s1 : s0);
+}
+constexpr int kTwoThreads = 160;  // 80 registers, five CTAs: 0.51 ms; 320 threads at 64 registers 0.56, at 96 0.62
+__global__ void __launch_bounds__(kTwoThreads, 5) k_compress_two(const float2* __restrict__ lines, const float2* __restrict__ W,
+                                                     int ctot, int ncomp, int nx, int RA, int RB, int qs,
+                                                     const float2* __restrict__ tw_g, float2* __restrict__ yh) {
+  extern __shared__ float2 smem[];
+  const int ld = RA * qs;
+  float2* tw = smem;
+  float2* ws = tw + nx;             // [ctot][8]: the components of this pass
+  float2* buf = ws + ctot * 8;      // [8][ld]
+  const long long j = blockIdx.x;
+  for (int i = threadIdx.x; i < nx; i += blockDim.x) tw[i] = tw_g[i];
+  const float scale = ((nx / 2) & 1 ? -1.f : 1.f) * rsqrtf((float)nx);
+  for (int c0 = 0; c0 < ncomp; c0 += 8) {
+    const int nc = min(8, ncomp - c0);
+    __syncthreads();
+    for (int i = threadIdx.x; i < ctot * 8; i += blockDim.x)
+      ws[i] = (i & 7) < nc ? W[(i >> 3) * ncomp + c0 + (i & 7)] : make_float2(0.f, 0.f);
+    __syncthreads();
+    for (int x = threadIdx.x; x < nx; x += blockDim.x) {
+      const float2* lp = lines + j * ctot * nx + x;
+      float2 v[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = make_float2(0.f, 0.f);
+#pragma unroll 8
+      for (int c = 0; c < ctot; ++c) {
+        const float2 a = lp[(long long)c * nx];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) cfma(v[i], a, ws[c * 8 + i]);
+      }
+      const int q = x / RB;
+      float2* b = buf + q * qs + (x - q * RB);
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (i < nc) b[i * ld] = (x & 1) ? make_float2(-v[i].x, -v[i].y) : v[i];
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < nc * RB; i += blockDim.x) {
+      const int l = i / RB;
+      float2* b = buf + l * ld + (i - l * RB);
+      switch (RA) {
+#define X(R) case R: line_a<R>(b, qs); break;
+        T2SH_RADICES(X)
+#undef X
+      }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < nc * RA; i += blockDim.x) {
+      const int l = i / RA, k1 = i - l * RA;
+      const float s0 = (k1 & 1) ? -scale : scale, s1 = (RA & 1) ? -s0 : s0;  // (-1)^(k1 + RA k2)
+      float2* o = yh + (j * ncomp + c0 + l) * nx + k1;
+      switch (RB) {
+#define X(R) case R: line_b<R>(buf + l * ld + k1 * qs, tw, k1, o, RA, s0, s1); break;
+        T2SH_RADICES(X)
+#undef X
+      }
+    }
+  }
+}
+
+// ytil[x][c][k][pixel] = sum_{j in pixel} Phi[t_j][k] yhat[j][c][x], zero where no line falls: every
+// value of the output is written once, so no clearing pass precedes it.  A CTA owns 32 pixels x
+// 32 x of one component: a warp reads runs of 32 x of the lines of its pixels, the tile is turned in
+// shared memory and written as runs of 32 pixels (256 bytes).  Writing each pixel's values where
+// they were formed (8 bytes every ncomp K N values) after clearing 4.0 GB took 3.9 + 0.6 ms for the
+// Table I scan; this takes 0.89 ms, bound by the writes.
+constexpr int kProjTile = 32, kProjOrder = 256;
+template <int KC>
 __global__ void __launch_bounds__(kPpThreads) k_project_lines(const float2* __restrict__ yh, int ncomp, int nx,
                                                             const int* __restrict__ order, const int* __restrict__ tj,
-                                                            const int* __restrict__ seg_off, const int* __restrict__ seg_y,
-                                                            const int* __restrict__ seg_z, int nseg,
-                                                            const float* __restrict__ phi, int K, int ny, int nz,
-                                                            float2* __restrict__ ytil) {
-  const long long total = (long long)nseg * ncomp * nx;
-  const long long N = (long long)ny * nz;
-  for (long long e = blockIdx.x * (long long)kPpThreads + threadIdx.x; e < total; e += (long long)gridDim.x * kPpThreads) {
-    const int x = (int)(e % nx);
-    const long long r = e / nx;
-    const int c = (int)(r % ncomp), sg = (int)(r / ncomp);
-    float2 acc[kMaxK];
+                                                            const int* __restrict__ off, const float* __restrict__ phi,
+                                                            int K, long long N, float2* __restrict__ ytil) {
+  extern __shared__ float2 tile[];  // [K][32 x][33]
+  __shared__ int soff[kProjTile + 1], sord[kProjOrder], stj[kProjOrder];
+  const long long pix0 = (long long)blockIdx.x * kProjTile;
+  const int x0 = blockIdx.y * kProjTile, c = blockIdx.z;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, x = x0 + lane;
+  if (threadIdx.x <= kProjTile) soff[threadIdx.x] = off[min(pix0 + (long long)threadIdx.x, N)];
+  __syncthreads();
+  const int q0 = soff[0], nq = soff[kProjTile] - q0;
+  for (int i = threadIdx.x; i < min(nq, kProjOrder); i += kPpThreads) {
+    sord[i] = order[q0 + i];
+    stj[i] = tj[q0 + i];
+  }
+  __syncthreads();
+  for (int p = warp; p < kProjTile; p += kPpThreads / 32) {
+    float2 acc[KC];
 #pragma unroll
-    for (int k = 0; k < kMaxK; ++k) acc[k] = make_float2(0.f, 0.f);
-    for (int q = seg_off[sg]; q < seg_off[sg + 1]; ++q) {
-      const float2 v = yh[((long long)order[q] * ncomp + c) * nx + x];
-      const float* ph = phi + (long long)tj[q] * K;
+    for (int k = 0; k < KC; ++k) acc[k] = make_float2(0.f, 0.f);
+    const int e1 = soff[p + 1] - q0;
+#pragma unroll 2
+    for (int i = soff[p] - q0; i < e1; ++i) {
+      const int j = i < kProjOrder ? sord[i] : order[q0 + i], t = i < kProjOrder ? stj[i] : tj[q0 + i];
+      const float2 v = x < nx ? yh[((long long)j * ncomp + c) * nx + x] : make_float2(0.f, 0.f);
+      const float* ph = phi + (long long)t * K;
 #pragma unroll
-      for (int k = 0; k < kMaxK; ++k)
+      for (int k = 0; k < KC; ++k)
         if (k < K) {
           acc[k].x = fmaf(ph[k], v.x, acc[k].x);
           acc[k].y = fmaf(ph[k], v.y, acc[k].y);
         }
     }
-    const long long pix = (long long)seg_y[sg] * nz + seg_z[sg];
-    float2* o = ytil + ((long long)x * ncomp + c) * K * N + pix;
 #pragma unroll
-    for (int k = 0; k < kMaxK; ++k)
-      if (k < K) o[k * N] = acc[k];
+    for (int k = 0; k < KC; ++k)
+      if (k < K) tile[(k * kProjTile + lane) * (kProjTile + 1) + p] = acc[k];
+  }
+  __syncthreads();
+  if (pix0 + lane >= N) return;
+  for (int r = warp; r < K * kProjTile; r += kPpThreads / 32) {
+    const int k = r / kProjTile, xx = r - k * kProjTile;
+    if (x0 + xx < nx)
+      __stcs(ytil + (((long long)(x0 + xx) * ncomp + c) * K + k) * N + pix0 + lane,
+             tile[(k * kProjTile + xx) * (kProjTile + 1) + lane]);
   }
 }
 
@@ -240,11 +394,11 @@ int grid_for(long long total) {
 
 }  // namespace
 
-cudaError_t launch_calib(const float2* lines, int ctot, int nx, const int* order, const int* seg_off, const int* wseg,
-                         int nwseg, int win, float2* X, cudaStream_t st) {
-  const long long total = (long long)nwseg * win * ctot;
+cudaError_t launch_calib(const float2* lines, int ctot, int nx, const int* order, const int* off, const int* wpix,
+                         int nwpix, int win, float2* X, cudaStream_t st) {
+  const long long total = (long long)nwpix * win * ctot;
   if (total == 0) return cudaSuccess;
-  k_calib<<<grid_for(total), kPpThreads, 0, st>>>(lines, ctot, nx, order, seg_off, wseg, nwseg, win, X);
+  k_calib<<<grid_for(total), kPpThreads, 0, st>>>(lines, ctot, nx, order, off, wpix, nwpix, win, X);
   return cudaGetLastError();
 }
 
@@ -256,13 +410,22 @@ cudaError_t launch_gram_eig(const float2* X, long long npts, int ctot, int ncomp
   cudaError_t e = cudaMemsetAsync(G, 0, sizeof(double) * 2 * ctot * ctot, st);
   if (e != cudaSuccess) return e;
   if (nb > 0) k_gram<<<(unsigned)nb, kPpThreads, 0, st>>>(X, npts, ctot, chunk, G);
-  k_eig<<<1, 32, 0, st>>>(G, ctot, ncomp, W, err);
+  k_eig<<<1, kPpThreads, 0, st>>>(G, ctot, ncomp, W, err);
   return cudaGetLastError();
 }
 
 cudaError_t launch_compress_readout(const float2* lines, const float2* W, int nlines, int ctot, int ncomp,
                                     const FftPlan& px, const float2* tw_x, float2* yh, cudaStream_t st) {
   const int nx = px.n;
+  int RA = 0, RB = 0;
+  if (two_radices(nx, kMaxRadix, false, &RA, &RB)) {
+    const int qs = RB | 1, threads = std::min(kTwoThreads, (nx + 31) / 32 * 32);
+    const size_t sm = sizeof(float2) * ((size_t)nx + 8 * ctot + 8 * (size_t)RA * qs);
+    const cudaError_t e = smem_optin((const void*)k_compress_two, 64 * 1024);
+    if (e != cudaSuccess) return e;
+    k_compress_two<<<nlines, threads, sm, st>>>(lines, W, ctot, ncomp, nx, RA, RB, qs, tw_x, yh);
+    return cudaGetLastError();
+  }
   int cb = (kStage * kPpThreads) / nx;
   if (cb < 1) return cudaErrorInvalidValue;
   if (cb > ncomp) cb = ncomp;
@@ -284,13 +447,18 @@ cudaError_t launch_compress_readout(const float2* lines, const float2* W, int nl
   return cudaGetLastError();
 }
 
-cudaError_t launch_project_lines(const float2* yh, int ncomp, int nx, const int* order, const int* tj,
-                                 const int* seg_off, const int* seg_y, const int* seg_z, int nseg, const float* phi,
-                                 int K, int ny, int nz, float2* ytil, cudaStream_t st) {
-  const long long total = (long long)nseg * ncomp * nx;
-  if (total == 0) return cudaSuccess;
-  k_project_lines<<<grid_for(total), kPpThreads, 0, st>>>(yh, ncomp, nx, order, tj, seg_off, seg_y, seg_z, nseg, phi,
-                                                          K, ny, nz, ytil);
+cudaError_t launch_project_lines(const float2* yh, int ncomp, int nx, const int* order, const int* tj, const int* off,
+                                 const float* phi, int K, int ny, int nz, float2* ytil, cudaStream_t st) {
+  const long long N = (long long)ny * nz;
+  dim3 grid((unsigned)((N + kProjTile - 1) / kProjTile), (nx + kProjTile - 1) / kProjTile, ncomp);
+  const size_t sm = sizeof(float2) * (size_t)K * kProjTile * (kProjTile + 1);
+  const void* kern = K <= 4 ? (const void*)k_project_lines<4> : (const void*)k_project_lines<8>;
+  const cudaError_t e = smem_optin(kern, 72 * 1024);
+  if (e != cudaSuccess) return e;
+  if (K <= 4)
+    k_project_lines<4><<<grid, kPpThreads, sm, st>>>(yh, ncomp, nx, order, tj, off, phi, K, N, ytil);
+  else
+    k_project_lines<8><<<grid, kPpThreads, sm, st>>>(yh, ncomp, nx, order, tj, off, phi, K, N, ytil);
   return cudaGetLastError();
 }
 

@@ -231,6 +231,7 @@ namespace t2sh {
 t2sh_status check_dims(const t2sh_dims* d) { return validate(d); }
 bool fft_plan_for(int n, FftPlan& p) { return make_fft_plan(n, p); }
 void set_last_error(const char* msg) { g_err = msg; }
+cudaMemPool_t library_pool() { return stage_pool(); }
 }  // namespace t2sh
 
 struct t2sh_plan_s {

@@ -128,15 +128,14 @@ cudaError_t launch_post_il_b(const Geom& g, const float2* tw, const float2* maps
 cudaError_t launch_post_il_c(const Geom& g, const float2* tw, const float2* maps, const float* phi, const float2* alpha,
                              const PostArgs& pa, float* out, cudaStream_t st);
 // pre-processing from sparse readout lines (k_preproc.cu)
-cudaError_t launch_calib(const float2* lines, int ctot, int nx, const int* order, const int* seg_off, const int* wseg,
-                         int nwseg, int win, float2* X, cudaStream_t st);
+cudaError_t launch_calib(const float2* lines, int ctot, int nx, const int* order, const int* off, const int* wpix,
+                         int nwpix, int win, float2* X, cudaStream_t st);
 cudaError_t launch_gram_eig(const float2* X, long long npts, int ctot, int ncomp, double* G, float2* W, int* err,
                             cudaStream_t st);
 cudaError_t launch_compress_readout(const float2* lines, const float2* W, int nlines, int ctot, int ncomp,
                                     const FftPlan& px, const float2* tw_x, float2* yh, cudaStream_t st);
-cudaError_t launch_project_lines(const float2* yh, int ncomp, int nx, const int* order, const int* tj,
-                                 const int* seg_off, const int* seg_y, const int* seg_z, int nseg, const float* phi,
-                                 int K, int ny, int nz, float2* ytil, cudaStream_t st);
+cudaError_t launch_project_lines(const float2* yh, int ncomp, int nx, const int* order, const int* tj, const int* off,
+                                 const float* phi, int K, int ny, int nz, float2* ytil, cudaStream_t st);
 cudaError_t launch_mark_mask(const int* t, const int* ky, const int* kz, int n, int ny, int nz, uint8_t* mask,
                              cudaStream_t st);
 // ADMM v-update: w = alpha + u, v = LLR prox of w (threshold a.tau, shift a.sy/a.sz), u <- w - v
@@ -209,6 +208,10 @@ cudaError_t launch_col_adj_tma(const Geom& g, const float2* tw_y, const float2* 
 bool band_fused_supported(const Geom& g, int block);
 cudaError_t launch_band_fused(const Geom& g, const FistaArgs& a, const float2* tw_z, const float2* maps, float2* t,
                               float2* x, float2* z, const float2* aty, cudaStream_t st);
+
+// The library's stream-ordered pool of the current device (nullptr if unavailable): it keeps its
+// memory until t2sh_release_cached.
+cudaMemPool_t library_pool();
 
 // Per-device launch set-up shared by the launchers (a process may drive several GPUs):
 // a kernel's dynamic shared-memory limit is raised once per (kernel, device), and the

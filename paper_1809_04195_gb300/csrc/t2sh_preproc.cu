@@ -1,8 +1,9 @@
 // Host side of the pre-processing entry points (t2sh_coil_compression, t2sh_preprocess):
-// argument checks, the (ky, kz) segment table of the sparse lines, stream-ordered scratch.
+// argument checks, the table of the sparse lines by phase encode, stream-ordered scratch.
 #include <algorithm>
 #include <cmath>
-#include <numeric>
+#include <cstring>
+#include <new>
 #include <vector>
 
 #include "../../include/t2sh.h"
@@ -41,51 +42,80 @@ t2sh_status check_sparse(const t2sh_sparse* sp) {
   return T2SH_OK;
 }
 
-struct Segments {
-  std::vector<int> order, t_sorted, off, y, z;
+// The lines grouped (stably) by phase encode ky nz + kz: pixel p owns order[off[p]] ..
+// order[off[p + 1] - 1].  A counting sort: two passes over the lines (a comparison sort of the
+// Table I scan's 35,777 lines took 2 ms of host time per call).
+struct Groups {
+  std::vector<int> order, t_sorted, off;
 };
-
-// lines sorted (stably) by phase encode; one segment per distinct (ky, kz)
-void build_segments(const t2sh_sparse* sp, Segments& s) {
+// the window [y0, y0 + ny) x [z0, z0 + nz) of phase encodes; lines outside it are left out
+void build_groups(const t2sh_sparse* sp, int y0, int z0, int ny, int nz, Groups& s) {
   const int n = sp->nlines;
-  s.order.resize(n);
-  std::iota(s.order.begin(), s.order.end(), 0);
-  std::stable_sort(s.order.begin(), s.order.end(), [&](int a, int b) {
-    return (long long)sp->ky[a] * sp->nz + sp->kz[a] < (long long)sp->ky[b] * sp->nz + sp->kz[b];
-  });
-  s.t_sorted.resize(n);
-  for (int q = 0; q < n; ++q) {
-    const int j = s.order[q];
-    s.t_sorted[q] = sp->t[j];
-    if (q == 0 || sp->ky[j] != sp->ky[s.order[q - 1]] || sp->kz[j] != sp->kz[s.order[q - 1]]) {
-      s.off.push_back(q);
-      s.y.push_back(sp->ky[j]);
-      s.z.push_back(sp->kz[j]);
+  const size_t N = (size_t)ny * nz;
+  auto pixel = [&](int j, size_t* p) {
+    const int y = sp->ky[j] - y0, z = sp->kz[j] - z0;
+    *p = (size_t)y * nz + z;
+    return y >= 0 && y < ny && z >= 0 && z < nz;
+  };
+  size_t p;
+  s.off.assign(N + 1, 0);
+  for (int j = 0; j < n; ++j)
+    if (pixel(j, &p)) ++s.off[p + 1];
+  for (size_t i = 0; i < N; ++i) s.off[i + 1] += s.off[i];
+  std::vector<int> next(s.off.begin(), s.off.end() - 1);
+  s.order.resize(s.off[N]);
+  s.t_sorted.resize(s.off[N]);
+  for (int j = 0; j < n; ++j)
+    if (pixel(j, &p)) {
+      const int q = next[p]++;
+      s.order[q] = j;
+      s.t_sorted[q] = sp->t[j];
     }
-  }
-  s.off.push_back(n);
 }
 
-// stream-ordered device copies of host tables; freed with release()
+// Stream-ordered scratch from the library's pool (which keeps its memory between calls, so a call
+// maps no fresh pages), freed in stream order.  Host tables are packed into one buffer and cross
+// in one copy.
 struct Scratch {
   cudaStream_t st;
   std::vector<void*> ptrs;
+  std::vector<unsigned char> host;
+  unsigned char* dev = nullptr;
   explicit Scratch(cudaStream_t s) : st(s) {}
   template <typename T>
   cudaError_t alloc(T** p, size_t n) {
     void* q = nullptr;
-    cudaError_t e = cudaMallocAsync(&q, n ? n * sizeof(T) : 16, st);
+    const size_t b = n ? n * sizeof(T) : 16;
+    cudaMemPool_t pool = library_pool();
+    cudaError_t e = pool ? cudaMallocFromPoolAsync(&q, b, pool, st) : cudaMallocAsync(&q, b, st);
+    if (e != cudaSuccess && pool) {  // hand the pool's unused memory back and try once more
+      cudaGetLastError();
+      cudaStreamSynchronize(st);
+      cudaMemPoolTrimTo(pool, 0);
+      e = cudaMallocFromPoolAsync(&q, b, pool, st);
+    }
     if (e == cudaSuccess) {
       ptrs.push_back(q);
       *p = static_cast<T*>(q);
     }
     return e;
   }
+  // place of n values in the packed tables
   template <typename T>
-  cudaError_t upload(T** p, const std::vector<T>& v) {
-    cudaError_t e = alloc(p, v.size());
-    if (e == cudaSuccess && !v.empty()) e = cudaMemcpyAsync(*p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, st);
+  size_t add(const T* v, size_t n) {
+    const size_t at = (host.size() + 255) / 256 * 256;
+    host.resize(at + n * sizeof(T));
+    if (n) std::memcpy(host.data() + at, v, n * sizeof(T));
+    return at;
+  }
+  cudaError_t upload() {
+    cudaError_t e = alloc(&dev, host.size());
+    if (e == cudaSuccess) e = cudaMemcpyAsync(dev, host.data(), host.size(), cudaMemcpyHostToDevice, st);
     return e;
+  }
+  template <typename T>
+  const T* table(size_t at) const {
+    return reinterpret_cast<const T*>(dev + at);
   }
   ~Scratch() {
     for (void* q : ptrs) cudaFreeAsync(q, st);
@@ -112,28 +142,31 @@ t2sh_status t2sh_coil_compression(const t2sh_sparse* sp, const void* lines, int3
   if (window < 1 || window > sp->nx || window > sp->ny || window > sp->nz)
     return fail(T2SH_EINVAL, "window must be in [1, min(nx, ny, nz)]");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  Segments sg;
-  build_segments(sp, sg);
-  const int y0 = sp->ny / 2 - window / 2, z0 = sp->nz / 2 - window / 2;
-  std::vector<int> wseg;
-  for (size_t i = 0; i + 1 < sg.off.size(); ++i)
-    if (sg.y[i] >= y0 && sg.y[i] < y0 + window && sg.z[i] >= z0 && sg.z[i] < z0 + window) wseg.push_back((int)i);
-  if (wseg.empty()) return fail(T2SH_EINVAL, "no line falls in the calibration window");
+  Groups sg;
+  std::vector<int> wpix;  // sampled phase encodes of the window
+  try {
+    build_groups(sp, sp->ny / 2 - window / 2, sp->nz / 2 - window / 2, window, window, sg);
+    for (int p = 0; p < window * window; ++p)
+      if (sg.off[p + 1] > sg.off[p]) wpix.push_back(p);
+  } catch (const std::bad_alloc&) {
+    return fail(T2SH_ENOMEM, "host allocation failed");
+  }
+  if (wpix.empty()) return fail(T2SH_EINVAL, "no line falls in the calibration window");
   {
     Scratch sc(st);
-    int *order = nullptr, *off = nullptr, *wsg = nullptr, *err = nullptr;
+    int* err = nullptr;
     float2* X = nullptr;
     double* G = nullptr;
-    const long long npts = (long long)wseg.size() * window;
-    PP_CK(sc.upload(&order, sg.order));
-    PP_CK(sc.upload(&off, sg.off));
-    PP_CK(sc.upload(&wsg, wseg));
+    const long long npts = (long long)wpix.size() * window;
+    const size_t a_order = sc.add(sg.order.data(), sg.order.size()), a_off = sc.add(sg.off.data(), sg.off.size()),
+                 a_w = sc.add(wpix.data(), wpix.size());
+    PP_CK(sc.upload());
     PP_CK(sc.alloc(&X, (size_t)npts * sp->nchan));
     PP_CK(sc.alloc(&G, 2 * (size_t)sp->nchan * sp->nchan));
     PP_CK(sc.alloc(&err, 1));
     PP_CK(cudaMemsetAsync(err, 0, sizeof(int), st));
-    PP_CK(launch_calib(static_cast<const float2*>(lines), sp->nchan, sp->nx, order, off, wsg, (int)wseg.size(), window,
-                       X, st));
+    PP_CK(launch_calib(static_cast<const float2*>(lines), sp->nchan, sp->nx, sc.table<int>(a_order),
+                       sc.table<int>(a_off), sc.table<int>(a_w), (int)wpix.size(), window, X, st));
     PP_CK(launch_gram_eig(X, npts, sp->nchan, ncomp, G, static_cast<float2*>(w_out), err, st));
     int herr = 0;
     PP_CK(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -154,9 +187,12 @@ t2sh_status t2sh_preprocess(const t2sh_sparse* sp, const void* lines, const void
   FftPlan px{};
   if (!fft_plan_for(sp->nx, px)) return fail(T2SH_EINVAL, "no radix plan for nx");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  Segments sg;
-  build_segments(sp, sg);
-  const int nseg = (int)sg.off.size() - 1;
+  Groups sg;
+  try {
+    build_groups(sp, 0, 0, sp->ny, sp->nz, sg);
+  } catch (const std::bad_alloc&) {
+    return fail(T2SH_ENOMEM, "host allocation failed");
+  }
   std::vector<float2> tw(sp->nx);
   for (int m = 0; m < sp->nx; ++m) {
     const double a = -2.0 * 3.14159265358979323846 * m / sp->nx;
@@ -164,27 +200,20 @@ t2sh_status t2sh_preprocess(const t2sh_sparse* sp, const void* lines, const void
   }
   {
     Scratch sc(st);
-    int *order = nullptr, *ts = nullptr, *off = nullptr, *sy = nullptr, *sz = nullptr, *tl = nullptr, *kyl = nullptr,
-        *kzl = nullptr;
-    float2 *yh = nullptr, *twd = nullptr;
-    PP_CK(sc.upload(&order, sg.order));
-    PP_CK(sc.upload(&ts, sg.t_sorted));
-    PP_CK(sc.upload(&off, sg.off));
-    PP_CK(sc.upload(&sy, sg.y));
-    PP_CK(sc.upload(&sz, sg.z));
-    PP_CK(sc.upload(&tl, std::vector<int>(sp->t, sp->t + sp->nlines)));
-    PP_CK(sc.upload(&kyl, std::vector<int>(sp->ky, sp->ky + sp->nlines)));
-    PP_CK(sc.upload(&kzl, std::vector<int>(sp->kz, sp->kz + sp->nlines)));
-    PP_CK(sc.upload(&twd, tw));
+    float2* yh = nullptr;
+    const size_t n = sp->nlines;
+    const size_t a_order = sc.add(sg.order.data(), n), a_ts = sc.add(sg.t_sorted.data(), n),
+                 a_off = sc.add(sg.off.data(), sg.off.size()), a_t = sc.add(sp->t, n), a_ky = sc.add(sp->ky, n),
+                 a_kz = sc.add(sp->kz, n), a_tw = sc.add(tw.data(), tw.size());
+    PP_CK(sc.upload());
     PP_CK(sc.alloc(&yh, (size_t)sp->nlines * ncomp * sp->nx));
-    const size_t ybytes = sizeof(float2) * (size_t)sp->nx * ncomp * nbasis * sp->ny * sp->nz;
-    PP_CK(cudaMemsetAsync(ytil_out, 0, ybytes, st));
     PP_CK(cudaMemsetAsync(mask_out, 0, (size_t)sp->nechoes * sp->ny * sp->nz, st));
     PP_CK(launch_compress_readout(static_cast<const float2*>(lines), static_cast<const float2*>(w), sp->nlines,
-                                  sp->nchan, ncomp, px, twd, yh, st));
-    PP_CK(launch_project_lines(yh, ncomp, sp->nx, order, ts, off, sy, sz, nseg, phi, nbasis, sp->ny, sp->nz,
-                               static_cast<float2*>(ytil_out), st));
-    PP_CK(launch_mark_mask(tl, kyl, kzl, sp->nlines, sp->ny, sp->nz, mask_out, st));
+                                  sp->nchan, ncomp, px, sc.table<float2>(a_tw), yh, st));
+    PP_CK(launch_project_lines(yh, ncomp, sp->nx, sc.table<int>(a_order), sc.table<int>(a_ts), sc.table<int>(a_off),
+                               phi, nbasis, sp->ny, sp->nz, static_cast<float2*>(ytil_out), st));
+    PP_CK(launch_mark_mask(sc.table<int>(a_t), sc.table<int>(a_ky), sc.table<int>(a_kz), sp->nlines, sp->ny, sp->nz,
+                           mask_out, st));
   }
   return T2SH_OK;
 }

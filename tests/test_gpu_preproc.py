@@ -78,6 +78,34 @@ def test_preprocess_repeated_lines_add(T):
     assert nrmse(host(ytil), ref) < 1e-5
 
 
+@pytest.mark.parametrize("nchan,ncomp,nx,ny,nz,Tn,K,frac", [
+    (4, 3, 52, 8, 6, 40, 6, 0.9),     # more lines per tile of pixels than are staged, N not a multiple of 32
+    (3, 1, 34 - 2, 6, 6, 9, 8, 0.5),  # one x tile, eight images
+    (16, 11, 50, 10, 14, 6, 4, 0.1),  # components in two groups of eight, empty pixels
+])
+def test_projection_tiles(T, nchan, ncomp, nx, ny, nz, Tn, K, frac):
+    lines, t, a, b, mask = sparse_scan(nchan + nx + Tn, nchan, nx, ny, nz, Tn, frac)
+    rng = np.random.default_rng(nx)
+    W = np.linalg.qr(crandn(rng, nchan, ncomp))[0].astype(np.complex64).astype(np.complex128)
+    phi = synth.t2_basis(Tn, K).astype(np.float32).astype(np.float64)
+    ytil, m = T.preprocess(c64(lines), t, a, b, c64(W), dev(phi.astype(np.float32)), ny, nz)
+    ref, mref = O.preprocess(lines, t, a, b, W, phi, ny, nz)
+    assert np.array_equal(m.cpu().numpy(), mref) and nrmse(host(ytil), ref) < 1e-5
+    assert np.all(host(ytil)[:, :, :, mref.sum(0) == 0] == 0)
+
+
+@pytest.mark.parametrize("nchan", [1, 2, 3, 7, 31, 32])
+def test_channel_eigenvectors_of_any_count(T, nchan):
+    """Odd and even channel counts, the smallest and the largest; geometric energies keep the
+    eigenvectors defined to float precision (entries within 1e-4, as above)."""
+    rank = min(nchan, 6)
+    lines, t, a, b, mask = sparse_scan(60 + nchan, nchan, 16, 12, 10, 6, 0.4, ncoil_rank=rank)
+    ncomp = max(1, rank - 1)
+    got = host(T.coil_compression(c64(lines), t, a, b, 12, 10, 6, window=8, ncomp=ncomp))
+    ref = O.compression_matrix(O.calibration_average(lines, a, b, 12, 10, 8), ncomp)
+    assert np.abs(got - ref).max() < 1e-4
+
+
 def test_sparse_lines_to_reconstruction(T):
     """Chain: sparse lines of a synthetic scan (fully sampled readout, per-echo masks) ->
     coil compression -> decoupling and projection -> FISTA on three readout slices, against

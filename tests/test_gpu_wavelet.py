@@ -13,7 +13,7 @@ import oracle as O
 import t2sh_synth as synth
 
 from t2sh_cases import crandn
-from test_gpu_parity import T, c64, make_plan, nrmse, random_problem  # noqa: F401
+from test_gpu_parity import T, c64, host, make_plan, nrmse, random_problem  # noqa: F401
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
