@@ -76,7 +76,7 @@ __device__ __forceinline__ int llr_row0(const Geom& g, const FistaArgs& a, const
 
 // 1. gather the band into gs [K][rb][llr_ld(nz)] (gradient step fused for FISTA), threads
 // t0 .. t0 + nth - 1 of the CTA
-template <int MODE>
+template <int KC, int MODE>
 __device__ __forceinline__ void llr_gather(const Geom& g, const FistaArgs& a, const LlrUnit& un, float2* gs,
                                            const float2* x, const float2* z, const float2* __restrict__ grad,
                                            const float2* __restrict__ aty, const float2* u, int t0, int nth) {
@@ -85,38 +85,39 @@ __device__ __forceinline__ void llr_gather(const Geom& g, const FistaArgs& a, co
   if (!c.active) return;
   const int y0 = llr_row0(g, a, un);
   const long long base = ((long long)un.s * g.M + un.m0) * K * (long long)N + 2 * c.c2;
-  int k = 0, r = c.lp;
-  while (r >= rb) {
-    r -= rb;
-    ++k;
-  }
-#pragma unroll 4
-  for (int l = c.lp; l < K * rb; l += c.P) {
+  const float2 *xb = x + base, *zb = z + base, *gb = grad + base, *ab = aty + base, *ub = u + base;
+  const int ld = llr_ld(nz);
+  // all images of a row in one step: one row offset, and the loads of KC images in flight together.
+  // Global-space loads (ld.global.cg): the compiler may batch them ahead of the shared-memory
+  // stores, which generic loads could alias
+  for (int r = c.lp; r < rb; r += c.P) {
     int y = y0 + r;
     y -= y >= ny ? ny : 0;
-    const long long gi = base + (long long)k * N + (long long)y * nz;
-    float4 v;
-    // global-space loads (ld.global.cg): the compiler may then batch them across iterations
-    // ahead of the shared-memory stores, which generic loads could alias
-    if (MODE == LLR_ADMM) {
-      const float4 av = __ldcg(reinterpret_cast<const float4*>(x + gi));
-      const float4 uv = __ldcg(reinterpret_cast<const float4*>(u + gi));
-      v = make_float4(av.x + uv.x, av.y + uv.y, av.z + uv.z, av.w + uv.w);
-    } else if (MODE == LLR_FISTA) {
-      const float4 zv = __ldcg(reinterpret_cast<const float4*>(z + gi));
-      const float4 gv = __ldcg(reinterpret_cast<const float4*>(grad + gi));
-      const float4 av = __ldcg(reinterpret_cast<const float4*>(aty + gi));
-      v = make_float4(zv.x - a.mu * (gv.x - av.x), zv.y - a.mu * (gv.y - av.y), zv.z - a.mu * (gv.z - av.z),
-                      zv.w - a.mu * (gv.w - av.w));
-    } else {
-      v = __ldcg(reinterpret_cast<const float4*>(x + gi));
+    const int row = y * nz;
+    float2* gr = gs + r * ld + 2 * c.c2;
+    float4 v[KC];
+#pragma unroll
+    for (int k = 0; k < KC; ++k) {
+      if (k < K) {
+        const int gi = row + k * N;
+        if (MODE == LLR_ADMM) {
+          const float4 av = __ldcg(reinterpret_cast<const float4*>(xb + gi));
+          const float4 uv = __ldcg(reinterpret_cast<const float4*>(ub + gi));
+          v[k] = make_float4(av.x + uv.x, av.y + uv.y, av.z + uv.z, av.w + uv.w);
+        } else if (MODE == LLR_FISTA) {
+          const float4 zv = __ldcg(reinterpret_cast<const float4*>(zb + gi));
+          const float4 gv = __ldcg(reinterpret_cast<const float4*>(gb + gi));
+          const float4 av = __ldcg(reinterpret_cast<const float4*>(ab + gi));
+          v[k] = make_float4(zv.x - a.mu * (gv.x - av.x), zv.y - a.mu * (gv.y - av.y), zv.z - a.mu * (gv.z - av.z),
+                             zv.w - a.mu * (gv.w - av.w));
+        } else {
+          v[k] = __ldcg(reinterpret_cast<const float4*>(xb + gi));
+        }
+      }
     }
-    *reinterpret_cast<float4*>(gs + (long long)l * llr_ld(nz) + 2 * c.c2) = v;
-    r += c.P;
-    while (r >= rb) {
-      r -= rb;
-      ++k;
-    }
+#pragma unroll
+    for (int k = 0; k < KC; ++k)
+      if (k < K) *reinterpret_cast<float4*>(gr + k * rb * ld) = v[k];
   }
 }
 
@@ -152,17 +153,32 @@ __device__ __forceinline__ void llr_gram(const Geom& g, const FistaArgs& a, cons
           if (l > k) gr[l][k] = fmaf(xv[k].x, xv[l].y, fmaf(-xv[k].y, xv[l].x, gr[l][k]));
         }
     }
+    // sums over the lanes by halving: in each step a lane hands half of its values to its partner and
+    // keeps the other half's sums (the same pairwise sums as a butterfly per value, at an eighth of
+    // its shuffles), until lane i holds entry i
+    float* val = &gr[0][0];
+    constexpr int NV = KC * KC;
 #pragma unroll
-    for (int k = 0; k < KC; ++k)
+    for (int st = 0; st < 5; ++st) {
+      const int o = 16 >> st, n = NV >> st;  // lanes to the partner, values before the step
+      if (n > 1) {
+        const bool up = lane & o;  // keeps the upper half
 #pragma unroll
-      for (int l = 0; l < KC; ++l)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) gr[k][l] += __shfl_xor_sync(0xffffffffu, gr[k][l], o);
-    if (lane == 0) {
-#pragma unroll
-      for (int k = 0; k < KC; ++k)
-#pragma unroll
-        for (int l = 0; l < KC; ++l) gram[blk * kGramStride<KC> + k * KC + l] = gr[k][l];
+        for (int i = 0; i < n / 2; ++i) {
+          const float send = up ? val[i] : val[i + n / 2];
+          const float keep = up ? val[i + n / 2] : val[i];
+          val[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+      } else {
+        val[0] += __shfl_xor_sync(0xffffffffu, val[0], o);
+      }
+    }
+    // entry of this lane: bit 4 of the lane chose the half of the first step, and so on
+    if constexpr (NV == 16) {
+      if (!(lane & 1)) gram[blk * kGramStride<KC> + (lane >> 1)] = val[0];
+    } else {
+      gram[blk * kGramStride<KC> + 2 * lane] = val[0];
+      gram[blk * kGramStride<KC> + 2 * lane + 1] = val[1];
     }
   }
 }
@@ -193,20 +209,23 @@ __device__ __forceinline__ void llr_apply(const Geom& g, const FistaArgs& a, con
   const float2* w1 = wm + (size_t)(d1 / b) * kWStride<KC>;
   const int y0 = llr_row0(g, a, un);
   const long long gb0 = ((long long)(un.s * g.M + un.m0) * K) * N + zz;
+  float2 *xb = x + gb0, *zb = z + gb0, *ub = u + gb0;
+  const int ld = llr_ld(nz);
   for (int r = c.lp; r < rb; r += c.P) {
     int y = y0 + r;
     y -= y >= ny ? ny : 0;
+    const float2* gr = gs + r * ld + zz;
     float4 xv[KC];  // (pixel zz, pixel zz + 1) of each basis image
 #pragma unroll
     for (int k = 0; k < KC; ++k)
-      xv[k] = (k < K) ? *reinterpret_cast<const float4*>(gs + (k * rb + r) * llr_ld(nz) + zz)
+      xv[k] = (k < K) ? *reinterpret_cast<const float4*>(gr + k * rb * ld)
                       : make_float4(0.f, 0.f, 0.f, 0.f);
-    const long long gb = gb0 + (long long)y * nz;
+    const int gb = y * nz;
     float4 xp[KC];  // x_k of the pair in every basis image, requested before any store of the row
     if (MODE == LLR_FISTA) {
 #pragma unroll
       for (int k = 0; k < KC; ++k)
-        xp[k] = (k < K) ? *reinterpret_cast<const float4*>(x + gb + (long long)k * N) : make_float4(0.f, 0.f, 0.f, 0.f);
+        xp[k] = (k < K) ? *reinterpret_cast<const float4*>(xb + gb + k * N) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
 #pragma unroll
     for (int k = 0; k < KC; ++k) {
@@ -219,29 +238,29 @@ __device__ __forceinline__ void llr_apply(const Geom& g, const FistaArgs& a, con
         }
         const float4 o = make_float4(o0.x, o0.y, o1.x, o1.y);
         const float4 xk = xv[k];
-        const long long gi = gb + (long long)k * N;
+        const int gi = gb + k * N;
         if (MODE == LLR_ADMM) {
           if (want_res) {
-            const float4 zo = *reinterpret_cast<const float4*>(z + gi);
+            const float4 zo = *reinterpret_cast<const float4*>(zb + gi);
             const float dx0 = o.x - zo.x, dy0 = o.y - zo.y, dx1 = o.z - zo.z, dy1 = o.w - zo.w;
             d2 = fmaf(dx0, dx0, fmaf(dy0, dy0, fmaf(dx1, dx1, fmaf(dy1, dy1, d2))));
             x2 = fmaf(o.x, o.x, fmaf(o.y, o.y, fmaf(o.z, o.z, fmaf(o.w, o.w, x2))));
           }
-          *reinterpret_cast<float4*>(z + gi) = o;
-          *reinterpret_cast<float4*>(u + gi) = make_float4(xk.x - o.x, xk.y - o.y, xk.z - o.z, xk.w - o.w);
+          *reinterpret_cast<float4*>(zb + gi) = o;
+          *reinterpret_cast<float4*>(ub + gi) = make_float4(xk.x - o.x, xk.y - o.y, xk.z - o.z, xk.w - o.w);
           continue;
         }
         if (MODE == LLR_FISTA) {
           const float4 xo = xp[k];
           const float4 dx = make_float4(o.x - xo.x, o.y - xo.y, o.z - xo.z, o.w - xo.w);
-          *reinterpret_cast<float4*>(z + gi) =
+          *reinterpret_cast<float4*>(zb + gi) =
               make_float4(o.x + a.beta * dx.x, o.y + a.beta * dx.y, o.z + a.beta * dx.z, o.w + a.beta * dx.w);
           if (want_res) {
             d2 = fmaf(dx.x, dx.x, fmaf(dx.y, dx.y, fmaf(dx.z, dx.z, fmaf(dx.w, dx.w, d2))));
             x2 = fmaf(o.x, o.x, fmaf(o.y, o.y, fmaf(o.z, o.z, fmaf(o.w, o.w, x2))));
           }
         }
-        *reinterpret_cast<float4*>(x + gi) = o;
+        *reinterpret_cast<float4*>(xb + gi) = o;
       }
     }
   }
@@ -290,7 +309,7 @@ __device__ __forceinline__ void llr_band(const Geom& g, const FistaArgs& a, int 
   float2* gs = smem;                                         // [K][rb][llr_ld(nz)]
   float2* wm = gs + (size_t)g.K * un.rb * llr_ld(g.nz);      // [nbz][kWStride]: KC x KC weights
   float* gram = reinterpret_cast<float*>(wm + (size_t)nbz * kWStride<KC>);  // [nbz][kGramStride]
-  llr_gather<MODE>(g, a, un, gs, x, z, grad, aty, u, 0, NT);
+  llr_gather<KC, MODE>(g, a, un, gs, x, z, grad, aty, u, 0, NT);
   __syncthreads();
   llr_gram<KC>(g, a, un, gs, gram, 0, NT / 32);
   __syncthreads();
