@@ -18,6 +18,7 @@
 #include <algorithm>
 
 #define T2SH_PACKED_ADD 1
+#include "launch.h"
 #include "t2sh_device.cuh"
 #include "two_radix.h"
 
@@ -118,6 +119,8 @@ __global__ void __launch_bounds__(kColThreads, KC == 4 ? 3 : 2)
       }
     }
   };
+  pdl_wait();
+  pdl_trigger();
   if (fwd && lo < hi) issue(lo, bufs);
   cp_async_commit();
   int have = -1;  // column chunk whose Psi is in shared memory
@@ -320,8 +323,10 @@ __global__ void __launch_bounds__(kRowThreads, MC == 1 ? 3 : 2)
       for (int i = threadIdx.x; i < rb * h; i += blockDim.x)  // the band's rows are contiguous
         cp_async16(md + m * rows * N + 2 * i, mp + (long long)m * NN + 2 * i);
   };
-  issue(0, 0);
+  issue(0, 0);  // the plan's maps
   cp_async_commit();
+  pdl_wait();
+  pdl_trigger();
   const int y = y0 + r;
   const int slot = a.trb ? (k + y % a.trb + y / a.trb) & 3 : k;
   float2* tp = t + ((long long)s * g.C * g.ny + y) * (K * N) + slot * a.W;
@@ -446,11 +451,8 @@ cudaError_t launch_col_any(const Geom& g, int W, IlPass pass, const float2* tw_y
   if (e == cudaSuccess) e = ctas_per_sm(kern, threads, sm, &per);
   if (e != cudaSuccess) return e;
   const int grid = (int)std::min<long long>(ntiles, (long long)nsm * per);
-  if (g.K <= 4)
-    k_col_any<4><<<grid, threads, sm, st>>>(g, a, tw_y, psi, in, out, (int)nsc, (int)ntiles);
-  else
-    k_col_any<8><<<grid, threads, sm, st>>>(g, a, tw_y, psi, in, out, (int)nsc, (int)ntiles);
-  return cudaGetLastError();
+  return launch_pdl(g.K <= 4 ? k_col_any<4> : k_col_any<8>, dim3(grid), threads, sm, st, g, a, tw_y, psi, in, out,
+                    (int)nsc, (int)ntiles);
 }
 
 template <int MODE, int MC>
@@ -460,8 +462,7 @@ static cudaError_t row_any_go(const Geom& g, const AnyRow& a, const float2* tw, 
   if (e != cudaSuccess) return e;
   const int threads = (g.K * a.rows * std::max(a.RI, a.RT) + 31) / 32 * 32;
   dim3 grid((g.ny + a.rows - 1) / a.rows, g.S);
-  k_row_any<MODE, MC><<<grid, threads, row_any_smem(g, a), st>>>(g, a, tw, maps, x, t, out);
-  return cudaGetLastError();
+  return launch_pdl(k_row_any<MODE, MC>, grid, threads, row_any_smem(g, a), st, g, a, tw, maps, x, t, out);
 }
 
 cudaError_t launch_row_any(const Geom& g, RowMode mode, int W, int trb, const float2* tw_z, const float2* maps,

@@ -10,6 +10,7 @@
 // (a zero denominator gives a zero quotient), so an iteration needs no host round trip.
 #include <algorithm>
 
+#include "launch.h"
 #include "t2sh_device.cuh"
 
 namespace t2sh {
@@ -58,6 +59,8 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_init(long long L, const float
                                                        const float2* __restrict__ v, const float2* __restrict__ u,
                                                        float rho, float2* __restrict__ r, float2* __restrict__ p,
                                                        double* rr) {
+  pdl_wait();
+  pdl_trigger();
   const long long base = (long long)blockIdx.y * L;
   float4 xa[kCgPerThread], wa[kCgPerThread], ya[kCgPerThread], va[kCgPerThread], ua[kCgPerThread];
 #pragma unroll
@@ -89,6 +92,8 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_init(long long L, const float
 // pq[s] += Re <p, w + rho p>  (w = A^H A p)
 __global__ void __launch_bounds__(kCgThreads) k_cg_dot(long long L, const float2* __restrict__ p,
                                                       const float2* __restrict__ w, float rho, double* pq) {
+  pdl_wait();
+  pdl_trigger();
   const long long base = (long long)blockIdx.y * L;
   float4 pa[kCgPerThread], wa[kCgPerThread];
 #pragma unroll
@@ -113,6 +118,8 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_step(long long L, float2* __r
                                                        const float2* __restrict__ p, const float2* __restrict__ w,
                                                        float rho, const double* rr, const double* pq,
                                                        double* rr_new) {
+  pdl_wait();
+  pdl_trigger();
   const int s = blockIdx.y;
   const long long base = (long long)s * L;
   float4 pa[kCgPerThread], wa[kCgPerThread], xa[kCgPerThread], ra[kCgPerThread];
@@ -151,6 +158,8 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_step(long long L, float2* __r
 __global__ void __launch_bounds__(kCgThreads) k_cg_dir(long long L, const float2* __restrict__ r,
                                                       float2* __restrict__ p, const double* rr, const double* rr_new,
                                                       double* pq, double* rr_next) {
+  pdl_wait();
+  pdl_trigger();
   const int s = blockIdx.y;
   const long long base = (long long)s * L;
   float4 ra[kCgPerThread], pa[kCgPerThread];
@@ -210,21 +219,18 @@ dim3 cg_grid(const Geom& g, long long L) {
 cudaError_t launch_cg_init(const Geom& g, const float2* x, const float2* w, const float2* aty, const float2* v,
                            const float2* u, float rho, float2* r, float2* p, double* rr, cudaStream_t st) {
   const long long L = (long long)g.M * g.K * g.ny * g.nz;
-  k_cg_init<<<cg_grid(g, L), kCgThreads, 0, st>>>(L, x, w, aty, v, u, rho, r, p, rr);
-  return cudaGetLastError();
+  return launch_pdl(k_cg_init, cg_grid(g, L), kCgThreads, 0, st, L, x, w, aty, v, u, rho, r, p, rr);
 }
 
 cudaError_t launch_cg_dot(const Geom& g, const float2* p, const float2* w, float rho, double* pq, cudaStream_t st) {
   const long long L = (long long)g.M * g.K * g.ny * g.nz;
-  k_cg_dot<<<cg_grid(g, L), kCgThreads, 0, st>>>(L, p, w, rho, pq);
-  return cudaGetLastError();
+  return launch_pdl(k_cg_dot, cg_grid(g, L), kCgThreads, 0, st, L, p, w, rho, pq);
 }
 
 cudaError_t launch_cg_step(const Geom& g, float2* x, float2* r, const float2* p, const float2* w, float rho,
                            const double* rr, const double* pq, double* rr_new, cudaStream_t st) {
   const long long L = (long long)g.M * g.K * g.ny * g.nz;
-  k_cg_step<<<cg_grid(g, L), kCgThreads, 0, st>>>(L, x, r, p, w, rho, rr, pq, rr_new);
-  return cudaGetLastError();
+  return launch_pdl(k_cg_step, cg_grid(g, L), kCgThreads, 0, st, L, x, r, p, w, rho, rr, pq, rr_new);
 }
 
 cudaError_t launch_masked_energy(const Geom& g, const unsigned* bits, const float2* y, double* out, cudaStream_t st) {
@@ -237,8 +243,7 @@ cudaError_t launch_masked_energy(const Geom& g, const unsigned* bits, const floa
 cudaError_t launch_cg_dir(const Geom& g, const float2* r, float2* p, const double* rr, const double* rr_new,
                           double* pq, double* rr_next, cudaStream_t st) {
   const long long L = (long long)g.M * g.K * g.ny * g.nz;
-  k_cg_dir<<<cg_grid(g, L), kCgThreads, 0, st>>>(L, r, p, rr, rr_new, pq, rr_next);
-  return cudaGetLastError();
+  return launch_pdl(k_cg_dir, cg_grid(g, L), kCgThreads, 0, st, L, r, p, rr, rr_new, pq, rr_next);
 }
 
 }  // namespace t2sh

@@ -35,6 +35,7 @@
 // packed two-lane complex additions: 1.77 -> 1.75 ms at 256 points, 1.94 -> 1.86 ms at 260
 #define T2SH_PACKED_ADD 1
 
+#include "launch.h"
 #include "t2sh_device.cuh"
 
 // length, RA, RB: even products of 2, 3, 5 and 13 from 48 to 320 that are two radices of at most 20
@@ -185,7 +186,8 @@ __global__ void __launch_bounds__(Il<N>::THREADS, 1)
     const int end = min(hi, (zt + 1) * nsc);
     const int first = seg + grp;
     __syncthreads();  // the barriers are set up, and nobody reads the previous columns' Psi any more
-    if (gt == 0 && first < end && !dead) {
+    const bool start = seg == lo;  // the first columns' Psi (the plan's) is copied before t is touched
+    if (!start && gt == 0 && first < end && !dead) {
       request(first, zt);
       pending = true;
     }
@@ -199,6 +201,14 @@ __global__ void __launch_bounds__(Il<N>::THREADS, 1)
       pso[pos * 8 + 4 + w] = make_float4(pp[7 * NN], pp[8 * NN], pp[9 * NN], 0.f);
       psx[pos * 8 + w] = make_float4(p02, p03, p12, p13);
       psx[pos * 8 + 4 + w] = make_float4(p02, p12, p03, p13);
+    }
+    if (start) {
+      pdl_wait();
+      pdl_trigger();
+      if (gt == 0 && first < end) {
+        request(first, zt);
+        pending = true;
+      }
     }
     __syncthreads();
     for (int tile = first; tile < end; tile += ngroups) {
@@ -320,6 +330,8 @@ __global__ void __launch_bounds__(Il<N>::THREADS, 1)
   for (int i = threadIdx.x; i < N; i += blockDim.x) tws[i] = tw_g[(i / RA) * (i % RA)];
   const float2* tw = tws + it.j;
   __syncthreads();
+  pdl_wait();
+  pdl_trigger();
   // tiles in slice-and-coil-major order: neighbouring groups read neighbouring columns
   const int ntz = nz / 4;
   const long long step = (long long)gridDim.x * ngroups;
@@ -398,6 +410,8 @@ __global__ void __launch_bounds__(Il<N>::THREADS, 1)
   for (int i = threadIdx.x; i < N; i += blockDim.x) tws[i] = tw_g[(i / RA) * (i % RA)];
   const float2* tw = tws + it.j;
   __syncthreads();
+  pdl_wait();
+  pdl_trigger();
   const int ntz = nz / 4;
   const float scale0 = g.gsign * g.inv_sqrt_n * parity_sign(it.j + it.w);  // of frequency k1; 4 zt is even
   const long long step = (long long)gridDim.x * ngroups;
@@ -503,8 +517,7 @@ cudaError_t il_normal(const Geom& g, const float2* tw, const float* psi, float2*
   if (e != cudaSuccess) return e;
   const int ng = il_groups<N>(ntiles, nsm);
   const int grid = (int)std::min<long long>(nsm, (ntiles + ng - 1) / ng);
-  k_col_il<N><<<grid, ng * L::GT, L::smem(ng), st>>>(g, tm, tw, psi, t, (int)nsc, (int)ntiles, ng);
-  return cudaGetLastError();
+  return launch_pdl(k_col_il<N>, dim3(grid), ng * L::GT, L::smem(ng), st, g, tm, tw, psi, t, (int)nsc, (int)ntiles, ng);
 }
 
 template <int N, bool IN_IL>
@@ -517,8 +530,7 @@ cudaError_t il_adj(const Geom& g, const float2* tw, const float2* in, float2* t,
   if (e != cudaSuccess) return e;
   const int ng = il_groups<N>(ntiles, nsm);
   const int grid = (int)std::min<long long>(nsm, (ntiles + ng - 1) / ng);
-  k_col_il_adj<N, IN_IL><<<grid, ng * L::GT, L::smem_adj(ng), st>>>(g, tw, in, t, ntiles, ng);
-  return cudaGetLastError();
+  return launch_pdl(k_col_il_adj<N, IN_IL>, dim3(grid), ng * L::GT, L::smem_adj(ng), st, g, tw, in, t, ntiles, ng);
 }
 
 template <int N, bool PROJ>
@@ -531,8 +543,7 @@ cudaError_t il_fwd(const Geom& g, const float2* tw, const float* psi, const floa
   if (e != cudaSuccess) return e;
   const int ng = il_groups<N>(ntiles, nsm);
   const int grid = (int)std::min<long long>(nsm, (ntiles + ng - 1) / ng);
-  k_col_il_fwd<N, PROJ><<<grid, ng * L::GT, L::smem_adj(ng), st>>>(g, tw, psi, t, out, ntiles, ng);
-  return cudaGetLastError();
+  return launch_pdl(k_col_il_fwd<N, PROJ>, dim3(grid), ng * L::GT, L::smem_adj(ng), st, g, tw, psi, t, out, ntiles, ng);
 }
 
 template <int N>

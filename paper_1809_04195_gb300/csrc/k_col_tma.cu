@@ -23,6 +23,7 @@
 #include <algorithm>
 #include <mutex>
 
+#include "launch.h"
 #include "t2sh_device.cuh"
 
 namespace t2sh {
@@ -91,6 +92,8 @@ __global__ void __launch_bounds__(ColTma<N, W>::THREADS, ColTma<N, W>::MINB) k_c
   }
   for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = tw_g[i];
   __syncthreads();
+  pdl_wait();
+  pdl_trigger();
   int tile = blockIdx.x;
   if (threadIdx.x == 0 && tile < ntiles) {
     const int sc = tile / ntz, z0 = (tile - sc * ntz) * W;
@@ -258,6 +261,8 @@ __global__ void __launch_bounds__(ColTma<N, W>::THREADS, ColTma<N, W>::MINB) k_c
   }
   for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = tw_g[i];
   __syncthreads();
+  pdl_wait();
+  pdl_trigger();
   int tile = blockIdx.x;
   if (threadIdx.x == 0 && tile < ntiles) {
     const int sc = tile / ntz, z0 = (tile - sc * ntz) * W;
@@ -387,8 +392,7 @@ cudaError_t col_tma_go(const Geom& g, const float2* tw, const float* psi, float2
   const long long ntiles = (long long)g.S * g.C * ntz;
   if (ntiles > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int grid = (int)std::min<long long>(ntiles, (long long)nsm * CT::MINB);
-  k_col_tma<N, W><<<grid, CT::THREADS, sm, st>>>(g, tm_t, tm_psi, tw, t, ntz, (int)ntiles);
-  return cudaGetLastError();
+  return launch_pdl(k_col_tma<N, W>, dim3(grid), CT::THREADS, sm, st, g, tm_t, tm_psi, tw, t, ntz, (int)ntiles);
 }
 
 template <int W>
@@ -427,8 +431,7 @@ cudaError_t col_tma_adj_go(const Geom& g, const float2* tw, const float2* tin, f
   if (ntiles > 0x7fffffffLL) return cudaErrorInvalidValue;
   if (ntiles == 0) return cudaSuccess;
   const int grid = (int)std::min<long long>(ntiles, (long long)nsm * CT::MINB);
-  k_col_tma_adj<N, W><<<grid, CT::THREADS, sm, st>>>(g, tm_in, tw, tout, ntz, (int)ntiles);
-  return cudaGetLastError();
+  return launch_pdl(k_col_tma_adj<N, W>, dim3(grid), CT::THREADS, sm, st, g, tm_in, tw, tout, ntz, (int)ntiles);
 }
 
 }  // namespace

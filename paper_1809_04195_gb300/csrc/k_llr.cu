@@ -17,6 +17,7 @@
 // shape: its two CTAs per SM hide less memory latency than three single-buffer CTAs.)
 #include <algorithm>
 
+#include "launch.h"
 #include "t2sh_device.cuh"
 
 namespace t2sh {
@@ -304,6 +305,8 @@ template <int KC, int MODE, typename ET, int NT>
 __device__ __forceinline__ void llr_band(const Geom& g, const FistaArgs& a, int unit, float2* x, float2* z,
                                          const float2* __restrict__ grad, const float2* __restrict__ aty, float2* u) {
   extern __shared__ float2 smem[];
+  pdl_wait();
+  pdl_trigger();
   const LlrUnit un = llr_unit(g, a.b, unit);
   const int nbz = (g.nz + a.b - 1) / a.b;
   float2* gs = smem;                                         // [K][rb][llr_ld(nz)]
@@ -349,8 +352,7 @@ cudaError_t llr_launch(const Geom& g, const FistaArgs& a, size_t sm, float2* x, 
     if (e != cudaSuccess) return e;
   }
   dim3 grid((g.ny + a.b - 1) / a.b, g.S, g.M);
-  k_llr<KC, MODE, ET, MINB, NT><<<grid, NT, sm, st>>>(g, a, x, z, grad, aty, u);
-  return cudaGetLastError();
+  return launch_pdl(k_llr<KC, MODE, ET, MINB, NT>, grid, NT, sm, st, g, a, x, z, grad, aty, u);
 }
 
 // CTAs per SM whose shared memory (plus the 1 KB each reserves) fits in 228 KB

@@ -1,5 +1,6 @@
 // Plan-time kernels: coil-map preparation, the space-time kernel Psi (Sec. IV.B) and
 // the projection of per-echo k-space onto the basis (re-sort and project, Sec. III.A).
+#include "launch.h"
 #include "t2sh_device.cuh"
 
 namespace t2sh {
@@ -206,6 +207,8 @@ __global__ void __launch_bounds__(kThreads) k_project(Geom g, TLayout lt, const 
   extern __shared__ float sphi[];
   for (int i = threadIdx.x; i < g.T * g.K; i += blockDim.x) sphi[i] = phi[i];
   __syncthreads();
+  pdl_wait();
+  pdl_trigger();
   const int N = g.ny * g.nz;
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= N) return;
@@ -274,6 +277,8 @@ __global__ void __launch_bounds__(kThreads) k_expand_te(Geom g, TLayout lt, cons
   extern __shared__ float sphi[];
   for (int i = threadIdx.x; i < g.T * g.K; i += blockDim.x) sphi[i] = phi[i];
   __syncthreads();
+  pdl_wait();
+  pdl_trigger();
   const int N = g.ny * g.nz;
   const int n = 2 * (blockIdx.x * blockDim.x + threadIdx.x);  // nz is even: both points share a row
   if (n >= N) return;
@@ -340,8 +345,7 @@ static cudaError_t project_go(const Geom& g, const TLayout& lt, const float* phi
   const int N = g.ny * g.nz;
   const long long planes = ((long long)g.S * g.C + NP - 1) / NP;
   dim3 grid((N + kThreads - 1) / kThreads, (unsigned)(planes < 65535 ? planes : 65535));
-  k_project<KC, NP, NS><<<grid, kThreads, sizeof(float) * g.T * g.K, st>>>(g, lt, phi, bits, y, out);
-  return cudaGetLastError();
+  return launch_pdl(k_project<KC, NP, NS>, grid, kThreads, sizeof(float) * g.T * g.K, st, g, lt, phi, bits, y, out);
 }
 
 cudaError_t launch_project(const Geom& g, const TLayout& lt, const float* phi, const unsigned* bits, const float2* y_te,
@@ -366,9 +370,7 @@ cudaError_t launch_expand_te(const Geom& g, const TLayout& lt, const float* phi,
   const long long nsc = (long long)g.S * g.C;
   dim3 grid((N2 + kThreads - 1) / kThreads, (unsigned)(nsc < 65535 ? nsc : 65535));
   const size_t sm = sizeof(float) * g.T * g.K;
-  if (g.K <= 4) k_expand_te<4><<<grid, kThreads, sm, st>>>(g, lt, phi, bits, v, y_te);
-  else k_expand_te<8><<<grid, kThreads, sm, st>>>(g, lt, phi, bits, v, y_te);
-  return cudaGetLastError();
+  return launch_pdl(g.K <= 4 ? k_expand_te<4> : k_expand_te<8>, grid, kThreads, sm, st, g, lt, phi, bits, v, y_te);
 }
 
 }  // namespace t2sh

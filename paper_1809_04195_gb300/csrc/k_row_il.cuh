@@ -26,6 +26,7 @@
 
 // packed two-lane complex additions in the butterflies: fewer issue slots
 #define T2SH_PACKED_ADD 1
+#include "launch.h"
 #include "t2sh_device.cuh"
 
 namespace t2sh {
@@ -92,7 +93,7 @@ __global__ void __launch_bounds__(RowIl<N, RI, RT, MODE, MC>::THREADS, RowIl<N, 
       if (row < rb) cp_async16(md + line * N + col, mp + (long long)m * NN + row * N + col);
     }
   };
-  issue(0, 0);
+  issue(0, 0);  // the plan's maps: not written by any kernel of the solve
   cp_async_commit();
 
   // t-side address of coil 0: row, slot and the thread's column within its line of t
@@ -104,6 +105,8 @@ __global__ void __launch_bounds__(RowIl<N, RI, RT, MODE, MC>::THREADS, RowIl<N, 
   float2* ext = ex + ((in_t ? rt : 0) * 4 + k) * LINE;
   const long long img = (long long)s * MC * 4 * NN + (long long)k * NN + (long long)(y0 + ri) * N + ji;
 
+  pdl_wait();
+  pdl_trigger();
   if constexpr (MODE == ROW_FWD) {
     float2 xr[MC][RI];
 #pragma unroll
@@ -207,8 +210,7 @@ cudaError_t row_il_go(const Geom& g, int trb, const float2* tw, const float2* ma
   const cudaError_t e = smem_optin((const void*)k_row_il<N, RI, RT, MODE, MC>, (int)R::smem);
   if (e != cudaSuccess) return e;
   dim3 grid((g.ny + R::RB - 1) / R::RB, g.S);
-  k_row_il<N, RI, RT, MODE, MC><<<grid, R::THREADS, R::smem, st>>>(g, trb, tw, maps, x, t, out);
-  return cudaGetLastError();
+  return launch_pdl(k_row_il<N, RI, RT, MODE, MC>, grid, R::THREADS, R::smem, st, g, trb, tw, maps, x, t, out);
 }
 
 }  // namespace

@@ -1,0 +1,30 @@
+// Kernel launches that may start before the previous kernel of the stream has ended (programmatic
+// stream serialisation).  The kernel runs its prologue (tables, barriers, plan-owned constants) and
+// then pdl_wait(), after which the previous kernels' results are visible; pdl_trigger() lets the next
+// such kernel do the same.  A kernel triggers only after its own wait, so whatever ran before the
+// previous kernel has completed when a prologue runs.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace t2sh {
+
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+}  // namespace t2sh
