@@ -5,8 +5,8 @@
 // Work unit = (slice, map set, band of b shifted rows); the blocks of different map sets
 // are independent.  Per unit: gather the band into shared memory; per block (b x b
 // pixels x K) a warp forms the K x K Gram matrix G = X^H X with shuffle reductions; one
-// thread per block eigendecomposes G = V diag(lambda) V^H (cyclic Jacobi, float32 by
-// default, float64 on request), sigma_i = sqrt(lambda_i), and forms
+// thread per block eigendecomposes G = V diag(lambda) V^H (float32 by default: a real
+// tridiagonal form and real Jacobi for K <= 4; float64 on request), sigma_i = sqrt(lambda_i), and forms
 // W = V diag(max(1 - tau/sigma_i, 0)) V^H, so that X W = U max(Sigma - tau, 0) V^H
 // (since X V = U Sigma); then X' = X W is written back.  The FISTA variant fuses the
 // gradient step before the prox and the momentum update after it (Sec. II.A); the ADMM
