@@ -19,7 +19,7 @@
 //
 // Bound by instruction issue and HBM together.  Knee scan (320 slices of 256x160, C = 12, 10.1 GB
 // per launch): 2.52 -> 1.75 ms against the 8-column planar tiles of k_col_tma.cu, 0.85 of the
-// measured copy bandwidth; 260-point columns of Table I (8.05 GB): 2.51 -> 1.86 ms.  What it
+// measured copy bandwidth; 260-point columns of Table I (8.05 GB): 2.51 -> 1.72 ms.  What it
 // saves: the two exchanges around Psi (a frequency's four images sit in two neighbouring lanes),
 // two of five barriers, and the barriers join 128 threads instead of 512, so the four groups of
 // an SM drift apart and hide each other's stalls.  Psi stays in shared memory for a whole run of
@@ -32,7 +32,7 @@
 
 #include <algorithm>
 
-// packed two-lane complex additions: 1.77 -> 1.75 ms at 256 points, 1.94 -> 1.86 ms at 260
+// packed two-lane complex additions: 1.77 -> 1.75 ms at 256 points, 1.94 -> 1.86 ms at 260 (before spare buffers)
 #define T2SH_PACKED_ADD 1
 
 #include "launch.h"
@@ -69,14 +69,20 @@ struct Il : IlRadix<N> {
   static constexpr int BOX = N <= 256 ? N : N / 2;    // rows of one tensor-map box
   static_assert(N % BOX == 0 && BOX <= 256, "whole boxes");
   static constexpr size_t psi_bytes = (size_t)N * 4 * 64;
-  static constexpr size_t smem(int groups) { return (size_t)groups * TILE + psi_bytes + N * 8 + 16 * 8; }
+  // `bufs` tile buffers, Psi of a tile's columns, roots of unity, a barrier and a tile number per buffer
+  static constexpr size_t smem(int bufs) { return (size_t)bufs * TILE + psi_bytes + N * 8 + 16 * 12; }
   static constexpr size_t smem_adj(int groups) { return (size_t)groups * TILE + N * 8; }
   // groups of a CTA, which share the Psi block of their columns: 512 threads at 128 registers,
   // or what fits in shared memory
-  static constexpr int GS = (int)((232448 - psi_bytes - N * 8 - 128) / TILE);
+  static constexpr int GS = (int)((232448 - psi_bytes - N * 8 - 192) / TILE);
   static constexpr int G = 512 / GT < GS ? 512 / GT : GS;
+  // Tile buffers: one per group, and up to as many spare ones where a CTA has fewer than four groups
+  // to hide a tile's way from memory.  260 points (three groups, one spare buffer; 288 slices of
+  // 260x240) 1.85 -> 1.72 ms; with four groups spare buffers gave nothing (192 points 0.232 and
+  // 0.237 ms, 256 points 1.71 and 1.73 ms).
+  static constexpr int NB = G >= 4 || GS <= G ? G : 2 * G < GS ? 2 * G : GS;
   static constexpr int THREADS = G * GT;
-  static_assert(G >= 1 && smem(G) <= 232448, "shared memory");
+  static_assert(G >= 1 && NB >= G && NB <= 16 && smem(NB) <= 232448, "shared memory");
   static constexpr int E = RA <= 16 ? 2 : 1;  // basis images held in registers while the next tile is requested
   static constexpr bool FULL = 8 * RA == GT;  // every thread has an item in stage B
 };
@@ -87,6 +93,15 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const void* tmap, unsigne
           "r"(smem_u32(dst)),
       "l"(tmap), "r"(smem_u32(bar)), "r"(x), "r"(y)
       : "memory");
+}
+
+// wait until *seq has reached `tile`; false if it has not within the bounded wait
+__device__ __forceinline__ bool seq_wait_bounded(const volatile int* seq, int tile) {
+  if (*seq >= tile) return true;
+  const unsigned long long t0 = global_ns();
+  while (*seq < tile)
+    if (global_ns() - t0 > kWaitNs) return false;
+  return true;
 }
 
 // barrier among the GT threads of group `grp`
@@ -128,11 +143,15 @@ __device__ __forceinline__ void il_store(float2 (&c)[NK][RA], int i0, float2* gp
 
 // Normal-operator column pass, in place on t.  CTAs walk contiguous runs of the (column tile,
 // slice x coil) list in column-tile-major order: Psi of four columns stays in shared memory for
-// all slices and coils of the run.
+// all slices and coils of the run.  Tile p of a run belongs to group p mod ngroups and lands in
+// buffer p mod nbuf; the group that has read tile p requests tile p + nbuf into its buffer.  So with
+// spare buffers a tile is on its way while the group that will take it still works on its last one.
+// seq[b] is the tile last requested into buffer b: a group looks there before it waits for the
+// buffer's barrier, whose phase alone would not tell this tile from the one two visits earlier.
 template <int N>
 __global__ void __launch_bounds__(Il<N>::THREADS, 1)
     k_col_il(Geom g, const __grid_constant__ CUtensorMap tm, const float2* __restrict__ tw_g,
-             const float* __restrict__ psi, float2* t, int nsc, int ntiles, int ngroups) {
+             const float* __restrict__ psi, float2* t, int nsc, int ntiles, int ngroups, int nbuf) {
   using L = Il<N>;
   constexpr int RA = L::RA, RB = L::RB, GT = L::GT, E = L::E;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -140,15 +159,17 @@ __global__ void __launch_bounds__(Il<N>::THREADS, 1)
   unsigned char* buf = smem_raw + (size_t)grp * L::TILE;
   // Psi by point [k2][k1][kp][w]: the pair's own block (aa, ab, bb, -), and its block with the
   // other pair (ac, ad, bc, bd)
-  float4* pso = reinterpret_cast<float4*>(smem_raw + (size_t)ngroups * L::TILE);
+  float4* pso = reinterpret_cast<float4*>(smem_raw + (size_t)nbuf * L::TILE);
   float4* psx = pso + N * 8;
   float2* tws = reinterpret_cast<float2*>(psx + N * 8);  // [j][k1]: w_N^(j k1)
-  unsigned long long* bar = reinterpret_cast<unsigned long long*>(tws + N) + grp;
+  unsigned long long* bar = reinterpret_cast<unsigned long long*>(tws + N);
+  volatile int* seq = reinterpret_cast<volatile int*>(bar + 16);
   for (int i = threadIdx.x; i < N; i += blockDim.x) tws[i] = tw_g[(i / RA) * (i % RA)];
   const int nz = g.nz;
   const int rowlen = 4 * nz;
-  if (gt == 0) {
-    mbar_init(bar, 1);
+  if (threadIdx.x < nbuf) {
+    mbar_init(bar + threadIdx.x, 1);
+    seq[threadIdx.x] = -1;
     fence_mbar_init();
   }
   const IlItem it = il_item<N>(gt);
@@ -169,28 +190,25 @@ __global__ void __launch_bounds__(Il<N>::THREADS, 1)
   const float2* tw = tws + it.j;
   const int lo = (int)((long long)ntiles * blockIdx.x / gridDim.x),
             hi = (int)((long long)ntiles * (blockIdx.x + 1) / gridDim.x);
+  int b = grp;  // the group's next buffer
   unsigned phase = 0;
   bool dead = false;  // a bounded wait ran out: nothing is requested or waited for any more
-  bool pending = false;
 
-  auto request = [&](int tile, int zt) {  // one thread: the group's next tile
-    const int sc = tile - zt * nsc;
-    mbar_expect_tx(bar, L::TILE);
+  auto request = [&](int tile, int buffer) {  // one thread
+    const int zt = tile / nsc, sc = tile - zt * nsc;
+    mbar_expect_tx(bar + buffer, L::TILE);
 #pragma unroll
     for (int h = 0; h < N / L::BOX; ++h)
-      tma_load_2d(buf + h * L::BOX * 128, &tm, bar, zt * 16, sc * N + h * L::BOX);
+      tma_load_2d(smem_raw + (size_t)buffer * L::TILE + h * L::BOX * 128, &tm, bar + buffer, zt * 16, sc * N + h * L::BOX);
+    __threadfence_block();
+    seq[buffer] = tile;
   };
 
+  int tile = lo + grp;
   for (int seg = lo; seg < hi;) {
     const int zt = seg / nsc;
     const int end = min(hi, (zt + 1) * nsc);
-    const int first = seg + grp;
     __syncthreads();  // the barriers are set up, and nobody reads the previous columns' Psi any more
-    const bool start = seg == lo;  // the first columns' Psi (the plan's) is copied before t is touched
-    if (!start && gt == 0 && first < end && !dead) {
-      request(first, zt);
-      pending = true;
-    }
     for (int e = threadIdx.x; e < N * 4; e += blockDim.x) {
       const int w = e & 3, pos = e >> 2, k2 = pos / RA, k1 = pos - k2 * RA;
       const float* pp = psi + (long long)(k1 + RA * k2) * nz + zt * 4 + w;
@@ -202,21 +220,18 @@ __global__ void __launch_bounds__(Il<N>::THREADS, 1)
       psx[pos * 8 + w] = make_float4(p02, p03, p12, p13);
       psx[pos * 8 + 4 + w] = make_float4(p02, p12, p03, p13);
     }
-    if (start) {
+    if (seg == lo) {  // the first columns' Psi (the plan's) is copied before t is touched
       pdl_wait();
       pdl_trigger();
-      if (gt == 0 && first < end) {
-        request(first, zt);
-        pending = true;
-      }
+      if (threadIdx.x == 0)
+        for (int i = 0; i < nbuf && lo + i < hi; ++i) request(lo + i, i);
     }
     __syncthreads();
-    for (int tile = first; tile < end; tile += ngroups) {
-      if (!dead && !mbar_wait_bounded(bar, phase)) {
+    for (; tile < end; tile += ngroups) {
+      if (!dead && !(seq_wait_bounded(seq + b, tile) && mbar_wait_bounded(bar + b, phase))) {
         dead = true;
         if (g.err) atomicExch(g.err, 1);
       }
-      phase ^= 1;
       if (wa) {
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
@@ -283,20 +298,26 @@ __global__ void __launch_bounds__(Il<N>::THREADS, 1)
         for (int q = 0; q < RA; ++q) c[k][q] = lds2(pa[(2 - E + k + q) & 3], q * RB * 128);
       fence_proxy_async_smem();
       group_sync<GT>(grp);  // the buffer is read: the next tile lands while this one is finished
-      const int nxt = tile + ngroups;
-      if (gt == 0) {
-        pending = false;
-        if (nxt < end && !dead) {
-          request(nxt, zt);
-          pending = true;
-        }
+      if (gt == 0 && tile + nbuf < hi && !dead) request(tile + nbuf, b);
+      int step = ngroups;
+      b += ngroups;
+      if (b >= nbuf) {
+        b -= nbuf;
+        step -= nbuf;
+        phase ^= 1;
+      }
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        pa[m] += step * L::TILE;
+        pb[m] += step * L::TILE;
       }
       if (wa) il_store<RA, RB, E>(c, 2 - E, gp, gs, rowlen, on);
     }
     seg = end;
   }
   // copies in flight are given one more bounded wait before the CTA leaves
-  if (dead && pending) mbar_wait_bounded(bar, phase);
+  if (__syncthreads_or(dead) && threadIdx.x < nbuf && seq[threadIdx.x] >= 0)
+    mbar_wait_bounded(bar + threadIdx.x, ((seq[threadIdx.x] - lo) / nbuf) & 1);
 }
 
 // A^H y column pass: IDFT_y of the projected k-space column scaled by gsign (-1)^(ky + kz) /
@@ -512,12 +533,14 @@ cudaError_t il_normal(const Geom& g, const float2* tw, const float* psi, float2*
           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return cudaErrorNotSupported;
   int nsm = 0;
-  cudaError_t e = smem_optin((const void*)k_col_il<N>, (int)L::smem(L::G));
+  cudaError_t e = smem_optin((const void*)k_col_il<N>, (int)L::smem(L::NB));
   if (e == cudaSuccess) e = sm_count(&nsm);
   if (e != cudaSuccess) return e;
   const int ng = il_groups<N>(ntiles, nsm);
   const int grid = (int)std::min<long long>(nsm, (ntiles + ng - 1) / ng);
-  return launch_pdl(k_col_il<N>, dim3(grid), ng * L::GT, L::smem(ng), st, g, tm, tw, psi, t, (int)nsc, (int)ntiles, ng);
+  const int nbuf = (int)std::max<long long>(ng, std::min<long long>(L::NB, (ntiles + grid - 1) / grid));
+  return launch_pdl(k_col_il<N>, dim3(grid), ng * L::GT, L::smem(nbuf), st, g, tm, tw, psi, t, (int)nsc, (int)ntiles, ng,
+                    nbuf);
 }
 
 template <int N, bool IN_IL>

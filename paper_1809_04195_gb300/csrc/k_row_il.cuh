@@ -17,7 +17,10 @@
 //
 // Bound by HBM (maps and t once each, image rows once).  Knee scan (320 slices of 256x160, C = 12,
 // 6.71 GB per launch): forward 1.11 -> 0.99 ms, adjoint 1.15 -> 1.01 ms against the planar passes,
-// 0.98 of the measured copy bandwidth; Table I (M = 2, 7.19 GB): 1.39 -> 1.04 and 1.48 -> 1.22 ms.
+// 0.98 of the measured copy bandwidth; Table I (M = 2, 7.19 GB): 1.39 -> 1.04 and 1.48 -> 1.27 ms.
+// The adjoint's loads in flight wait in L1, so the SM's split is set to what the resident CTAs'
+// shared memory needs: after a column pass that leaves 28 KB of L1, 1.59 ms (M = 2, 240 points)
+// against 1.27, 1.28 against 1.05 (160 points).
 // Reading t with half-warps of one image (four lines per load instead of one) took 1.43 ms, and
 // storing it as runs of R1 columns (partial sectors) 1.30 ms.
 #pragma once
@@ -207,7 +210,8 @@ template <int N, int RI, int RT, int MODE, int MC>
 cudaError_t row_il_go(const Geom& g, int trb, const float2* tw, const float2* maps, const float2* x, float2* t,
                       float2* out, cudaStream_t st) {
   using R = RowIl<N, RI, RT, MODE, MC>;
-  const cudaError_t e = smem_optin((const void*)k_row_il<N, RI, RT, MODE, MC>, (int)R::smem);
+  const cudaError_t e = smem_optin((const void*)k_row_il<N, RI, RT, MODE, MC>, (int)R::smem,
+                                   R::MINB * ((int)R::smem + 1024));
   if (e != cudaSuccess) return e;
   dim3 grid((g.ny + R::RB - 1) / R::RB, g.S);
   return launch_pdl(k_row_il<N, RI, RT, MODE, MC>, grid, R::THREADS, R::smem, st, g, trb, tw, maps, x, t, out);

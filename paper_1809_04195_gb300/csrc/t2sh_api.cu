@@ -89,7 +89,7 @@ std::map<std::tuple<const void*, int, int, size_t>, int> g_per; // (kernel, devi
 
 namespace t2sh {
 
-cudaError_t smem_optin(const void* kernel, int bytes) {
+cudaError_t smem_optin(const void* kernel, int bytes, int sm_bytes) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -97,6 +97,9 @@ cudaError_t smem_optin(const void* kernel, int bytes) {
   auto it = g_optin.find({kernel, dev});
   if (it != g_optin.end() && it->second >= bytes) return cudaSuccess;
   e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess && sm_bytes > 0)
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                             std::min(100, (sm_bytes * 25 + 58367) / 58368));  // percent of 228 KB, rounded up
   if (e == cudaSuccess) g_optin[{kernel, dev}] = bytes;
   return e;
 }

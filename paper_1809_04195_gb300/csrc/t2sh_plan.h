@@ -214,10 +214,11 @@ cudaError_t launch_band_fused(const Geom& g, const FistaArgs& a, const float2* t
 cudaMemPool_t library_pool();
 
 // Per-device launch set-up shared by the launchers (a process may drive several GPUs):
-// a kernel's dynamic shared-memory limit is raised once per (kernel, device), and the
-// SM count and a kernel's resident CTAs per SM are cached per device.  All act on the
+// a kernel's dynamic shared-memory limit is raised once per (kernel, device), with sm_bytes
+// also the split of an SM's 256 KB set to leave all but that to L1 (the launch after one with
+// large shared memory otherwise keeps its split), and the SM count and a kernel's resident CTAs per SM are cached per device.  All act on the
 // current device.
-cudaError_t smem_optin(const void* kernel, int bytes);
+cudaError_t smem_optin(const void* kernel, int bytes, int sm_bytes = 0);
 cudaError_t sm_count(int* n);
 cudaError_t ctas_per_sm(const void* kernel, int threads, size_t smem, int* per);
 

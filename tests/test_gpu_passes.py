@@ -23,6 +23,9 @@ LENGTHS = [
     (1, 240, 64, 5, 1),
     (9, 256, 128, 4, 1),
     (5, 260, 240, 6, 1),     # two tensor-map boxes per column
+    (20, 260, 64, 12, 1),    # three groups and a spare tile buffer that goes round several times
+    (16, 300, 60, 11, 1),    # runs that cross column tiles there
+    (21, 234, 52, 7, 2),
 ]
 
 
