@@ -65,9 +65,36 @@ struct RowIl {
   static constexpr size_t smem = sizeof(float2) * ((size_t)N + 4 * RB * LINE + 2 * (size_t)MC * RB * N);
 };
 
+// barrier among all threads of the cluster, shared-memory writes before it visible after it
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// *p in the shared memory of CTA `rank` of the cluster
+__device__ __forceinline__ float2 cluster_lds2(const float2* p, int rank) {
+  unsigned a;
+  float2 v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+  return v;
+}
+
+// CTAs that share a band's coils: as many as keep the launch within one wave of resident CTAs, more
+// than four only within half a wave, and at most eight, the portable size of the cluster in which the
+// adjoint sums over the coils.  One slice of 64 x 48, C = 8: forward 4.6 -> 2.3 us, adjoint 5.6 -> 4.2,
+// a 50-iteration solve 1.22 -> 1.11 ms (1.14 with four CTAs); two slices with M = 2: 1.26 ms with four,
+// 1.35 with eight.  Beyond one wave the sum costs the adjoint more than a fuller last wave gives (32
+// slices of 192 x 192: 148 -> 167 us with a split by waves).
+inline int row_split(long long ctas, long long resident, int C) {
+  for (int n = std::min(8, C); n > 1; --n) {
+    const int cs = (C + n - 1) / n;
+    if ((C + cs - 1) / cs == n && ctas * n <= (n > 4 ? resident / 2 : resident)) return n;  // every CTA has a coil
+  }
+  return 1;
+}
+
 template <int N, int RI, int RT, int MODE, int MC>
 __global__ void __launch_bounds__(RowIl<N, RI, RT, MODE, MC>::THREADS, RowIl<N, RI, RT, MODE, MC>::MINB)
-    k_row_il(Geom g, int trb, const float2* __restrict__ tw_g, const float2* __restrict__ maps,
+    k_row_il(Geom g, int trb, int cs, const float2* __restrict__ tw_g, const float2* __restrict__ maps,
              const float2* __restrict__ x, float2* __restrict__ t, float2* __restrict__ out) {
   using R = RowIl<N, RI, RT, MODE, MC>;
   constexpr int LINE = R::LINE, S = R::S, RB = R::RB;
@@ -75,6 +102,7 @@ __global__ void __launch_bounds__(RowIl<N, RI, RT, MODE, MC>::THREADS, RowIl<N, 
   const int NN = g.ny * N;
   const int s = blockIdx.y, y0 = blockIdx.x * RB;
   const int rb = min(RB, g.ny - y0);
+  const int c0 = blockIdx.z * cs, c1 = min(g.C, c0 + cs);  // this CTA's coils
   // basis image k, item i of the band: t-side items (jt < RI, row rt), image-side items (ji < RT, row ri)
   const int k = threadIdx.x & 3, i = threadIdx.x >> 2;
   const int rt = i / RI, jt = i - rt * RI;
@@ -96,13 +124,13 @@ __global__ void __launch_bounds__(RowIl<N, RI, RT, MODE, MC>::THREADS, RowIl<N, 
       if (row < rb) cp_async16(md + line * N + col, mp + (long long)m * NN + row * N + col);
     }
   };
-  issue(0, 0);  // the plan's maps: not written by any kernel of the solve
+  issue(c0, 0);  // the plan's maps: not written by any kernel of the solve
   cp_async_commit();
 
-  // t-side address of coil 0: row, slot and the thread's column within its line of t
+  // t-side address of coil c0: row, slot and the thread's column within its line of t
   const int yt = y0 + (in_t ? rt : 0);
   const int slot = trb ? (k + yt % trb + yt / trb) & 3 : k;
-  float2* tp = t + ((long long)s * g.C * g.ny + yt) * (4 * N) + slot * 4 + (jt >> 2) * 16 + (jt & 3);
+  float2* tp = t + ((long long)(s * g.C + c0) * g.ny + yt) * (4 * N) + slot * 4 + (jt >> 2) * 16 + (jt & 3);
   const long long tcoil = 4LL * NN;
   const float2* exi = ex + ((ri < RB ? ri : 0) * 4 + k) * LINE;
   float2* ext = ex + ((in_t ? rt : 0) * 4 + k) * LINE;
@@ -118,11 +146,11 @@ __global__ void __launch_bounds__(RowIl<N, RI, RT, MODE, MC>::THREADS, RowIl<N, 
       for (int q = 0; q < RI; ++q)
         xr[m][q] = on_i ? x[img + (long long)m * 4 * NN + RT * q] : make_float2(0.f, 0.f);
     float2* exw = const_cast<float2*>(exi) + ji * S;
-    for (int c = 0; c < g.C; ++c) {
-      const int buf = c & 1;
+    for (int c = c0; c < c1; ++c) {
+      const int buf = (c - c0) & 1;
       cp_async_wait<0>();
       __syncthreads();  // coil c's maps are here, and nobody is in the previous coil any more
-      if (c + 1 < g.C) issue(c + 1, buf ^ 1);
+      if (c + 1 < c1) issue(c + 1, buf ^ 1);
       cp_async_commit();
       if (ri < RB) {
         const float2* mrow = mst + (buf * MC * RB + ri) * N + ji;
@@ -162,17 +190,17 @@ __global__ void __launch_bounds__(RowIl<N, RI, RT, MODE, MC>::THREADS, RowIl<N, 
     float2 tn[RT];
 #pragma unroll
     for (int q = 0; q < RT; ++q) tn[q] = on_t ? tp[q * (4 * RI)] : make_float2(0.f, 0.f);
-    for (int c = 0; c < g.C; ++c) {
-      const int buf = c & 1;
+    for (int c = c0; c < c1; ++c) {
+      const int buf = (c - c0) & 1;
       cp_async_wait<0>();
       __syncthreads();  // coil c's maps are here, and nobody is in the previous coil any more
-      if (c + 1 < g.C) issue(c + 1, buf ^ 1);
+      if (c + 1 < c1) issue(c + 1, buf ^ 1);
       cp_async_commit();
       float2 a[RT];
 #pragma unroll
       for (int q = 0; q < RT; ++q) a[q] = tn[q];
       tp += tcoil;
-      if (c + 1 < g.C) {
+      if (c + 1 < c1) {
 #pragma unroll
         for (int q = 0; q < RT; ++q) tn[q] = on_t ? tp[q * (4 * RI)] : make_float2(0.f, 0.f);
       }
@@ -196,11 +224,38 @@ __global__ void __launch_bounds__(RowIl<N, RI, RT, MODE, MC>::THREADS, RowIl<N, 
           for (int q = 0; q < RI; ++q) cfmac(acc[m][q], mrow[m * RB * N + RT * q], b[q]);
       }
     }
-    if (on_i) {
+    if (gridDim.z == 1) {
+      if (on_i) {
 #pragma unroll
-      for (int m = 0; m < MC; ++m)
+        for (int m = 0; m < MC; ++m)
 #pragma unroll
-        for (int q = 0; q < RI; ++q) out[img + (long long)m * 4 * NN + RT * q] = acc[m][q];
+          for (int q = 0; q < RI; ++q) out[img + (long long)m * 4 * NN + RT * q] = acc[m][q];
+      }
+    } else {
+      // the cluster's CTAs hold the sums over their coils: each leaves its own in shared memory, in
+      // the order [map set][row][column][image], and adds up a share of all of them
+      static_assert(LINE >= N, "the sums fit in the exchange and the map rows");
+      cp_async_wait<0>();
+      __syncthreads();
+      if (ri < RB) {
+#pragma unroll
+        for (int m = 0; m < MC; ++m)
+#pragma unroll
+          for (int q = 0; q < RI; ++q) ex[((m * RB + ri) * N + ji + RT * q) * 4 + k] = acc[m][q];
+      }
+      cluster_sync();
+      const int ns = gridDim.z;
+      for (int e = blockIdx.z * R::THREADS + threadIdx.x; e < MC * RB * N * 4; e += ns * R::THREADS) {
+        float2 v = cluster_lds2(ex + e, 0);
+        for (int r = 1; r < ns; ++r) {
+          const float2 w = cluster_lds2(ex + e, r);
+          v.x += w.x;
+          v.y += w.y;
+        }
+        const int pos = (e >> 2) % N, row = (e >> 2) / N % RB, m = (e >> 2) / (N * RB);
+        if (row < rb) out[((long long)(s * MC + m) * 4 + (e & 3)) * NN + (long long)(y0 + row) * N + pos] = v;
+      }
+      cluster_sync();  // nobody leaves while its sums are read
     }
   }
   cp_async_wait<0>();
@@ -213,8 +268,14 @@ cudaError_t row_il_go(const Geom& g, int trb, const float2* tw, const float2* ma
   const cudaError_t e = smem_optin((const void*)k_row_il<N, RI, RT, MODE, MC>, (int)R::smem,
                                    R::MINB * ((int)R::smem + 1024));
   if (e != cudaSuccess) return e;
-  dim3 grid((g.ny + R::RB - 1) / R::RB, g.S);
-  return launch_pdl(k_row_il<N, RI, RT, MODE, MC>, grid, R::THREADS, R::smem, st, g, trb, tw, maps, x, t, out);
+  int nsm = 0;
+  const cudaError_t es = sm_count(&nsm);
+  if (es != cudaSuccess) return es;
+  const int nb = (g.ny + R::RB - 1) / R::RB;
+  const int ns = row_split((long long)nb * g.S, (long long)nsm * R::MINB, g.C);
+  const int cs = (g.C + ns - 1) / ns;
+  return launch_pdl_cluster(k_row_il<N, RI, RT, MODE, MC>, dim3(nb, g.S, ns), MODE == ROW_ADJ ? ns : 1, R::THREADS,
+                            R::smem, st, g, trb, cs, tw, maps, x, t, out);
 }
 
 }  // namespace

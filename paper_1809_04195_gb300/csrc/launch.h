@@ -9,19 +9,30 @@
 
 namespace t2sh {
 
+// cluster_z > 1: CTAs of a cluster are neighbours along the grid's z axis
 template <typename... P, typename... A>
-inline cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+inline cudaError_t launch_pdl_cluster(void (*kern)(P...), dim3 grid, int cluster_z, int threads, size_t smem,
+                                      cudaStream_t st, A... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  cudaLaunchAttribute at[2] = {};
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = 1;
+  at[1].val.clusterDim.y = 1;
+  at[1].val.clusterDim.z = (unsigned)cluster_z;
+  cfg.attrs = at;
+  cfg.numAttrs = cluster_z > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+  return launch_pdl_cluster(kern, grid, 1, threads, smem, st, args...);
 }
 
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

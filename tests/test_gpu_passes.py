@@ -26,6 +26,10 @@ LENGTHS = [
     (20, 260, 64, 12, 1),    # three groups and a spare tile buffer that goes round several times
     (16, 300, 60, 11, 1),    # runs that cross column tiles there
     (21, 234, 52, 7, 2),
+    (1, 60, 160, 7, 1),      # coils shared by up to eight CTAs
+    (1, 64, 64, 13, 2),
+    (3, 78, 240, 6, 2),
+    (2, 48, 192, 1, 1),      # one coil
 ]
 
 
