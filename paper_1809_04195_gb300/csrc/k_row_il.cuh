@@ -36,13 +36,30 @@ namespace t2sh {
 
 namespace {
 
-// length, RI, RT: multiples of four from 48 to 320 that are two radices of at most 20, RI a multiple
-// of four so that a half-warp's columns on the side of t are one aligned chunk
-#define T2SH_ROW_LENGTHS(X)                                                                                        \
-  X(48, 16, 3) X(52, 4, 13) X(60, 12, 5) X(64, 16, 4) X(72, 8, 9) X(80, 16, 5) X(96, 16, 6) X(100, 20, 5) X(104, 8, 13) \
-  X(108, 12, 9) X(120, 12, 10) X(128, 16, 8) X(144, 12, 12) X(156, 12, 13) X(160, 16, 10) X(180, 12, 15)               \
-  X(192, 16, 12) X(200, 20, 10) X(208, 16, 13) X(216, 12, 18) X(240, 16, 15) X(256, 16, 16) X(260, 20, 13)           \
-  X(288, 16, 18) X(300, 20, 15) X(320, 16, 20)
+// length, RI, RT, rows of a CTA: multiples of four from 48 to 320 that are two radices of at most 20,
+// RI a multiple of four so that a half-warp's columns on the side of t are one aligned chunk.  The
+// rows are four digits, forward and adjoint with one map set, then with two: each the fastest of one
+// to four at 60 slices of 128 x 192 points' worth of lines, C = 10.  One row where the items of both
+// sides fill their warps or the registers limit the CTAs, two or three where 4 RI or 4 RT leaves a warp
+// part empty: 144 points 5.8 -> 6.1 TB/s forward, 72 points 4.6 -> 6.0, 52 points 2.8 -> 4.9, 256 points
+// 6.0 with one row and with two.  Balanced radices for short lines, which use more threads of a warp
+// on the image side: 48 = 8 x 6 5.9 and 5.3 TB/s (forward, adjoint), 16 x 3 3.0 and 2.5; 64 = 8 x 8
+// 6.5 and 5.7, 16 x 4 3.8 and 3.2; 160 = 8 x 20 is slower than 16 x 10 (5.7 and 6.1).
+#define T2SH_ROW_LENGTHS(X) \
+  X(48, 8, 6, 1111) X(52, 4, 13, 2222) X(60, 12, 5, 2222) X(64, 8, 8, 2121) X(72, 8, 9, 2233)               \
+  X(80, 8, 10, 3233) X(96, 8, 12, 2222) X(100, 20, 5, 2211) X(104, 8, 13, 2222) X(108, 12, 9, 2222)         \
+  X(120, 12, 10, 2222) X(128, 16, 8, 1222) X(144, 12, 12, 2222) X(156, 12, 13, 2211) X(160, 16, 10, 1211)   \
+  X(180, 12, 15, 1111) X(192, 16, 12, 1111) X(200, 20, 10, 2212) X(208, 16, 13, 1111) X(216, 12, 18, 2222)  \
+  X(240, 16, 15, 1111) X(256, 16, 16, 1111) X(260, 20, 13, 2211) X(288, 16, 18, 2212) X(300, 20, 15, 2212)  \
+  X(320, 16, 20, 2211)
+
+constexpr int row_rows(int n, bool adj, int mc) {
+  int d = 1111;
+#define X(len, ri, rt, r) d = n == len ? r : d;
+  T2SH_ROW_LENGTHS(X)
+#undef X
+  return d / (mc == 1 ? (adj ? 100 : 1000) : (adj ? 1 : 10)) % 10;
+}
 
 template <int N, int RI_, int RT_, int MODE, int MC>
 struct RowIl {
@@ -53,13 +70,12 @@ struct RowIl {
   static constexpr int L0 = (MODE == ROW_FWD ? RT : RI) * S;
   static constexpr int LINE = L0 + ((4 - L0 % 16) + 16) % 16;
   static constexpr int J = RI > RT ? RI : RT;
-  // One-row bands where the items of the smaller side fill their warps or lines are short, two-row
-  // bands otherwise: adjoint at N = 160 1.02 ms with two rows, 1.09 with one (40
-  // items leave the second warp three quarters empty); forward with two map sets at N = 240
-  // 1.04 ms with one row, 1.09 with two.  MINB holds the registers to 80 (forward), 96 or 128.
-  static constexpr int RB = (MODE == ROW_FWD || N <= 64 || RT == 8 || RT >= 15) ? 1 : 2;
+  // MINB holds the registers to 80 (forward), 96 or 128; 144 for the adjoint of two map sets at radix
+  // 16 and more on both sides, which otherwise spills (288 points 4.2 -> 4.5 TB/s, 320 points 4.2 -> 5.0,
+  // 256 points 5.2 -> 5.4; 240 points 5.3 with 128 and 5.1 with 144).
+  static constexpr int RB = row_rows(N, MODE == ROW_ADJ, MC);
   static constexpr int THREADS = (4 * J * RB + 31) / 32 * 32;
-  static constexpr int REGS = MC == 2 ? (RI > 16 ? 168 : 128) : MODE == ROW_FWD ? (RI > 16 || RT > 16 ? 96 : 80)
+  static constexpr int REGS = MC == 2 ? (RI > 16 ? 168 : MODE == ROW_ADJ && RI == 16 && RT >= 16 ? 144 : 128) : MODE == ROW_FWD ? (RI > 16 || RT > 16 ? 96 : 80)
                                                                                : RT <= 10 && RI <= 16 ? 96 : 128;
   static constexpr int MINB = 65536 / (REGS * THREADS) > 0 ? 65536 / (REGS * THREADS) : 1;
   static constexpr size_t smem = sizeof(float2) * ((size_t)N + 4 * RB * LINE + 2 * (size_t)MC * RB * N);
@@ -286,7 +302,7 @@ cudaError_t row_il_go(const Geom& g, int trb, const float2* tw, const float2* ma
 cudaError_t T2SH_ROW_NAME(T2SH_ROW_MODE)(const Geom& g, int trb, const float2* tw, const float2* maps, const float2* x,
                                          float2* t, float2* out, cudaStream_t st) {
   switch (g.nz) {
-#define X(n, ri, rt)                                                                                     \
+#define X(n, ri, rt, r)                                                                                   \
   case n:                                                                                                \
     return g.M == 1 ? row_il_go<n, ri, rt, T2SH_ROW_MODE, 1>(g, trb, tw, maps, x, t, out, st)            \
                     : row_il_go<n, ri, rt, T2SH_ROW_MODE, 2>(g, trb, tw, maps, x, t, out, st);
@@ -303,7 +319,7 @@ cudaError_t launch_row_il_ROW_ADJ(const Geom& g, int trb, const float2* tw, cons
 bool row_il_supported(const Geom& g) {
   if (g.K != 4 || g.M > 2) return false;
   switch (g.nz) {
-#define X(n, ri, rt) case n:
+#define X(n, ri, rt, r) case n:
     T2SH_ROW_LENGTHS(X)
 #undef X
     return true;
