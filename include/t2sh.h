@@ -331,8 +331,8 @@ t2sh_status t2sh_batch_schedule(int32_t per_scan_llr);
 
 /*
  * t2sh_autotune -- choose, for the plan's problem shape, the column-pass variant
- * (0: tiles of 8 columns moved by TMA, 4: tiles of 4 by TMA, 1: tiles of 8 by cp.async,
- * 2: tiles of 4 by cp.async; a T2SH_MIXED_BF16 plan keeps its tensor-core column pass,
+ * (0: the default kernels of the shape; on the planar intermediate, 4: tiles of 4 columns
+ * by TMA, 1: tiles of 8 by cp.async, 2: tiles of 4 by cp.async; a T2SH_MIXED_BF16 plan keeps its tensor-core column pass,
  * variant 3) and
  * separate versus fused row kernels, by timing probe_iters
  * iterations (default 3 when <= 0) of each candidate on the plan's buffers; the choice

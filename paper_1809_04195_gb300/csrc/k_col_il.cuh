@@ -17,15 +17,18 @@
 // stay where stage B leaves them, and Psi is read in that order.  A tile has three barriers among
 // its own 64 ... 160 threads.
 //
-// Bound by instruction issue and HBM together.  Knee scan (320 slices of 256x160, C = 12, 10.1 GB
-// per launch): 2.52 -> 1.75 ms against the 8-column planar tiles of k_col_tma.cu, 0.85 of the
-// measured copy bandwidth; 260-point columns of Table I (8.05 GB): 2.51 -> 1.72 ms.  What it
-// saves: the two exchanges around Psi (a frequency's four images sit in two neighbouring lanes),
-// two of five barriers, and the barriers join 128 threads instead of 512, so the four groups of
-// an SM drift apart and hide each other's stalls.  Psi stays in shared memory for a whole run of
-// slices and coils instead of being copied per tile.  With all four images in one thread the code
-// outgrew the instruction cache (2.58 ms, a third of the stalls "no instruction"); five groups at
-// 96 registers took 1.91 ms.
+// Bound by shared-memory wavefronts (77 % of the L1 data pipe while active at 256 points), issue and HBM
+// together.  Knee scan (320 slices of 256x160, C = 12, 10.1 GB per launch): 2.52 -> 1.69 ms against the
+// 8-column planar tiles of k_col_tma.cu, 0.88 of the measured copy bandwidth; 260-point columns of
+// Table I (8.05 GB): 2.51 -> 1.72 ms.  What it saves: the two exchanges around Psi (a frequency's four
+// images sit in two neighbouring lanes), two of five barriers, and the barriers join 128 threads instead
+// of 512, so the four groups of an SM drift apart and hide each other's stalls.  Psi stays in shared
+// memory for a whole run of slices and coils instead of being copied per tile.  Where RB is even the two
+// lanes of a point take half of its frequencies each, which reads ten floats of Psi per point instead of
+// sixteen: 200 slices of 256x160 1.08 -> 1.06 ms, 60 slices of 288x96 0.28 -> 0.26, and of 320x96 0.39 ->
+// 0.30, where the shared memory that this frees holds a spare buffer.  With all four images in one thread the code outgrew the instruction cache (2.58 ms, a
+// third of the stalls "no instruction"); five groups at 96 registers took 1.91 ms at 256 points and
+// 0.26 instead of 0.17 at 192.
 #pragma once
 
 #include <cuda.h>
@@ -68,13 +71,17 @@ struct Il : IlRadix<N> {
   static constexpr int TILE = N * 128;                // bytes
   static constexpr int BOX = N <= 256 ? N : N / 2;    // rows of one tensor-map box
   static_assert(N % BOX == 0 && BOX <= 256, "whole boxes");
-  static constexpr size_t psi_bytes = (size_t)N * 4 * 64;
+  // an even RB: the two lanes of a point take half of the frequencies each in Psi (ten floats a point)
+  static constexpr bool HALF = RB % 2 == 0;
+  static constexpr size_t psi_bytes = (size_t)N * 4 * (HALF ? 40 : 64);
+  static constexpr int TWS = (N + 15) / 16 * 16 + 8;  // between the lanes' tables, half the banks apart
+  static constexpr int TW = HALF ? TWS + N : N;        // roots of unity
   // `bufs` tile buffers, Psi of a tile's columns, roots of unity, a barrier and a tile number per buffer
-  static constexpr size_t smem(int bufs) { return (size_t)bufs * TILE + psi_bytes + N * 8 + 16 * 12; }
+  static constexpr size_t smem(int bufs) { return (size_t)bufs * TILE + psi_bytes + TW * 8 + 16 * 12; }
   static constexpr size_t smem_adj(int groups) { return (size_t)groups * TILE + N * 8; }
   // groups of a CTA, which share the Psi block of their columns: 512 threads at 128 registers,
   // or what fits in shared memory
-  static constexpr int GS = (int)((232448 - psi_bytes - N * 8 - 192) / TILE);
+  static constexpr int GS = (int)((232448 - psi_bytes - TW * 8 - 192) / TILE);
   static constexpr int G = 512 / GT < GS ? 512 / GT : GS;
   // Tile buffers: one per group, and up to as many spare ones where a CTA has fewer than four groups
   // to hide a tile's way from memory.  260 points (three groups, one spare buffer; 288 slices of
@@ -113,6 +120,11 @@ __device__ __forceinline__ void group_sync(int grp) {
 
 __device__ __forceinline__ float2 lds2(const unsigned char* p, int off) { return *reinterpret_cast<const float2*>(p + off); }
 __device__ __forceinline__ void sts2(unsigned char* p, int off, float2 v) { *reinterpret_cast<float2*>(p + off) = v; }
+
+// the value in the neighbouring lane, which holds the other two basis images of the point
+__device__ __forceinline__ float2 shfl_xor2(float2 v) {
+  return make_float2(__shfl_xor_sync(0xffffffffu, v.x, 4), __shfl_xor_sync(0xffffffffu, v.y, 4));
+}
 
 // A thread's place in its group: column w, basis pair kp, item j
 struct IlItem {
@@ -157,14 +169,22 @@ __global__ void __launch_bounds__(Il<N>::THREADS, 1)
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const int grp = threadIdx.x / GT, gt = threadIdx.x - grp * GT;
   unsigned char* buf = smem_raw + (size_t)grp * L::TILE;
-  // Psi by point [k2][k1][kp][w]: the pair's own block (aa, ab, bb, -), and its block with the
-  // other pair (ac, ad, bc, bd)
+  // Psi by point.  HALF: [k2 mod RB / 2][k1][k2 div RB / 2][w], images a, b of the lane that takes the
+  // frequency and c, d of the other: (aa, ab, bb, ac), (ad, bc, bd, cc), (cd, dd).  Otherwise
+  // [k2][k1][kp][w]: the pair's own block (aa, ab, bb, -), and its block with the other pair (ac, ad, bc, bd)
+  constexpr int NP = L::HALF ? N * 4 : N * 8;
   float4* pso = reinterpret_cast<float4*>(smem_raw + (size_t)nbuf * L::TILE);
-  float4* psx = pso + N * 8;
-  float2* tws = reinterpret_cast<float2*>(psx + N * 8);  // [j][k1]: w_N^(j k1)
-  unsigned long long* bar = reinterpret_cast<unsigned long long*>(tws + N);
+  float4* psx = pso + NP;
+  float2* psz = reinterpret_cast<float2*>(psx + NP);  // HALF only
+  // [j][k1]: w_N^(j k1); HALF: [kp][j][k1], for kp = 1 times (-1)^j, which turns the frequencies by RB / 2
+  float2* tws = reinterpret_cast<float2*>(smem_raw + (size_t)nbuf * L::TILE + L::psi_bytes);
+  unsigned long long* bar = reinterpret_cast<unsigned long long*>(tws + L::TW);
   volatile int* seq = reinterpret_cast<volatile int*>(bar + 16);
-  for (int i = threadIdx.x; i < N; i += blockDim.x) tws[i] = tw_g[(i / RA) * (i % RA)];
+  for (int i = threadIdx.x; i < N; i += blockDim.x) {
+    const float2 v = tw_g[(i / RA) * (i % RA)];
+    tws[i] = v;
+    if (L::HALF) tws[L::TWS + i] = (i / RA) % 2 ? make_float2(-v.x, -v.y) : v;
+  }
   const int nz = g.nz;
   const int rowlen = 4 * nz;
   if (threadIdx.x < nbuf) {
@@ -187,7 +207,7 @@ __global__ void __launch_bounds__(Il<N>::THREADS, 1)
     pb[m] = buf + it.j * RB * 128 + ((m + 2 * it.kp + it.j) & 3) * 32 + it.w * 8;
     gs[m] = ((m + 2 * it.kp + ja) & 3) * 4;
   }
-  const float2* tw = tws + it.j;
+  const float2* tw = tws + (L::HALF ? it.kp * L::TWS : 0) + it.j;
   const int lo = (int)((long long)ntiles * blockIdx.x / gridDim.x),
             hi = (int)((long long)ntiles * (blockIdx.x + 1) / gridDim.x);
   int b = grp;  // the group's next buffer
@@ -215,10 +235,19 @@ __global__ void __launch_bounds__(Il<N>::THREADS, 1)
       const long long NN = (long long)N * nz;
       // upper triangle, row by row: 00 01 02 03 11 12 13 22 23 33
       const float p02 = pp[2 * NN], p03 = pp[3 * NN], p12 = pp[5 * NN], p13 = pp[6 * NN];
-      pso[pos * 8 + w] = make_float4(pp[0], pp[NN], pp[4 * NN], 0.f);
-      pso[pos * 8 + 4 + w] = make_float4(pp[7 * NN], pp[8 * NN], pp[9 * NN], 0.f);
-      psx[pos * 8 + w] = make_float4(p02, p03, p12, p13);
-      psx[pos * 8 + 4 + w] = make_float4(p02, p12, p03, p13);
+      if constexpr (L::HALF) {
+        const bool up = k2 >= RB / 2;  // the lane of images 2 and 3 takes it
+        const int e1 = ((k2 - (up ? RB / 2 : 0)) * RA + k1) * 8 + (up ? 4 : 0) + w;
+        const float p00 = pp[0], p01 = pp[NN], p11 = pp[4 * NN], p22 = pp[7 * NN], p23 = pp[8 * NN], p33 = pp[9 * NN];
+        pso[e1] = up ? make_float4(p22, p23, p33, p02) : make_float4(p00, p01, p11, p02);
+        psx[e1] = up ? make_float4(p12, p03, p13, p00) : make_float4(p03, p12, p13, p22);
+        psz[e1] = up ? make_float2(p01, p11) : make_float2(p23, p33);
+      } else {
+        pso[pos * 8 + w] = make_float4(pp[0], pp[NN], pp[4 * NN], 0.f);
+        pso[pos * 8 + 4 + w] = make_float4(pp[7 * NN], pp[8 * NN], pp[9 * NN], 0.f);
+        psx[pos * 8 + w] = make_float4(p02, p03, p12, p13);
+        psx[pos * 8 + 4 + w] = make_float4(p02, p12, p03, p13);
+      }
     }
     if (seg == lo) {  // the first columns' Psi (the plan's) is copied before t is touched
       pdl_wait();
@@ -256,20 +285,44 @@ __global__ void __launch_bounds__(Il<N>::THREADS, 1)
           for (int j = 1; j < RB; ++j) b[k][j] = twiddle_mul<false>(b[k][j], tw[j * RA]);
           dft_r<RB, false>(b[k]);
         }
+        if constexpr (L::HALF) {
+          // register r holds frequency k2 = r in the lane of images 0 and 1 and r + RB / 2 (mod RB) in that of
+          // 2 and 3, so each lane takes the frequencies of its lower registers, with the other lane's upper ones
+          constexpr int H = RB / 2;
 #pragma unroll
-        for (int k2 = 0; k2 < RB; ++k2) {
-          const int e = (k2 * RA + it.j) * 8 + it.kp * 4 + it.w;
-          const float4 po = pso[e], px = psx[e];
-          const float2 va = b[0][k2], vb = b[1][k2];
-          float2 vc, vd;  // the other pair, from the lane that holds it
-          vc.x = __shfl_xor_sync(0xffffffffu, va.x, 4);
-          vc.y = __shfl_xor_sync(0xffffffffu, va.y, 4);
-          vd.x = __shfl_xor_sync(0xffffffffu, vb.x, 4);
-          vd.y = __shfl_xor_sync(0xffffffffu, vb.y, 4);
-          b[0][k2].x = fmaf(px.y, vd.x, fmaf(px.x, vc.x, fmaf(po.y, vb.x, po.x * va.x)));
-          b[0][k2].y = fmaf(px.y, vd.y, fmaf(px.x, vc.y, fmaf(po.y, vb.y, po.x * va.y)));
-          b[1][k2].x = fmaf(px.w, vd.x, fmaf(px.z, vc.x, fmaf(po.z, vb.x, po.y * va.x)));
-          b[1][k2].y = fmaf(px.w, vd.y, fmaf(px.z, vc.y, fmaf(po.z, vb.y, po.y * va.y)));
+          for (int r = 0; r < H; ++r) {
+            const int e = (r * RA + it.j) * 8 + it.kp * 4 + it.w;
+            const float4 po = pso[e], px = psx[e];
+            const float2 pz = psz[e];
+            const float2 va = b[0][r], vb = b[1][r], vc = shfl_xor2(b[0][r + H]), vd = shfl_xor2(b[1][r + H]);
+            b[0][r].x = fmaf(px.x, vd.x, fmaf(po.w, vc.x, fmaf(po.y, vb.x, po.x * va.x)));
+            b[0][r].y = fmaf(px.x, vd.y, fmaf(po.w, vc.y, fmaf(po.y, vb.y, po.x * va.y)));
+            b[1][r].x = fmaf(px.z, vd.x, fmaf(px.y, vc.x, fmaf(po.z, vb.x, po.y * va.x)));
+            b[1][r].y = fmaf(px.z, vd.y, fmaf(px.y, vc.y, fmaf(po.z, vb.y, po.y * va.y)));
+            float2 yc, yd;
+            yc.x = fmaf(pz.x, vd.x, fmaf(px.w, vc.x, fmaf(px.y, vb.x, po.w * va.x)));
+            yc.y = fmaf(pz.x, vd.y, fmaf(px.w, vc.y, fmaf(px.y, vb.y, po.w * va.y)));
+            yd.x = fmaf(pz.y, vd.x, fmaf(pz.x, vc.x, fmaf(px.z, vb.x, px.x * va.x)));
+            yd.y = fmaf(pz.y, vd.y, fmaf(pz.x, vc.y, fmaf(px.z, vb.y, px.x * va.y)));
+            b[0][r + H] = shfl_xor2(yc);
+            b[1][r + H] = shfl_xor2(yd);
+          }
+        } else {
+#pragma unroll
+          for (int k2 = 0; k2 < RB; ++k2) {
+            const int e = (k2 * RA + it.j) * 8 + it.kp * 4 + it.w;
+            const float4 po = pso[e], px = psx[e];
+            const float2 va = b[0][k2], vb = b[1][k2];
+            float2 vc, vd;  // the other pair, from the lane that holds it
+            vc.x = __shfl_xor_sync(0xffffffffu, va.x, 4);
+            vc.y = __shfl_xor_sync(0xffffffffu, va.y, 4);
+            vd.x = __shfl_xor_sync(0xffffffffu, vb.x, 4);
+            vd.y = __shfl_xor_sync(0xffffffffu, vb.y, 4);
+            b[0][k2].x = fmaf(px.y, vd.x, fmaf(px.x, vc.x, fmaf(po.y, vb.x, po.x * va.x)));
+            b[0][k2].y = fmaf(px.y, vd.y, fmaf(px.x, vc.y, fmaf(po.y, vb.y, po.x * va.y)));
+            b[1][k2].x = fmaf(px.w, vd.x, fmaf(px.z, vc.x, fmaf(po.z, vb.x, po.y * va.x)));
+            b[1][k2].y = fmaf(px.w, vd.y, fmaf(px.z, vc.y, fmaf(po.z, vb.y, po.y * va.y)));
+          }
         }
 #pragma unroll
         for (int k = 0; k < 2; ++k) {

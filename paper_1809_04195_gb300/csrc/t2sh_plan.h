@@ -41,8 +41,9 @@ struct Geom {
   int P;               // K (K + 1) / 2: stored entries of Psi(n)
   float gsign;         // (-1)^(ny/2 + nz/2): global sign of the centred DFT
   float inv_sqrt_n;    // 1 / sqrt(ny nz)
-  int colvar;          // normal-operator column pass: 0 TMA tiles of 8 columns, 1 cp.async
-                       // tiles of 8, 2 cp.async tiles of 4 (size-specialised kernels),
+  int colvar;          // normal-operator column pass: 0 the default for the shape (interleaved
+                       // tiles of 4 columns x 4 images where K = 4, else planar TMA tiles of
+                       // 8 columns or run-time radices), planar variants: 1 cp.async tiles of 8, 2 cp.async tiles of 4 (size-specialised kernels),
                        // 3 tensor-core DFT-as-GEMM in split BF16 (mixed precision),
                        // 4 TMA tiles of 4 columns (two CTAs per SM)
   int* err;            // nullable device flag: set to 1 when a bounded wait ran out
