@@ -5,8 +5,8 @@
 // Work unit = (slice, map set, band of b shifted rows); the blocks of different map sets
 // are independent.  Per unit: gather the band into shared memory; per block (b x b
 // pixels x K) a warp forms the K x K Gram matrix G = X^H X with shuffle reductions; one
-// thread per block eigendecomposes G = V diag(lambda) V^H (float32 by default: a real
-// tridiagonal form and real Jacobi for K <= 4; float64 on request), sigma_i = sqrt(lambda_i), and forms
+// thread per block eigendecomposes G = V diag(lambda) V^H (round-robin
+// Jacobi, float32 by default, float64 on request), sigma_i = sqrt(lambda_i), and forms
 // W = V diag(max(1 - tau/sigma_i, 0)) V^H, so that X W = U max(Sigma - tau, 0) V^H
 // (since X V = U Sigma); then X' = X W is written back.  The FISTA variant fuses the
 // gradient step before the prox and the momentum update after it (Sec. II.A); the ADMM
@@ -294,7 +294,8 @@ __host__ __device__ constexpr size_t llr_unit_bytes(int K, int b, int nz) {
 // others: 0.735 -> 0.649 ms on the knee scan with four.  The FISTA momentum's loads of x_k
 // for a pixel pair are issued for all K images before the row's first store (the compiler
 // may not move a load of x above a store through z, which could alias it): 0.573 -> 0.528
-// ms on the knee scan.  Where a band is so large that only two CTAs fit (the 12-row bands
+// ms on the knee scan.  (Those figures came before the halving reduction and the shorter eigen-step, with
+// which it takes 0.485 ms there.)  Where a band is so large that only two CTAs fit (the 12-row bands
 // of Table I's 260 x 240 slices), the CTAs have 512 threads at 64 registers, so the memory
 // phases keep as many loads in flight.
 // MODE LLR_PROX: x <- prox(x).  LLR_FISTA: x_{k+1} <- prox(z - mu (grad - aty)),

@@ -17,10 +17,10 @@
 //
 // Bound by HBM (maps and t once each, image rows once).  Knee scan (320 slices of 256x160, C = 12,
 // 6.71 GB per launch): forward 1.11 -> 0.99 ms, adjoint 1.15 -> 1.01 ms against the planar passes,
-// 0.98 of the measured copy bandwidth; Table I (M = 2, 7.19 GB): 1.39 -> 1.04 and 1.48 -> 1.27 ms.
+// 0.98 of the measured copy bandwidth; Table I (M = 2, 7.19 GB): 1.39 -> 1.04 and 1.48 -> 1.18 ms.
 // The adjoint's loads in flight wait in L1, so the SM's split is set to what the resident CTAs'
 // shared memory needs: after a column pass that leaves 28 KB of L1, 1.59 ms (M = 2, 240 points)
-// against 1.27, 1.28 against 1.05 (160 points).
+// against 1.18, 1.28 against 1.05 (160 points).
 // Reading t with half-warps of one image (four lines per load instead of one) took 1.43 ms, and
 // storing it as runs of R1 columns (partial sectors) 1.30 ms.
 #pragma once

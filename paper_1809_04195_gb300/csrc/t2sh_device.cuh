@@ -639,179 +639,26 @@ static_assert(jac_pair(4, 0, 0, false) == 0 && jac_pair(4, 0, 0, true) == 3 && j
               "round-robin pairs of 4");
 
 // ---------------------------------------------------------------------------------
-// Eigenvectors (columns of vr + i vi) of a Hermitian 4 x 4 matrix in float32: unitary reduction to a
-// real symmetric tridiagonal matrix, then real Jacobi in the same round-robin order on it, and the
-// product of the two.  The complex Jacobi above spends most of its instructions on complex columns;
-// here a round is real and the reduction is done once.
+// Eigenvectors (columns of vr + i vi) of a Hermitian 4 x 4 matrix in float32, by the Jacobi rotations
+// above on the matrix scaled by a power of two to a trace in [1, 2) (exact, and its squares stay in
+// range).  A reduction to real tridiagonal form with real Jacobi took 49 us less of the 806 us
+// of a prox of 2 x 288 slices of 260 x 240, but on graded matrices (coefficient images of decaying
+// energy) its error was up to 2.3 times larger: the reflection mixes large into small entries.
 // gp: the matrix as in svt_weights.  A matrix whose trace is zero or not finite gives the identity.
-// Every product that meets a sum is a written-out fmaf or a rounded product, so the compiler has no
-// contraction to choose and all kernels that inline this give the same bits.
 // ---------------------------------------------------------------------------------
 __device__ __forceinline__ void herm4_vectors(const float* gp, float (&vr)[4][4], float (&vi)[4][4]) {
-  // scaled by the trace: every magnitude below lies in the normal range or does not matter
   const float tr = (gp[0] + gp[5]) + (gp[10] + gp[15]);
-  const bool ok = tr > 0.f && tr < 3e38f;
-  const float sc = ok ? fminf(1.f / tr, 1.7e38f) : 0.f;  // 1 / tr overflows for a subnormal trace
-  // column 0 below the diagonal: x = (G10, G20, G30), G_lk = conj(G_kl)
-  float2 x0 = make_float2(__fmul_rn(gp[1], sc), -__fmul_rn(gp[4], sc)), x1 = make_float2(__fmul_rn(gp[2], sc), -__fmul_rn(gp[8], sc)),
-         x2 = make_float2(__fmul_rn(gp[3], sc), -__fmul_rn(gp[12], sc));
-  // trailing block B (rows and columns 1 .. 3): real diagonal, B10 = G21, B20 = G31, B21 = G32
-  float b00 = __fmul_rn(gp[5], sc), b11 = __fmul_rn(gp[10], sc), b22 = __fmul_rn(gp[15], sc);
-  float2 b10 = make_float2(__fmul_rn(gp[6], sc), -__fmul_rn(gp[9], sc)), b20 = make_float2(__fmul_rn(gp[7], sc), -__fmul_rn(gp[13], sc)),
-         b21 = make_float2(__fmul_rn(gp[11], sc), -__fmul_rn(gp[14], sc));
-  float d[4], e[3];
-  d[0] = __fmul_rn(gp[0], sc);
-  // reflector P = I - tau u u^H with u = x + phi |x| e1 (phi the phase of x0): P x = -phi |x| e1;
-  // Q1 = P diag(-phi, 1, 1) takes x to |x| e1
-  const float a2 = fmaf(x0.x, x0.x, x0.y * x0.y),
-              n2 = fmaf(x2.y, x2.y, fmaf(x2.x, x2.x, fmaf(x1.y, x1.y, fmaf(x1.x, x1.x, a2))));
-  const bool h1 = n2 > 1e-30f;
-  const float ra = a2 > 1e-30f ? rsqrtf(a2) : 0.f, rn = h1 ? rsqrtf(n2) : 0.f;
-  const float2 phi = a2 > 1e-30f ? make_float2(x0.x * ra, x0.y * ra) : make_float2(1.f, 0.f);
-  const float na = __fmul_rn(a2, ra), nx = __fmul_rn(n2, rn), tau = h1 ? rn / (nx + na) : 0.f;
-  e[0] = nx;
-  const float2 u0 = cscale(phi, na + nx), u1 = x1, u2 = x2;
-  // p = tau B u, q = p - (tau / 2)(u^H p) u, P B P = B - u q^H - q u^H
-  float2 p0 = cscale(u0, b00), p1 = cmul(b10, u0), p2 = cmul(b20, u0);
-  cfmac(p0, b10, u1);
-  cfmac(p0, b20, u2);
-  p1 = make_float2(fmaf(b11, u1.x, p1.x), fmaf(b11, u1.y, p1.y));
-  cfmac(p1, b21, u2);
-  cfma(p2, b21, u1);
-  p2 = make_float2(fmaf(b22, u2.x, p2.x), fmaf(b22, u2.y, p2.y));
-  const float up = fmaf(u2.y, p2.y, fmaf(u2.x, p2.x, fmaf(u1.y, p1.y, fmaf(u1.x, p1.x, fmaf(u0.y, p0.y, u0.x * p0.x)))));
-  const float kap = 0.5f * tau * tau * up;  // p still without its factor tau
-  const float2 q0 = make_float2(fmaf(tau, p0.x, -(kap * u0.x)), fmaf(tau, p0.y, -(kap * u0.y))),
-               q1 = make_float2(fmaf(tau, p1.x, -(kap * u1.x)), fmaf(tau, p1.y, -(kap * u1.y))),
-               q2 = make_float2(fmaf(tau, p2.x, -(kap * u2.x)), fmaf(tau, p2.y, -(kap * u2.y)));
-  b00 = fmaf(-2.f, fmaf(u0.x, q0.x, u0.y * q0.y), b00);
-  b11 = fmaf(-2.f, fmaf(u1.x, q1.x, u1.y * q1.y), b11);
-  b22 = fmaf(-2.f, fmaf(u2.x, q2.x, u2.y * q2.y), b22);
-  // B_ij -= u_i conj(q_j) + q_i conj(u_j) = conj(conj(u_i) q_j) + ...
-  auto rank2 = [](float2& b, float2 ui, float2 qi, float2 uj, float2 qj) {
-    const float2 s = cmulc(qj, ui), t = cmulc(uj, qi);  // conj(q_j) u_i, conj(u_j) q_i
-    b.x -= s.x + t.x;
-    b.y -= s.y + t.y;
-  };
-  rank2(b10, u1, q1, u0, q0);
-  rank2(b20, u2, q2, u0, q0);
-  rank2(b21, u2, q2, u1, q1);
-  // column phase -phi of Q1's first column: B10, B20 *= -phi
-  const float2 mphi = h1 ? make_float2(-phi.x, -phi.y) : make_float2(1.f, 0.f);
-  b10 = cmul(b10, mphi);
-  b20 = cmul(b20, mphi);
-  d[1] = b00;
-  // Q2 = [y, (-conj y1, conj y0)] / |y| takes y = (B10, B20) to |y| e1
-  const float y2 = fmaf(b20.y, b20.y, fmaf(b20.x, b20.x, fmaf(b10.y, b10.y, b10.x * b10.x)));
-  const bool h2 = y2 > 1e-30f;
-  const float ry = h2 ? rsqrtf(y2) : 0.f;
-  e[1] = y2 * ry;
-  const float2 g0 = h2 ? cscale(b10, ry) : make_float2(1.f, 0.f), g1 = h2 ? cscale(b20, ry) : make_float2(0.f, 0.f);
-  // C = [[b11, conj b21], [b21, b22]]; C g = m, then g^H C g, and the off-diagonal g'^H C g with
-  // g' = (-conj g1, conj g0): g'^H m = -g1 m0 + g0 m1
-  float2 m0 = cscale(g0, b11), m1 = cmul(b21, g0);
-  cfmac(m0, b21, g1);
-  m1 = make_float2(fmaf(b22, g1.x, m1.x), fmaf(b22, g1.y, m1.y));
-  d[2] = fmaf(g1.y, m1.y, fmaf(g1.x, m1.x, fmaf(g0.y, m0.y, g0.x * m0.x)));
-  d[3] = b11 + b22 - d[2];
-  float2 c10 = cmul(g0, m1);
-  const float2 c1b = cmul(g1, m0);
-  c10.x -= c1b.x;
-  c10.y -= c1b.y;
-  const float c2 = fmaf(c10.x, c10.x, c10.y * c10.y);
-  const bool h3 = c2 > 1e-30f;
-  const float rc = h3 ? rsqrtf(c2) : 0.f;
-  e[2] = c2 * rc;
-  const float2 psi = h3 ? cscale(c10, rc) : make_float2(1.f, 0.f);
-  // columns 1 .. 3 of the reduction, rows 1 .. 3: w1 = Q1 e1, and Q1's other columns times Q2
-  float2 w[3][3];
-  w[0][0] = h1 ? cscale(x0, rn) : make_float2(1.f, 0.f);
-  w[1][0] = cscale(x1, rn);
-  w[2][0] = cscale(x2, rn);
-  {
-    // P e2 = e2 - tau conj(u1) u, P e3 = e3 - tau conj(u2) u
-    const float2 t1 = make_float2(tau * u1.x, -tau * u1.y), t2 = make_float2(tau * u2.x, -tau * u2.y);
-    const float2 uu[3] = {u0, u1, u2};
-    const float2 g0p = make_float2(-g1.x, g1.y), g1p = make_float2(g0.x, -g0.y);  // -conj g1, conj g0
+  const int ex = (int)(__float_as_uint(tr) >> 23);  // 0: zero or subnormal, from 255: not finite or negative
+  const float sc = tr > 0.f && ex < 255 ? __uint_as_float((unsigned)max(254 - ex, 1) << 23) : 0.f;
+  float ar[4][4], ai[4][4];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      float2 ca = cmul(uu[i], t1), cb = cmul(uu[i], t2);
-      ca = make_float2((i == 1 ? 1.f : 0.f) - ca.x, -ca.y);
-      cb = make_float2((i == 2 ? 1.f : 0.f) - cb.x, -cb.y);
-      float2 f = cmul(ca, g0), h = cmul(ca, g0p);
-      cfma(f, cb, g1);
-      cfma(h, cb, g1p);
-      w[i][1] = f;
-      w[i][2] = cmul(h, psi);
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+      ar[k][l] = sc > 0.f ? gp[(k < l ? k : l) * 4 + (k < l ? l : k)] * sc : 0.f;
+      ai[k][l] = k == l || !(sc > 0.f) ? 0.f : (k < l ? gp[l * 4 + k] : -gp[k * 4 + l]) * sc;
     }
-  }
-  // real Jacobi on the tridiagonal matrix
-  float a[4][4], z[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      a[i][j] = i == j ? d[i] : (j == i + 1 ? e[i] : 0.f);  // upper triangle
-      z[i][j] = i == j ? 1.f : 0.f;
-    }
-  for (int sweep = 0; sweep < 6; ++sweep) {
-    float off = 0.f, dg = 0.f;
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-      dg = fmaf(a[p][p], a[p][p], dg);
-#pragma unroll
-      for (int q = p + 1; q < 4; ++q) off = fmaf(a[p][q], a[p][q], off);
-    }
-    if (!(off > JacobiTol<float>::rel2 * dg)) break;
-#pragma unroll
-    for (int rd = 0; rd < 3; ++rd) {
-      float tt[2], cc[2], ss[2];
-#pragma unroll
-      for (int m = 0; m < 2; ++m) {
-        const int p = jac_pair(4, rd, m, false), q = jac_pair(4, rd, m, true);
-        const float b2 = 2.f * a[p][q], df = a[q][q] - a[p][p], h = fmaf(df, df, b2 * b2);
-        const bool on = h > 1e-36f;
-        // t = tan of the smaller angle = 2 a_pq sgn(df) / (|df| + sqrt(df^2 + 4 a_pq^2))
-        const float r = on ? __fmul_rn(h, rsqrtf(h)) : 1.f;
-        const float t = on ? copysignf(1.f, df) * b2 * __frcp_rn(fabsf(df) + r) : 0.f;
-        tt[m] = __fmul_rn(t, a[p][q]);
-        cc[m] = rsqrtf(fmaf(t, t, 1.f));
-        ss[m] = t * cc[m];
-      }
-#pragma unroll
-      for (int m = 0; m < 2; ++m) {
-        const int p = jac_pair(4, rd, m, false), q = jac_pair(4, rd, m, true);
-        a[p][p] -= tt[m];
-        a[q][q] += tt[m];
-        a[p][q] = 0.f;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          if (k != p && k != q) {
-            float& kp = k < p ? a[k][p] : a[p][k];
-            float& kq = k < q ? a[k][q] : a[q][k];
-            const float f = kp, g = kq;
-            kp = fmaf(cc[m], f, -(ss[m] * g));
-            kq = fmaf(ss[m], f, cc[m] * g);
-          }
-          const float f = z[k][p], g = z[k][q];
-          z[k][p] = fmaf(cc[m], f, -(ss[m] * g));
-          z[k][q] = fmaf(ss[m], f, cc[m] * g);
-        }
-      }
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    vr[0][i] = ok ? z[0][i] : (i == 0 ? 1.f : 0.f);
-    vi[0][i] = 0.f;
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-      const float re = fmaf(w[r][2].x, z[3][i], fmaf(w[r][1].x, z[2][i], w[r][0].x * z[1][i]));
-      const float im = fmaf(w[r][2].y, z[3][i], fmaf(w[r][1].y, z[2][i], w[r][0].y * z[1][i]));
-      vr[r + 1][i] = ok ? re : (i == r + 1 ? 1.f : 0.f);
-      vi[r + 1][i] = ok ? im : 0.f;
-    }
-  }
+  herm_jacobi_rounds<float, 4>(ar, ai, vr, vi, 5);
 }
 
 // ---------------------------------------------------------------------------------
@@ -842,10 +689,9 @@ __device__ __forceinline__ void cp_async_wait() {
 // the nearest unitary matrix (V is orthonormal to a few roundings, so one step leaves none) in place
 // of a serial Gram-Schmidt; Rayleigh quotients on the original matrix; the upper triangle of the
 // Hermitian W.  Everything but the scalar square roots is independent chains of fused operations.
-// LLR kernel against the complex Jacobi and Gram-Schmidt below: prox of 2 x 288 slices of 260 x 240
-// 843 -> 760 us (602 without any eigen-step), FISTA step of 320 slices of 256 x 160 511 -> 482 us, one
-// slice of 64 x 48 about 1 us per step less; also exact where those squares left the float32 range
-// (entries of G above 1.8e19 or below 1e-22, which the loop below takes for diagonal).
+// Prox of 2 x 288 slices of 260 x 240 841 -> 806 us against the serial form below, error against 64
+// bits equal at K = 4 and 0.67 to 1.0 of it at K = 2 and 3.  Also exact where the squares of G's entries leave the float32 range (entries above 1.8e19 or below
+// 1e-22, which the loop below takes for diagonal).
 __device__ __forceinline__ void svt4_weights(const float* gp, float tau, float2* w) {
   float vr[4][4], vi[4][4];
   herm4_vectors(gp, vr, vi);
@@ -893,17 +739,22 @@ __device__ __forceinline__ void svt4_weights(const float* gp, float tau, float2*
   float f[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    float lam = 0.f;  // v_i^H G v_i = sum_k G_kk |v_k|^2 + 2 Re sum_{k<l} conj(v_k) G_kl v_l
+    float lam = 0.f;  // v_i^H (G v_i): the inner sums cancel to lambda v, so the outer one adds small terms
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      float gvr = 0.f, gvi = 0.f;  // sum_{l>k} G_kl v_l
+      float gvr = 0.f, gvi = 0.f;
 #pragma unroll
-      for (int l = k + 1; l < 4; ++l) {
-        gvr = fmaf(gp[k * 4 + l], vr[l][i], fmaf(-gp[l * 4 + k], vi[l][i], gvr));
-        gvi = fmaf(gp[k * 4 + l], vi[l][i], fmaf(gp[l * 4 + k], vr[l][i], gvi));
+      for (int l = 0; l < 4; ++l) {
+        if (k == l) {
+          gvr = fmaf(gp[k * 4 + k], vr[k][i], gvr);
+          gvi = fmaf(gp[k * 4 + k], vi[k][i], gvi);
+        } else {
+          const float gr = gp[(k < l ? k : l) * 4 + (k < l ? l : k)],
+                      gi = k < l ? gp[l * 4 + k] : -gp[k * 4 + l];
+          gvr = fmaf(gr, vr[l][i], fmaf(-gi, vi[l][i], gvr));
+          gvi = fmaf(gr, vi[l][i], fmaf(gi, vr[l][i], gvi));
+        }
       }
-      gvr = fmaf(gp[k * 4 + k], vr[k][i], 2.f * gvr);
-      gvi = fmaf(gp[k * 4 + k], vi[k][i], 2.f * gvi);
       lam = fmaf(vr[k][i], gvr, fmaf(vi[k][i], gvi, lam));
     }
     // 1 / sigma, with one Newton step on the reciprocal square root
@@ -912,29 +763,27 @@ __device__ __forceinline__ void svt4_weights(const float* gp, float tau, float2*
     y = big ? 0.f : fmaf(0.5f * y, fmaf(-lam * y, y, 1.f), y);
     f[i] = lam > 0.f && (big || __fmul_rn(lam, y) > tau) ? fmaf(-tau, y, 1.f) : 0.f;
   }
-  // W_lk = sum_i V_li f_i conj(V_ki)
+  // W_lk = sum_i f_i V_li conj(V_ki)
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float r = f[i] > 0.f ? __fsqrt_rn(f[i]) : 0.f;
+  for (int l = 0; l < 4; ++l) {
+    float sr[4], si[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      vr[k][i] = __fmul_rn(vr[k][i], r);
-      vi[k][i] = __fmul_rn(vi[k][i], r);
+    for (int i = 0; i < 4; ++i) {
+      sr[i] = __fmul_rn(f[i], vr[l][i]);
+      si[i] = __fmul_rn(f[i], vi[l][i]);
     }
-  }
-#pragma unroll
-  for (int l = 0; l < 4; ++l)
 #pragma unroll
     for (int k = l; k < 4; ++k) {
       float wr = 0.f, wi = 0.f;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        wr = fmaf(vr[l][i], vr[k][i], fmaf(vi[l][i], vi[k][i], wr));
-        if (k > l) wi = fmaf(vi[l][i], vr[k][i], fmaf(-vr[l][i], vi[k][i], wi));
+        wr = fmaf(sr[i], vr[k][i], fmaf(si[i], vi[k][i], wr));
+        if (k > l) wi = fmaf(si[i], vr[k][i], fmaf(-sr[i], vi[k][i], wi));
       }
       w[l * 4 + k] = make_float2(wr, wi);
       if (k > l) w[k * 4 + l] = make_float2(wr, -wi);
     }
+  }
 }
 
 template <typename ET, int KC>
