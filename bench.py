@@ -578,7 +578,9 @@ def run_ours(args):
     if args.wavelet:  # read + write of each level's lattice, forward and inverse
         L = args.wavelet
         vol = S * sh.nmaps * sh.nbasis * N * 8
-        ab["post"] = ab.get("post", 0) + 2 * vol * (8.0 ** -(L - 1) + 2 * sum(8.0 ** -(l - 1) for l in range(1, L)))
+        # up to three levels run in one pass over the volume, deeper pyramids level by level
+        ab["post"] = ab.get("post", 0) + 2 * vol * (
+            1.0 if L <= 3 else 8.0 ** -(L - 1) + 2 * sum(8.0 ** -(l - 1) for l in range(1, L)))
     if args.solver == "admm":
         vec = (1 if args.form == "per-slice" else S) * sh.nmaps * sh.nbasis * N * 8
         ab["llr"] = 4 * vec  # read alpha, u; write v, u

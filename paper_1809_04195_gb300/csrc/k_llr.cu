@@ -295,7 +295,7 @@ __host__ __device__ constexpr size_t llr_unit_bytes(int K, int b, int nz) {
 // for a pixel pair are issued for all K images before the row's first store (the compiler
 // may not move a load of x above a store through z, which could alias it): 0.573 -> 0.528
 // ms on the knee scan.  (Those figures came before the halving reduction and the shorter eigen-step, with
-// which it takes 0.485 ms there.)  Where a band is so large that only two CTAs fit (the 12-row bands
+// which it takes 0.488 ms there.)  Where a band is so large that only two CTAs fit (the 12-row bands
 // of Table I's 260 x 240 slices), the CTAs have 512 threads at 64 registers, so the memory
 // phases keep as many loads in flight.
 // MODE LLR_PROX: x <- prox(x).  LLR_FISTA: x_{k+1} <- prox(z - mu (grad - aty)),
