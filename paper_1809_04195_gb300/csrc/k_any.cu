@@ -73,6 +73,22 @@ struct AnyCol {
   int psi_sm;  // Psi of the tile's columns kept in shared memory (up to four images)
 };
 
+// Threads of a column CTA: whole items of LK threads, in as few equal rounds as kColThreads allows.
+constexpr int col_threads(int LK, int items) {
+  const int at_once = kColThreads / LK, rounds = (items + at_once - 1) / at_once;
+  return (LK * ((items + rounds - 1) / rounds) + 31) / 32 * 32;
+}
+constexpr bool col_threads_fit() {
+  for (int k = 1; k <= kMaxK; ++k)
+    for (int w = 2; w <= 4; w += 2)
+      for (int items = 2; items <= kMaxRadix; ++items) {
+        const int t = col_threads(k * w, items);
+        if (t < k * w || t > kColThreads) return false;
+      }
+  return true;
+}
+static_assert(col_threads_fit(), "every column CTA within its launch bounds");
+
 // Persistent CTAs over contiguous runs of the (column chunk, slice x coil) list, column-chunk major:
 // Psi of a chunk's columns is copied to shared memory once per run.  The next tile streams in by
 // cp.async while the current one is transformed.
@@ -440,9 +456,7 @@ cudaError_t launch_col_any(const Geom& g, int W, IlPass pass, const float2* tw_y
   AnyCol a{};
   size_t sm = 0;
   if (!col_any_plan(g, W, pass, &a, &sm)) return cudaErrorNotSupported;
-  const int LK = g.K * W, items = std::max(a.RA, a.RB);
-  const int rounds = (LK * items + kColThreads - 1) / kColThreads;
-  const int threads = (LK * ((items + rounds - 1) / rounds) + 31) / 32 * 32;
+  const int threads = col_threads(g.K * W, std::max(a.RA, a.RB));
   const long long nsc = (long long)g.S * g.C, ntiles = nsc * (g.nz / W);
   const void* kern = g.K <= 4 ? (const void*)k_col_any<4> : (const void*)k_col_any<8>;
   int nsm = 0, per = 0;

@@ -132,7 +132,7 @@ cudaError_t ctas_per_sm(const void* kernel, int threads, size_t smem, int* per) 
   }
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per, kernel, threads, smem);
   if (e != cudaSuccess) return e;
-  if (*per < 1) *per = 1;
+  if (*per < 1) return cudaErrorLaunchOutOfResources;
   g_per[key] = *per;
   return cudaSuccess;
 }
