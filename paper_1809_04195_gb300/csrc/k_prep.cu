@@ -269,8 +269,9 @@ __global__ void __launch_bounds__(kThreads) k_project(Geom g, TLayout lt, const 
 // times the input): one thread owns two neighbouring points and writes 16 bytes per echo, whole
 // 512-byte runs per warp, so it is bound by HBM writes.  256x160, C = 12, T = 80, 8 slices
 // (2.5 GB): 400 us, 0.93 of the measured copy bandwidth; 745 us when the column pass wrote the
-// echoes itself in 64-byte runs, 445 us with the column pass now.
-template <int KC>
+// echoes itself in 64-byte runs, 445 us with the column pass now.  WIDE: y is 16-byte aligned; an
+// array that starts at an odd value of another takes 8-byte stores.
+template <int KC, bool WIDE>
 __global__ void __launch_bounds__(kThreads) k_expand_te(Geom g, TLayout lt, const float* __restrict__ phi,
                                                       const unsigned* __restrict__ bits,
                                                       const float2* __restrict__ v, float2* __restrict__ y) {
@@ -289,8 +290,7 @@ __global__ void __launch_bounds__(kThreads) k_expand_te(Geom g, TLayout lt, cons
 #pragma unroll
     for (int k = 0; k < KC; ++k)
       a[k] = k < g.K ? *reinterpret_cast<const float4*>(v + pl.at(k)) : make_float4(0.f, 0.f, 0.f, 0.f);
-    float4* yb = reinterpret_cast<float4*>(y + sc * g.T * (long long)N + n);
-    const long long step = N / 2;
+    float2* yb = y + sc * g.T * (long long)N + n;
     for (int t0 = 0; t0 < g.T; t0 += 32) {
       uint2 b = *reinterpret_cast<const uint2*>(bits + (long long)(t0 >> 5) * N + n);
       const int m = min(32, g.T - t0);
@@ -314,8 +314,13 @@ __global__ void __launch_bounds__(kThreads) k_expand_te(Geom g, TLayout lt, cons
               o.w = fmaf(ph[k], a[k].w, o.w);
             }
         }
-        __stcs(yb, o);
-        yb += step;
+        if constexpr (WIDE) {
+          __stcs(reinterpret_cast<float4*>(yb), o);
+        } else {
+          __stcs(yb, make_float2(o.x, o.y));
+          __stcs(yb + 1, make_float2(o.z, o.w));
+        }
+        yb += N;
       }
     }
   }
@@ -370,7 +375,10 @@ cudaError_t launch_expand_te(const Geom& g, const TLayout& lt, const float* phi,
   const long long nsc = (long long)g.S * g.C;
   dim3 grid((N2 + kThreads - 1) / kThreads, (unsigned)(nsc < 65535 ? nsc : 65535));
   const size_t sm = sizeof(float) * g.T * g.K;
-  return launch_pdl(g.K <= 4 ? k_expand_te<4> : k_expand_te<8>, grid, kThreads, sm, st, g, lt, phi, bits, v, y_te);
+  const bool wide = ((uintptr_t)y_te & 15) == 0;
+  auto kern = g.K <= 4 ? (wide ? k_expand_te<4, true> : k_expand_te<4, false>)
+                       : (wide ? k_expand_te<8, true> : k_expand_te<8, false>);
+  return launch_pdl(kern, grid, kThreads, sm, st, g, lt, phi, bits, v, y_te);
 }
 
 }  // namespace t2sh
