@@ -94,7 +94,8 @@ __device__ __forceinline__ float2 cluster_lds2(const float2* p, int rank) {
   return v;
 }
 
-// CTAs that share a band's coils: as many as keep the launch within one wave of resident CTAs, more
+// CTAs that share a band's coils: as many as keep the whole plan's launch within one wave of resident CTAs (a
+// launch over some of its slices takes the same number: it sets the order of the sum over the coils), more
 // than four only within half a wave, and at most eight, the portable size of the cluster in which the
 // adjoint sums over the coils.  One slice of 64 x 48, C = 8: forward 4.6 -> 2.3 us, adjoint 5.6 -> 4.2,
 // a 50-iteration solve 1.22 -> 1.11 ms (1.14 with four CTAs); two slices with M = 2: 1.26 ms with four,
@@ -288,7 +289,7 @@ cudaError_t row_il_go(const Geom& g, int trb, const float2* tw, const float2* ma
   const cudaError_t es = sm_count(&nsm);
   if (es != cudaSuccess) return es;
   const int nb = (g.ny + R::RB - 1) / R::RB;
-  const int ns = row_split((long long)nb * g.S, (long long)nsm * R::MINB, g.C);
+  const int ns = row_split((long long)nb * g.Sp, (long long)nsm * R::MINB, g.C);
   const int cs = (g.C + ns - 1) / ns;
   return launch_pdl_cluster(k_row_il<N, RI, RT, MODE, MC>, dim3(nb, g.S, ns), MODE == ROW_ADJ ? ns : 1, R::THREADS,
                             R::smem, st, g, trb, cs, tw, maps, x, t, out);

@@ -447,7 +447,7 @@ t2sh_status t2sh_plan(const t2sh_dims* dims, const float* phi, const uint8_t* ma
   p->host_io = (dims->flags & T2SH_HOST_IO) != 0;
   const t2sh_dims& d = p->d;
   Geom& g = p->g;
-  g.S = d.nslices; g.C = d.ncoils; g.M = d.nmaps; g.K = d.nbasis; g.T = d.nechoes;
+  g.S = g.Sp = d.nslices; g.C = d.ncoils; g.M = d.nmaps; g.K = d.nbasis; g.T = d.nechoes;
   g.ny = d.ny; g.nz = d.nz; g.P = d.nbasis * (d.nbasis + 1) / 2;
   g.gsign = (((d.ny / 2) + (d.nz / 2)) & 1) ? -1.f : 1.f;
   g.inv_sqrt_n = (float)(1.0 / std::sqrt((double)d.ny * d.nz));

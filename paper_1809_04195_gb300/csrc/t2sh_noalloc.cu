@@ -126,7 +126,7 @@ extern "C" t2sh_status t2sh_normal_op_noalloc(const t2sh_dims* dims, const float
   float2* t = reinterpret_cast<float2*>(base + off_t);
 
   Geom g{};
-  g.S = d.nslices; g.C = d.ncoils; g.M = d.nmaps; g.K = d.nbasis; g.T = d.nechoes;
+  g.S = g.Sp = d.nslices; g.C = d.ncoils; g.M = d.nmaps; g.K = d.nbasis; g.T = d.nechoes;
   g.ny = d.ny; g.nz = d.nz; g.P = P;
   g.gsign = (((d.ny / 2) + (d.nz / 2)) & 1) ? -1.f : 1.f;
   g.inv_sqrt_n = (float)(1.0 / sqrt((double)N));

@@ -37,6 +37,8 @@ inline bool plan_has13(const FftPlan& p) {
 // Geometry of one batch of slices, passed by value to every kernel.
 struct Geom {
   int S, C, M, K, T;   // slices, coils, map sets, basis size, echoes
+  int Sp;              // slices of the whole plan (S of them in this launch): what sets the order of a
+                       // sum goes by Sp, so a slice's bits do not depend on the launch it is part of
   int ny, nz;          // slice matrix
   int P;               // K (K + 1) / 2: stored entries of Psi(n)
   float gsign;         // (-1)^(ny/2 + nz/2): global sign of the centred DFT
