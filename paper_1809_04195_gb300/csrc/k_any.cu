@@ -317,7 +317,7 @@ __device__ __forceinline__ void row_t_adj(float2* ex, int xs, int i, const float
 template <int MODE, int MC>
 __global__ void __launch_bounds__(kRowThreads, MC == 1 ? 3 : 2)
     k_row_any(Geom g, AnyRow a, const float2* __restrict__ tw_g, const float2* __restrict__ maps,
-              const float2* __restrict__ x, float2* __restrict__ t, float2* __restrict__ out) {
+              const float2* x, float2* t, float2* __restrict__ out) {
   extern __shared__ float2 smem[];
   const int N = g.nz, K = g.K, RI = a.RI, RT = a.RT, rows = a.rows, nl = K * rows, LK = K * a.W, xs = a.xs;
   const int wl = a.W == 4 ? 2 : 1;

@@ -54,9 +54,8 @@ __device__ __forceinline__ float cta_quotient(const double* num, const double* d
 #define CG_INDEX(i) (2 * ((long long)(blockIdx.x * kCgPerThread + (i)) * kCgThreads + threadIdx.x))
 
 // r = aty + rho (v - u) - w - rho x  (w = A^H A x);  p = r;  rr[s] += |r|^2
-__global__ void __launch_bounds__(kCgThreads) k_cg_init(long long L, const float2* __restrict__ x,
-                                                       const float2* __restrict__ w, const float2* __restrict__ aty,
-                                                       const float2* __restrict__ v, const float2* __restrict__ u,
+__global__ void __launch_bounds__(kCgThreads) k_cg_init(long long L, const float2* x, const float2* w,
+                                                       const float2* aty, const float2* v, const float2* u,
                                                        float rho, float2* __restrict__ r, float2* __restrict__ p,
                                                        double* rr) {
   pdl_wait();
@@ -90,8 +89,8 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_init(long long L, const float
 }
 
 // pq[s] += Re <p, w + rho p>  (w = A^H A p)
-__global__ void __launch_bounds__(kCgThreads) k_cg_dot(long long L, const float2* __restrict__ p,
-                                                      const float2* __restrict__ w, float rho, double* pq) {
+__global__ void __launch_bounds__(kCgThreads) k_cg_dot(long long L, const float2* p, const float2* w, float rho,
+                                                      double* pq) {
   pdl_wait();
   pdl_trigger();
   const long long base = (long long)blockIdx.y * L;
@@ -114,9 +113,9 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_dot(long long L, const float2
 }
 
 // a = rr / pq;  x += a p;  r -= a (w + rho p);  rr_new[s] += |r|^2
-__global__ void __launch_bounds__(kCgThreads) k_cg_step(long long L, float2* __restrict__ x, float2* __restrict__ r,
-                                                       const float2* __restrict__ p, const float2* __restrict__ w,
-                                                       float rho, const double* rr, const double* pq,
+__global__ void __launch_bounds__(kCgThreads) k_cg_step(long long L, float2* x, float2* r, const float2* p,
+                                                       const float2* w, float rho,
+                                                       const double* rr, const double* pq,
                                                        double* rr_new) {
   pdl_wait();
   pdl_trigger();
@@ -155,8 +154,8 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_step(long long L, float2* __r
 
 // b = rr_new / rr;  p = r + b p.  The first CTA of each slice also clears the
 // accumulators the next iteration adds into (pq and the next rr_new slot).
-__global__ void __launch_bounds__(kCgThreads) k_cg_dir(long long L, const float2* __restrict__ r,
-                                                      float2* __restrict__ p, const double* rr, const double* rr_new,
+__global__ void __launch_bounds__(kCgThreads) k_cg_dir(long long L, const float2* r, float2* p,
+                                                      const double* rr, const double* rr_new,
                                                       double* pq, double* rr_next) {
   pdl_wait();
   pdl_trigger();

@@ -66,8 +66,8 @@ struct RowFastRB {
 
 template <int N, int MODE, int MC, int kRowRB = RowFastRB<N, MC, MODE>::value>
 __device__ __forceinline__ void row_fast_body(const Geom& g, const float2* __restrict__ tw_g,
-                                              const float2* __restrict__ maps, const float2* __restrict__ x,
-                                              float2* __restrict__ t, float2* __restrict__ out) {
+                                              const float2* __restrict__ maps, const float2* x, float2* t,
+                                              float2* __restrict__ out) {
   constexpr int R1 = N / 16;
   constexpr int LINE = RowPad<N>::LX;
   constexpr int MS = RowPad<N>::MS;
@@ -215,14 +215,14 @@ __device__ __forceinline__ void row_fast_body(const Geom& g, const float2* __res
 template <int N, int MODE, int MC>
 __global__ void __launch_bounds__(64 * RowFastRB<N, MC, MODE>::value, RowFastRB<N, MC, MODE>::min_blocks)
     k_row_fast(Geom g, const float2* __restrict__ tw_g, const float2* __restrict__ maps,
-               const float2* __restrict__ x, float2* __restrict__ t, float2* __restrict__ out) {
+               const float2* x, float2* t, float2* __restrict__ out) {
   row_fast_body<N, MODE, MC>(g, tw_g, maps, x, t, out);
 }
 
 template <int N, int MODE, int MC>
 __global__ void __launch_bounds__(64 * RowFastRB<N, MC, MODE>::value)
     k_row_fast_wide(Geom g, const float2* __restrict__ tw_g, const float2* __restrict__ maps,
-                    const float2* __restrict__ x, float2* __restrict__ t, float2* __restrict__ out) {
+                    const float2* x, float2* t, float2* __restrict__ out) {
   row_fast_body<N, MODE, MC>(g, tw_g, maps, x, t, out);
 }
 

@@ -79,8 +79,8 @@ __device__ __forceinline__ int llr_row0(const Geom& g, const FistaArgs& a, const
 // t0 .. t0 + nth - 1 of the CTA
 template <int KC, int MODE>
 __device__ __forceinline__ void llr_gather(const Geom& g, const FistaArgs& a, const LlrUnit& un, float2* gs,
-                                           const float2* x, const float2* z, const float2* __restrict__ grad,
-                                           const float2* __restrict__ aty, const float2* u, int t0, int nth) {
+                                           const float2* x, const float2* z, const float2* grad, const float2* aty,
+                                           const float2* u, int t0, int nth) {
   const int ny = g.ny, nz = g.nz, N = ny * nz, K = g.K, rb = un.rb;
   const LlrCols c = llr_cols(nz, t0, nth);
   if (!c.active) return;
@@ -304,7 +304,7 @@ __host__ __device__ constexpr size_t llr_unit_bytes(int K, int b, int nz) {
 // One CTA's work: unit = (slice s, map set m0, band) decoded by llr_unit.
 template <int KC, int MODE, typename ET, int NT>
 __device__ __forceinline__ void llr_band(const Geom& g, const FistaArgs& a, int unit, float2* x, float2* z,
-                                         const float2* __restrict__ grad, const float2* __restrict__ aty, float2* u) {
+                                         const float2* grad, const float2* aty, float2* u) {
   extern __shared__ float2 smem[];
   pdl_wait();
   pdl_trigger();
@@ -327,8 +327,7 @@ __device__ __forceinline__ void llr_band(const Geom& g, const FistaArgs& a, int 
 
 template <int KC, int MODE, typename ET, int MINB, int NT = kThreads>
 __global__ void __launch_bounds__(NT, MINB)
-    k_llr(Geom g, FistaArgs a, float2* x, float2* z, const float2* __restrict__ grad,
-          const float2* __restrict__ aty, float2* u) {
+    k_llr(Geom g, FistaArgs a, float2* x, float2* z, const float2* grad, const float2* aty, float2* u) {
   const int nbands = (g.ny + a.b - 1) / a.b;
   llr_band<KC, MODE, ET, NT>(g, a, (blockIdx.y * g.M + blockIdx.z) * nbands + blockIdx.x, x, z, grad, aty, u);
 }

@@ -190,7 +190,7 @@ struct TePlace {
 
 __device__ __forceinline__ float2 ld_sample(const float2* p) {
   float2 v;
-  asm("ld.global.nc.L1::no_allocate.L2::64B.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  asm volatile("ld.global.L1::no_allocate.L2::64B.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
   return v;
 }
 
@@ -203,7 +203,7 @@ __device__ __forceinline__ float2 ld_sample(const float2* p) {
 template <int KC, int NP, int NS>
 __global__ void __launch_bounds__(kThreads) k_project(Geom g, TLayout lt, const float* __restrict__ phi,
                                                     const unsigned* __restrict__ bits,
-                                                    const float2* __restrict__ y, float2* __restrict__ out) {
+                                                    const float2* y, float2* __restrict__ out) {
   extern __shared__ float sphi[];
   for (int i = threadIdx.x; i < g.T * g.K; i += blockDim.x) sphi[i] = phi[i];
   __syncthreads();
@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(kThreads) k_project(Geom g, TLayout lt, const 
 template <int KC, bool WIDE>
 __global__ void __launch_bounds__(kThreads) k_expand_te(Geom g, TLayout lt, const float* __restrict__ phi,
                                                       const unsigned* __restrict__ bits,
-                                                      const float2* __restrict__ v, float2* __restrict__ y) {
+                                                      const float2* v, float2* __restrict__ y) {
   extern __shared__ float sphi[];
   for (int i = threadIdx.x; i < g.T * g.K; i += blockDim.x) sphi[i] = phi[i];
   __syncthreads();

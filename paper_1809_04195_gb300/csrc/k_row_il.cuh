@@ -112,7 +112,7 @@ inline int row_split(long long ctas, long long resident, int C) {
 template <int N, int RI, int RT, int MODE, int MC>
 __global__ void __launch_bounds__(RowIl<N, RI, RT, MODE, MC>::THREADS, RowIl<N, RI, RT, MODE, MC>::MINB)
     k_row_il(Geom g, int trb, int cs, const float2* __restrict__ tw_g, const float2* __restrict__ maps,
-             const float2* __restrict__ x, float2* __restrict__ t, float2* __restrict__ out) {
+             const float2* x, float2* t, float2* __restrict__ out) {
   using R = RowIl<N, RI, RT, MODE, MC>;
   constexpr int LINE = R::LINE, S = R::S, RB = R::RB;
   extern __shared__ float2 smem[];

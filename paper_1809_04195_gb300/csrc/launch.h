@@ -2,7 +2,10 @@
 // stream serialisation).  The kernel runs its prologue (tables, barriers, plan-owned constants) and
 // then pdl_wait(), after which the previous kernels' results are visible; pdl_trigger() lets the next
 // such kernel do the same.  A kernel triggers only after its own wait, so whatever ran before the
-// previous kernel has completed when a prologue runs.
+// previous kernel has completed when a prologue runs.  What the previous kernel may have written is
+// not read-only while this one runs: an argument that is read after the wait and written by another
+// kernel carries no `__restrict__` (its loads could be hoisted above the wait, and a `const` one's
+// sent through the read-only path), and no asm load of it is without `volatile`.
 #pragma once
 
 #include <cuda_runtime.h>

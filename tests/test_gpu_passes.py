@@ -166,3 +166,27 @@ def test_operators_on_odd_views(T, ny, nz, K):  # noqa: F811
             assert torch.equal(out, ref) if shape == yt.shape else nrmse(host(out), host(ref)) < OP_TOL
             assert buf[0] == 7 and bool((buf[-2:] == 7).all())
         p.sync()
+
+
+def test_chained_operators_see_the_previous_result(T):  # noqa: F811
+    """Every kernel may start while the one before it still runs: operators chained on one array give the
+    bits that they give with a synchronisation after each, over many repetitions."""
+    import torch
+
+    rng, phi, mask, maps = random_problem(7, 6, 54, 50, 5, 20, 4, 1)   # rows that share DRAM sectors
+    x0 = c64(crandn(rng, 6, 1, 4, 54, 50))
+    with make_plan(T, phi, mask, maps) as p:
+        def chain(sync):
+            x, y = x0.clone(), torch.empty((6, 5, 20, 54, 50), dtype=torch.complex64, device="cuda")
+            for i in range(8):
+                p.forward(x, T.KSPACE_TE, out=y), sync()
+                p.adjoint(y, T.KSPACE_TE, out=x), sync()
+                p.llr_prox(x, 0.01, i % 4, i % 3), sync()
+                p.normal_op(x, out=x), sync()
+            torch.cuda.synchronize()
+            return x
+        ref = chain(torch.cuda.synchronize)
+        assert bool(torch.isfinite(torch.view_as_real(ref)).all()) and float(ref.abs().max()) > 0
+        for _ in range(20):
+            assert torch.equal(chain(lambda: None), ref)
+        p.sync()
