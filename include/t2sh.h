@@ -381,7 +381,8 @@ t2sh_status t2sh_get_step(t2sh_plan_t plan, float* step);
  */
 t2sh_status t2sh_shifts(uint64_t seed, int32_t iters, int32_t block, int32_t* out);
 
-/* Host only: device bytes a plan with these dims allocates (for admission control). */
+/* Host only: the most device bytes that making a plan with these dims and its FISTA solves through device
+ * buffers hold (for admission control). */
 t2sh_status t2sh_workspace_bytes(const t2sh_dims* dims, size_t* bytes);
 
 /*

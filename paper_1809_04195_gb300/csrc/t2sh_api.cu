@@ -179,9 +179,12 @@ bool make_fft_plan(int n, FftPlan& p) {
 
 size_t cbytes(long long n) { return (size_t)n * sizeof(float2); }
 
+// bits: the sampling pattern as bit words; mask: as bytes, which a host-IO plan stages in t where it fits
+// and in a buffer of its own, freed again, where not.  pattern: what both come to at most (never under
+// the byte mask, which callers' budgets have counted).
 struct Footprint {
-  size_t maps, psi, phi, mask, vec, t, tw, shifts, red;
-  size_t total() const { return maps + psi + phi + mask + 4 * vec + t + tw + shifts + red; }
+  size_t maps, psi, phi, mask, bits, pattern, vec, t, tw, shifts, red;
+  size_t total() const { return maps + psi + phi + pattern + 4 * vec + t + tw + shifts + red; }
 };
 
 Footprint footprint(const t2sh_dims& d) {
@@ -192,8 +195,10 @@ Footprint footprint(const t2sh_dims& d) {
   f.psi = sizeof(float) * P * N;
   f.phi = sizeof(float) * d.nechoes * d.nbasis;
   f.mask = (size_t)d.nechoes * N;
+  f.bits = sizeof(unsigned) * ((size_t)(d.nechoes + 31) / 32) * N;
   f.vec = cbytes((long long)d.nslices * d.nmaps * d.nbasis * N);
   f.t = cbytes((long long)d.nslices * d.ncoils * d.nbasis * N);
+  f.pattern = (d.flags & T2SH_HOST_IO) && f.mask > f.t ? f.mask + f.bits : std::max(f.mask, f.bits);
   f.tw = cbytes(d.ny + d.nz);
   f.shifts = 0;
   f.red = sizeof(double) * 2 * (size_t)(d.iters > 0 ? d.iters : 1) + 64;
@@ -310,6 +315,16 @@ struct t2sh_plan_s {
     allocs.emplace_back(q, pool != nullptr);
     *p = static_cast<T*>(q);
     return T2SH_OK;
+  }
+  // Frees the newest allocation; the pool may hand it on when this returns.
+  void release_last() {
+    if (allocs.back().second) {
+      cudaFreeAsync(allocs.back().first, st);
+      cudaStreamSynchronize(st);
+    } else {
+      cudaFree(allocs.back().first);
+    }
+    allocs.pop_back();
   }
   ~t2sh_plan_s() {
     if (cs) cudaStreamSynchronize(cs);
@@ -470,8 +485,7 @@ t2sh_status t2sh_plan(const t2sh_dims* dims, const float* phi, const uint8_t* ma
   ALLOC(p->maps, f.maps);
   ALLOC(p->psi, f.psi);
   ALLOC(p->phi, f.phi);
-  const size_t word_bytes = (size_t)((d.nechoes + 31) / 32) * 4 * d.ny * d.nz;
-  ALLOC(p->bits, word_bytes);
+  ALLOC(p->bits, f.bits);
   ALLOC(p->x, f.vec);
   ALLOC(p->z, f.vec);
   ALLOC(p->aty, f.vec);
@@ -534,6 +548,7 @@ t2sh_status t2sh_plan(const t2sh_dims* dims, const float* phi, const uint8_t* ma
   FAIL_CK(cudaMemcpyAsync(bits, p->red, sizeof(bits), cudaMemcpyDeviceToHost, p->st));
   FAIL_CK(cudaStreamSynchronize(p->st));
 #undef FAIL_CK
+  if (p->host_io && f.mask > f.t) p->release_last();  // the byte mask's buffer
   float lam_s, lam_psi;
   std::memcpy(&lam_s, &bits[0], 4);
   std::memcpy(&lam_psi, &bits[1], 4);

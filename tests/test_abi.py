@@ -94,6 +94,17 @@ def test_workspace_bytes_formula(lib):
     assert t2sh.workspace_bytes(d) == expect
 
 
+@pytest.mark.parametrize("T,K,S,flags,pattern", [
+    (1, 1, 1, 0, 4), (3, 2, 1, 0, 4), (33, 4, 1, 0, 33),  # bit words (4 bytes per 32 echoes) or bytes, the larger
+    (65, 1, 1, t2sh.HOST_IO, 65 + 12),                    # byte mask beyond t: staged beside the words
+    (65, 4, 40, t2sh.HOST_IO, 65),
+])
+def test_workspace_bytes_cover_the_sampling_pattern(lib, T, K, S, flags, pattern):
+    N = 64 * 48
+    rest = S * N * 8 + K * (K + 1) // 2 * N * 4 + T * K * 4 + 4 * S * K * N * 8 + S * K * N * 8 + (64 + 48) * 8 + 16 * 2 + 64
+    assert t2sh.workspace_bytes(t2sh.make_dims(64, 48, 1, T, K, nslices=S, block=8, iters=2, flags=flags)) == rest + pattern * N
+
+
 @pytest.mark.parametrize("kw,status", [
     (dict(ny=63), t2sh.EINVAL),          # odd
     (dict(nz=14 * 7), t2sh.EINVAL),      # 98 = 2 * 7^2: 7 is not a radix of the FFT passes

@@ -93,3 +93,24 @@ def test_plan_memory_is_reused_bitwise_and_released(T):
     # what torch's own allocator kept of the solve outputs is not the plan pool's
     torch_kept = torch.cuda.memory_reserved() - torch0
     assert free0 - torch.cuda.mem_get_info()[0] - torch_kept < 0.1 * ws
+
+
+def test_byte_mask_of_a_host_plan_is_not_kept(T):
+    """A host-buffer plan whose byte mask is larger than its per-coil buffer stages the mask beside the bit
+    words while it is made, within workspace_bytes, and does not keep it."""
+    ny, nz, Tn = 512, 512, 1024
+    d = T.make_dims(ny, nz, 1, Tn, 1, nslices=1, block=8, iters=2, flags=T.HOST_IO)
+    rng = np.random.default_rng(3)
+    phi = rng.normal(size=(Tn, 1)).astype(np.float32)
+    mask = (rng.random((Tn, ny, nz), dtype=np.float32) < 0.02).astype(np.uint8)
+    maps = np.ones((1, 1, 1, ny, nz), np.complex64)
+    torch.cuda.synchronize()
+    T.release_cached()
+    free0 = torch.cuda.mem_get_info()[0]
+    with T.Plan(d, phi, mask, maps):
+        peak = free0 - torch.cuda.mem_get_info()[0]
+        T.release_cached()
+        held = free0 - torch.cuda.mem_get_info()[0]
+    slack = 64 << 20  # the pool's granularity
+    assert peak <= T.workspace_bytes(d) + slack
+    assert held <= T.workspace_bytes(d) - mask.nbytes + slack
