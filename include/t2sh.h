@@ -337,7 +337,8 @@ t2sh_status t2sh_batch_schedule(int32_t per_scan_llr);
  * separate versus fused row kernels, by timing probe_iters
  * iterations (default 3 when <= 0) of each candidate on the plan's buffers; the choice
  * is remembered per shape (and appended to the file named by the environment variable
- * T2SH_TUNE_CACHE, read back by later processes).  With probe_iters >= 0 a shape that is
+ * T2SH_TUNE_CACHE, read back by later processes of builds with the same kernels to choose
+ * from; other lines of it are passed over).  With probe_iters >= 0 a shape that is
  * already known is not timed again; probe_iters < 0 forces a new measurement.  Clobbers
  * the plan's FISTA state: call it before t2sh_solve_begin.  Synchronises the stream.
  * col_variant_out / fused_out (nullable) receive the choice.

@@ -1306,6 +1306,10 @@ t2sh_status t2sh_objective(t2sh_plan_t p, const void* kspace, int32_t kform, con
 // memory and, when T2SH_TUNE_CACHE names a file, in that file (one line per shape).
 // ---------------------------------------------------------------------------------
 namespace {
+// First word of a line of the tuning file: the set of kernels that the choice was made among.  It
+// changes whenever a variant, or the default that variants are timed against, becomes another kernel;
+// lines that begin otherwise (those of the planar default had no such word) are not taken.
+constexpr char kTuneSet[] = "il1";
 std::mutex g_tune_mu;
 std::map<std::string, std::pair<int, int>> g_tune;  // shape -> (colw, fused)
 bool g_tune_loaded = false;
@@ -1324,8 +1328,12 @@ void tune_load() {
   FILE* fp = std::fopen(f, "r");
   if (!fp) return;
   int a[9];
-  while (std::fscanf(fp, "%d %d %d %d %d %d %d %d %d", &a[0], &a[1], &a[2], &a[3], &a[4], &a[5], &a[6], &a[7],
-                     &a[8]) == 9) {
+  char line[256], set[16];
+  while (std::fgets(line, sizeof(line), fp)) {
+    if (std::sscanf(line, "%15s %d %d %d %d %d %d %d %d %d", set, &a[0], &a[1], &a[2], &a[3], &a[4], &a[5], &a[6],
+                    &a[7], &a[8]) != 10 ||
+        std::strcmp(set, kTuneSet) != 0)
+      continue;
     char b[128];
     snprintf(b, sizeof(b), "%d %d %d %d %d %d %d", a[0], a[1], a[2], a[3], a[4], a[5], a[6]);
     if (a[7] >= 0 && a[7] <= 4) g_tune[b] = {a[7], a[8]};
@@ -1338,7 +1346,7 @@ void tune_store(const std::string& key, int colw, int fused) {
   if (!f) return;
   FILE* fp = std::fopen(f, "a");
   if (!fp) return;
-  std::fprintf(fp, "%s %d %d\n", key.c_str(), colw, fused);
+  std::fprintf(fp, "%s %s %d %d\n", kTuneSet, key.c_str(), colw, fused);
   std::fclose(fp);
 }
 }  // namespace

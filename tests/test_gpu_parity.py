@@ -591,6 +591,35 @@ def test_batch_of_the_three_scan_shapes_matches_oracle(T, precision):
         p.close()
 
 
+def test_tuning_file_of_another_kernel_set_is_not_taken(T, tmp_path):
+    """A line without the kernel set (as builds wrote it whose default was another kernel) does not decide:
+    the shape is timed and a line of this set appended, which the next process takes without timing."""
+    import os
+    import subprocess
+    import sys
+    script = """
+import sys, torch
+sys.path.insert(0, sys.argv[1])
+from paper_1809_04195_gb300 import t2sh as T
+d = T.make_dims(64, 48, 4, 8, 4, nslices=1, block=8, lam=0.01, iters=4, seed=1)
+phi = torch.eye(8, 4, device="cuda").contiguous()
+with T.Plan(d, phi, torch.ones((8, 64, 48), dtype=torch.uint8, device="cuda"),
+            torch.ones((1, 4, 1, 64, 48), dtype=torch.complex64, device="cuda")) as p:
+    print(*p.autotune(2))
+"""
+    f = tmp_path / "tune"
+    shape = "64 48 4 4 1 8 0"
+    f.write_text(f"{shape} 1 1\nil1 64 48\nother {shape} 2 1\n")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    run = lambda: subprocess.run([sys.executable, "-c", script, root], env=dict(os.environ, T2SH_TUNE_CACHE=str(f)),  # noqa: E731
+                                 capture_output=True, text=True, check=True).stdout.split()
+    var, fused = run()
+    lines = f.read_text().splitlines()
+    assert len(lines) == 4 and lines[3].split()[1:8] == shape.split() and lines[3].split()[8:] == [var, str(int(fused == "True"))]
+    f.write_text("\n".join(lines[:3]) + "\n" + lines[3][:-3] + "4 1\n")   # another choice: taken as it stands
+    assert run() == ["4", "True"] and len(f.read_text().splitlines()) == 4
+
+
 def test_autotuned_plan_still_matches_oracle(T):
     sh = synth.SINGLE_SLICE_64x48
     phi, mask, maps, y = te_case(sh)
