@@ -128,7 +128,7 @@ t2sh_status t2sh_plan(const t2sh_dims* dims, const float* phi, const uint8_t* ma
 t2sh_status t2sh_destroy(t2sh_plan_t plan);
 
 /* t2sh_release_cached -- return the pool's unused memory on the current device to the
- * device (memory of live plans stays).  Errors: ECUDA. */
+ * device (memory of live plans stays), that of the pre-processing calls included.  Errors: ECUDA. */
 t2sh_status t2sh_release_cached(void);
 
 /*
@@ -253,7 +253,9 @@ t2sh_status t2sh_wavelet_denoise(t2sh_plan_t plan, void* alpha, float tau, int32
  * holds the channels [nchan][nx] of phase encode (ky[j], kz[j]) at echo t[j]; every axis
  * has its DC sample at index n/2.  The index arrays are host memory (read during the
  * call); line data and results are device memory.  Both calls are plan-free; their
- * scratch is allocated and freed in stream order on `stream`.
+ * scratch is allocated and freed in stream order on `stream`.  Up to 1 GiB of it stays in the
+ * library's pool for the next call or plan, until t2sh_release_cached; what goes beyond returns to
+ * the device at the next synchronisation.
  */
 typedef struct {
   int32_t nlines, nchan, nx, ny, nz, nechoes;

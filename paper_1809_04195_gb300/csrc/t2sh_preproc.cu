@@ -73,20 +73,24 @@ void build_groups(const t2sh_sparse* sp, int y0, int z0, int ny, int nz, Groups&
     }
 }
 
-// Stream-ordered scratch from the library's pool (which keeps its memory between calls, so a call
-// maps no fresh pages), freed in stream order.  Host tables are packed into one buffer and cross
-// in one copy.
+// Stream-ordered scratch, freed in stream order.  The first kKeepScratch bytes of a call come from the
+// library's pool, which keeps them for the next call or plan (t2sh_release_cached returns them), so that
+// most calls map no fresh pages: the Table I scan (0.6 GB) 2.3 ms, 3.6 with the device's default pool, which
+// gives its memory back at the next synchronisation.  What goes beyond comes from that one, so a call leaves no
+// more than that behind.  Host tables are packed into one buffer and cross in one copy.
+constexpr size_t kKeepScratch = (size_t)1 << 30;
 struct Scratch {
   cudaStream_t st;
+  size_t kept = 0;
   std::vector<void*> ptrs;
   std::vector<unsigned char> host;
   unsigned char* dev = nullptr;
-  explicit Scratch(cudaStream_t s) : st(s) {}
+  explicit Scratch(cudaStream_t s) : st(s) { ptrs.reserve(8); }
   template <typename T>
   cudaError_t alloc(T** p, size_t n) {
     void* q = nullptr;
     const size_t b = n ? n * sizeof(T) : 16;
-    cudaMemPool_t pool = library_pool();
+    cudaMemPool_t pool = b <= kKeepScratch - kept ? library_pool() : nullptr;
     cudaError_t e = pool ? cudaMallocFromPoolAsync(&q, b, pool, st) : cudaMallocAsync(&q, b, st);
     if (e != cudaSuccess && pool) {  // hand the pool's unused memory back and try once more
       cudaGetLastError();
@@ -95,8 +99,11 @@ struct Scratch {
       e = cudaMallocFromPoolAsync(&q, b, pool, st);
     }
     if (e == cudaSuccess) {
+      if (pool) kept += b;
       ptrs.push_back(q);
       *p = static_cast<T*>(q);
+    } else {
+      cudaGetLastError();  // reported here: not to be met again by the next launch
     }
     return e;
   }
@@ -142,17 +149,13 @@ t2sh_status t2sh_coil_compression(const t2sh_sparse* sp, const void* lines, int3
   if (window < 1 || window > sp->nx || window > sp->ny || window > sp->nz)
     return fail(T2SH_EINVAL, "window must be in [1, min(nx, ny, nz)]");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  Groups sg;
-  std::vector<int> wpix;  // sampled phase encodes of the window
   try {
+    Groups sg;
     build_groups(sp, sp->ny / 2 - window / 2, sp->nz / 2 - window / 2, window, window, sg);
+    std::vector<int> wpix;  // sampled phase encodes of the window
     for (int p = 0; p < window * window; ++p)
       if (sg.off[p + 1] > sg.off[p]) wpix.push_back(p);
-  } catch (const std::bad_alloc&) {
-    return fail(T2SH_ENOMEM, "host allocation failed");
-  }
-  if (wpix.empty()) return fail(T2SH_EINVAL, "no line falls in the calibration window");
-  {
+    if (wpix.empty()) return fail(T2SH_EINVAL, "no line falls in the calibration window");
     Scratch sc(st);
     int* err = nullptr;
     float2* X = nullptr;
@@ -172,6 +175,8 @@ t2sh_status t2sh_coil_compression(const t2sh_sparse* sp, const void* lines, int3
     PP_CK(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st));
     PP_CK(cudaStreamSynchronize(st));
     if (herr) return fail(T2SH_ECUDA, "the channel eigendecomposition did not converge");
+  } catch (const std::bad_alloc&) {
+    return fail(T2SH_ENOMEM, "host allocation failed");
   }
   return T2SH_OK;
 }
@@ -187,18 +192,14 @@ t2sh_status t2sh_preprocess(const t2sh_sparse* sp, const void* lines, const void
   FftPlan px{};
   if (!fft_plan_for(sp->nx, px)) return fail(T2SH_EINVAL, "no radix plan for nx");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  Groups sg;
   try {
+    Groups sg;
     build_groups(sp, 0, 0, sp->ny, sp->nz, sg);
-  } catch (const std::bad_alloc&) {
-    return fail(T2SH_ENOMEM, "host allocation failed");
-  }
-  std::vector<float2> tw(sp->nx);
-  for (int m = 0; m < sp->nx; ++m) {
-    const double a = -2.0 * 3.14159265358979323846 * m / sp->nx;
-    tw[m] = make_float2((float)std::cos(a), (float)std::sin(a));
-  }
-  {
+    std::vector<float2> tw(sp->nx);
+    for (int m = 0; m < sp->nx; ++m) {
+      const double a = -2.0 * 3.14159265358979323846 * m / sp->nx;
+      tw[m] = make_float2((float)std::cos(a), (float)std::sin(a));
+    }
     Scratch sc(st);
     float2* yh = nullptr;
     const size_t n = sp->nlines;
@@ -214,6 +215,8 @@ t2sh_status t2sh_preprocess(const t2sh_sparse* sp, const void* lines, const void
                                phi, nbasis, sp->ny, sp->nz, static_cast<float2*>(ytil_out), st));
     PP_CK(launch_mark_mask(sc.table<int>(a_t), sc.table<int>(a_ky), sc.table<int>(a_kz), sp->nlines, sp->ny, sp->nz,
                            mask_out, st));
+  } catch (const std::bad_alloc&) {
+    return fail(T2SH_ENOMEM, "host allocation failed");
   }
   return T2SH_OK;
 }

@@ -1,7 +1,9 @@
 """CPU checks of the C ABI: the library loads, exports every function that
 include/t2sh.h declares, and its host-only entry points behave (no GPU calls)."""
 import ctypes
+import os
 import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -159,6 +161,29 @@ def test_mixed_precision_dims_accepted(lib):
     n = ctypes.c_size_t(0)
     assert lib.t2sh_workspace_bytes(ctypes.byref(d), ctypes.byref(n)) == t2sh.OK
     assert n.value == t2sh.workspace_bytes(t2sh.make_dims(256, 160, 12, 80, 4, nslices=2, block=8, iters=10))
+
+
+def test_preprocess_reports_a_failed_host_allocation(lib):
+    """The packed host tables are the first allocation that no longer fits: a status, not an exception."""
+    script = """
+import ctypes, resource, sys
+sys.path.insert(0, sys.argv[1])
+import numpy as np
+from paper_1809_04195_gb300 import t2sh
+L = t2sh.lib()
+n = 8 << 20
+z = np.zeros(n, np.int32)
+z.ctypes.data_as(ctypes.POINTER(ctypes.c_int32))
+p = z.ctypes.data_as(ctypes.POINTER(ctypes.c_int32))
+sp = t2sh.Sparse(n, 4, 48, 64, 48, 8, p, p, p)
+vm = int(open("/proc/self/statm").read().split()[0]) * resource.getpagesize()
+resource.setrlimit(resource.RLIMIT_AS, (vm + (110 << 20),) * 2)   # the grouping takes 64 MB, the tables 160
+some = ctypes.c_void_p(256)   # never read: the call ends on the host
+print(L.t2sh_preprocess(ctypes.byref(sp), some, some, 2, some, 2, some, some, None))
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", script, root], capture_output=True, text=True)
+    assert r.returncode == 0 and int(r.stdout) == t2sh.ENOMEM, (r.returncode, r.stdout, r.stderr[-400:])
 
 
 def test_null_arguments_rejected(lib):

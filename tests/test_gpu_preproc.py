@@ -159,3 +159,24 @@ def test_preprocess_rejects_bad_input(T):
     with pytest.raises(T.T2shError):   # nx = 14 = 2 * 7 is not a product of 2, 3, 5, 13
         l14 = c64(lines[:, :, :14].copy())
         T.preprocess(l14, t, a, b, c64(np.eye(4, 2)), phi, 8, 8)
+
+
+@pytest.mark.parametrize("nlines,big", [(2000, False), (60000, True)])
+def test_scratch_kept_after_a_call_is_bounded(T, nlines, big):
+    """Up to 1 GiB of the scratch stays in the library's pool until release_cached; a call that needs more
+    leaves no more than that behind."""
+    nx, ncomp, ny, nz = 256, 12, 48, 48
+    lines = torch.zeros((nlines, ncomp, nx), dtype=torch.complex64, device="cuda")
+    idx = [np.zeros(nlines, np.int32)] * 3
+    w = torch.eye(ncomp, dtype=torch.complex64, device="cuda")
+    phi = torch.ones((4, 1), device="cuda")
+    assert (nlines * ncomp * nx * 8 > 2 ** 30) == big
+    torch.cuda.synchronize()
+    T.release_cached()
+    free0, torch0 = torch.cuda.mem_get_info()[0], torch.cuda.memory_reserved()
+    T.preprocess(lines, *idx, w, phi, ny, nz)
+    torch.cuda.synchronize()
+    kept = lambda: free0 - torch.cuda.mem_get_info()[0] - (torch.cuda.memory_reserved() - torch0)  # noqa: E731
+    assert kept() <= 2 ** 30 + (64 << 20)
+    T.release_cached()
+    assert kept() <= 64 << 20
