@@ -409,7 +409,7 @@ __device__ __forceinline__ void fft_lines(float2* buf, int ld, int nbatch, const
 }
 
 // ---------------------------------------------------------------------------------
-// Cyclic Jacobi eigensolver for a Hermitian K x K matrix, real type T.  On entry
+// Jacobi eigensolver for a Hermitian K x K matrix (herm_jacobi_rounds below), real type T.  On entry
 // (ar, ai) hold the full matrix; on exit the diagonal of ar holds the eigenvalues and
 // (vr, vi) the eigenvectors as columns.  Each rotation first makes a_pq real with a
 // diagonal phase, then applies the real Jacobi rotation with tan(theta) the smaller
@@ -431,91 +431,6 @@ __device__ __forceinline__ double jac_rsqrt(double x) { return 1.0 / sqrt(x); }
 __device__ __forceinline__ float jac_rcp(float x) { return __frcp_rn(x); }
 __device__ __forceinline__ double jac_rcp(double x) { return 1.0 / x; }
 
-template <typename T, int K>
-__device__ __forceinline__ void herm_jacobi(T (&ar)[K][K], T (&ai)[K][K], T (&vr)[K][K], T (&vi)[K][K],
-                                            int max_sweeps) {
-#pragma unroll
-  for (int i = 0; i < K; ++i)
-#pragma unroll
-    for (int j = 0; j < K; ++j) {
-      vr[i][j] = (i == j) ? T(1) : T(0);
-      vi[i][j] = T(0);
-    }
-  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-    T off = 0, diag = 0;
-#pragma unroll
-    for (int p = 0; p < K; ++p) {
-      diag += ar[p][p] * ar[p][p];
-#pragma unroll
-      for (int q = p + 1; q < K; ++q) off += ar[p][q] * ar[p][q] + ai[p][q] * ai[p][q];
-    }
-    if (!(off > JacobiTol<T>::rel2 * diag)) break;
-#pragma unroll
-    for (int p = 0; p < K - 1; ++p) {
-#pragma unroll
-      for (int q = p + 1; q < K; ++q) {
-        const T xr = ar[p][q], xi = ai[p][q];
-        const T r2 = xr * xr + xi * xi;
-        if (r2 > JacobiTol<T>::pivot2) {
-          const T ir = jac_rsqrt(r2), r = r2 * ir;
-          // phase: column q *= d, row q *= conj(d), d = conj(a_pq) / |a_pq|
-          const T dr = xr * ir, di = -xi * ir;
-#pragma unroll
-          for (int k = 0; k < K; ++k) {
-            if (k != q) {
-              const T yr = ar[k][q] * dr - ai[k][q] * di;
-              const T yi = ar[k][q] * di + ai[k][q] * dr;
-              ar[k][q] = yr; ai[k][q] = yi;
-              ar[q][k] = yr; ai[q][k] = -yi;
-            }
-          }
-#pragma unroll
-          for (int k = 0; k < K; ++k) {
-            const T yr = vr[k][q] * dr - vi[k][q] * di;
-            const T yi = vr[k][q] * di + vi[k][q] * dr;
-            vr[k][q] = yr; vi[k][q] = yi;
-          }
-          // a_pq is now the real r: real rotation on rows/columns p, q
-          const T theta = (ar[q][q] - ar[p][p]) * (T(0.5) * ir);
-          const T at = fabs(theta);
-          T t;
-          if (at > T(1e18)) {  // theta^2 would overflow float32: t = 1 / (2 |theta|) to first order
-            t = T(0.5) / at;
-          } else {
-            const T u = at * at + T(1);
-            t = jac_rcp(at + u * jac_rsqrt(u));
-          }
-          if (theta < T(0)) t = -t;
-          const T c = jac_rsqrt(t * t + T(1));
-          const T s = t * c;
-          ar[p][p] -= t * r;
-          ar[q][q] += t * r;
-          ar[p][q] = T(0); ar[q][p] = T(0);
-          ai[p][q] = T(0); ai[q][p] = T(0);
-#pragma unroll
-          for (int k = 0; k < K; ++k) {
-            if (k != p && k != q) {
-              const T akp_r = ar[k][p], akp_i = ai[k][p];
-              const T akq_r = ar[k][q], akq_i = ai[k][q];
-              const T nkp_r = c * akp_r - s * akq_r, nkp_i = c * akp_i - s * akq_i;
-              const T nkq_r = s * akp_r + c * akq_r, nkq_i = s * akp_i + c * akq_i;
-              ar[k][p] = nkp_r; ai[k][p] = nkp_i; ar[p][k] = nkp_r; ai[p][k] = -nkp_i;
-              ar[k][q] = nkq_r; ai[k][q] = nkq_i; ar[q][k] = nkq_r; ai[q][k] = -nkq_i;
-            }
-          }
-#pragma unroll
-          for (int k = 0; k < K; ++k) {
-            const T vkp_r = vr[k][p], vkp_i = vi[k][p];
-            const T vkq_r = vr[k][q], vkq_i = vi[k][q];
-            vr[k][p] = c * vkp_r - s * vkq_r; vi[k][p] = c * vkp_i - s * vkq_i;
-            vr[k][q] = s * vkp_r + c * vkq_r; vi[k][q] = s * vkp_i + c * vkq_i;
-          }
-        }
-      }
-    }
-  }
-}
-
 // Round-robin (tournament) ordering of the K (K - 1) / 2 index pairs of an even K into
 // K - 1 rounds of K / 2 disjoint pairs: in round r, i < K - 1 meets j = (r - i) mod (K - 1),
 // and the i with j = i meets K - 1.
@@ -532,11 +447,10 @@ __host__ __device__ constexpr int jac_pair(int K, int r, int m, bool second) {
   return 0;
 }
 
-// The same Jacobi method with each sweep taken as K - 1 rounds of K / 2 disjoint pivots
-// (the parallel ordering): a round's rotations act on disjoint rows and columns, so they
-// commute and their parameters all come from the matrix before the round.  One thread
-// then works on K / 2 independent rotations at a time instead of one dependent chain.
-// Same interface and stopping rule as herm_jacobi; K even.
+// Each sweep is K - 1 rounds of K / 2 disjoint pivots (the parallel ordering): a round's
+// rotations act on disjoint rows and columns, so they commute and their parameters all come
+// from the matrix before the round.  One thread then works on K / 2 independent rotations at a
+// time instead of one dependent chain.  K even.
 template <typename T, int K>
 __device__ __forceinline__ void herm_jacobi_rounds(T (&ar)[K][K], T (&ai)[K][K], T (&vr)[K][K], T (&vi)[K][K],
                                                    int max_sweeps) {
