@@ -28,8 +28,7 @@ sys.path.insert(0, ROOT)
 
 METRIC = "slice-iterations/s (T2 Shuffling FISTA PICS solve, full scan)"
 UNIT = "slice-iter/s"
-KERNEL_FILES = ["t2sh_device.cuh", "t2sh_plan.h", "k_fft.cu", "k_fft_fast.cu", "k_col_tma.cu", "k_col_il.cuh", "k_row_il.cuh", "k_any.cu", "k_col_pr.cu", "k_fused.cu", "k_llr.cu",
-                "k_prep.cu", "t2sh_api.cu"]
+CSRC = os.path.join(ROOT, "paper_1809_04195_gb300", "csrc")
 
 
 def parse():
@@ -331,9 +330,10 @@ def measured_peaks():
 
 def kernel_source_sha1():
     h = hashlib.sha1()
-    for f in KERNEL_FILES:
-        with open(os.path.join(ROOT, "paper_1809_04195_gb300", "csrc", f), "rb") as fh:
-            h.update(fh.read())
+    for f in sorted(os.listdir(CSRC)):
+        if f.endswith((".cu", ".cuh", ".h")):
+            with open(os.path.join(CSRC, f), "rb") as fh:
+                h.update(f.encode() + b"\0" + fh.read())
     return h.hexdigest()
 
 

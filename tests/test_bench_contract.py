@@ -75,6 +75,24 @@ def test_cpu_sample_is_seeded_distinct_and_stable():
     assert bench.shape_by_name(bench.shape_name(synth.PAPER_288x260x240)) is synth.PAPER_288x260x240
 
 
+def test_every_kernel_source_counts_for_the_recorded_traffic(tmp_path, monkeypatch):
+    """The traffic record holds for the sources it was taken on: a change of any of them ends it."""
+    import shutil
+    from paper_1809_04195_gb300 import build
+    csrc = tmp_path / "csrc"
+    shutil.copytree(bench.CSRC, csrc)
+    monkeypatch.setattr(bench, "CSRC", str(csrc))
+    ref = bench.kernel_source_sha1()
+    names = sorted(f.name for f in csrc.iterdir())
+    assert set(build.SOURCES) | {"launch.h", "two_radix.h", "k_col_il.cuh", "k_row_il.cuh", "k_post_il.cuh"} <= set(names)
+    for f in names:
+        text = (csrc / f).read_bytes()
+        (csrc / f).write_bytes(text + b"\n")
+        assert bench.kernel_source_sha1() != ref, f
+        (csrc / f).write_bytes(text)
+    assert bench.kernel_source_sha1() == ref
+
+
 def test_batch3_config_names_the_three_scans():
     import t2sh_synth as synth
     c = bench.batch3_config(1)
