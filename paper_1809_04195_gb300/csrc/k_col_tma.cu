@@ -92,8 +92,7 @@ __global__ void __launch_bounds__(ColTma<N, W>::THREADS, ColTma<N, W>::MINB) k_c
   }
   for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = tw_g[i];
   __syncthreads();
-  pdl_wait();
-  pdl_trigger();
+  pdl_wait();  // and no early trigger: see row_fast_body
   int tile = blockIdx.x;
   if (threadIdx.x == 0 && tile < ntiles) {
     const int sc = tile / ntz, z0 = (tile - sc * ntz) * W;
@@ -261,8 +260,7 @@ __global__ void __launch_bounds__(ColTma<N, W>::THREADS, ColTma<N, W>::MINB) k_c
   }
   for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = tw_g[i];
   __syncthreads();
-  pdl_wait();
-  pdl_trigger();
+  pdl_wait();  // and no early trigger: see row_fast_body
   int tile = blockIdx.x;
   if (threadIdx.x == 0 && tile < ntiles) {
     const int sc = tile / ntz, z0 = (tile - sc * ntz) * W;

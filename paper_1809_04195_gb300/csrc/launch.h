@@ -1,7 +1,8 @@
 // Kernel launches that may start before the previous kernel of the stream has ended (programmatic
 // stream serialisation).  The kernel runs its prologue (tables, barriers, plan-owned constants) and
 // then pdl_wait(), after which the previous kernels' results are visible; pdl_trigger() lets the next
-// such kernel do the same.  A kernel triggers only after its own wait, so whatever ran before the
+// such kernel do the same (without it that kernel starts when every CTA of this one has ended, which
+// still hides the launch itself).  A kernel triggers only after its own wait, so whatever ran before the
 // previous kernel has completed when a prologue runs.  What the previous kernel may have written is
 // not read-only while this one runs: an argument that is read after the wait and written by another
 // kernel carries no `__restrict__` (its loads could be hoisted above the wait, and a `const` one's
