@@ -269,12 +269,14 @@ __global__ void __launch_bounds__(kThreads) k_project(Geom g, TLayout lt, const 
 // times the input): one thread owns two neighbouring points and writes 16 bytes per echo, whole
 // 512-byte runs per warp, so it is bound by HBM writes.  256x160, C = 12, T = 80, 8 slices
 // (2.5 GB): 400 us, 0.93 of the measured copy bandwidth; 745 us when the column pass wrote the
-// echoes itself in 64-byte runs, 445 us with the column pass now.  WIDE: y is 16-byte aligned; an
+// echoes itself in 64-byte runs, 445 us with the column pass now.  Where the points and planes give an SM
+// fewer than eight CTAs, the echoes are shared out too, in chunks of 32 down to 8 (blockIdx.z): A x of one
+// slice of 64x48, K = 4, C = 8, T = 32 10.0 -> 9.0 us, of 260x240, M = 2, C = 7, T = 80 64 -> 56 us.  WIDE: y is 16-byte aligned; an
 // array that starts at an odd value of another takes 8-byte stores.
 template <int KC, bool WIDE>
 __global__ void __launch_bounds__(kThreads) k_expand_te(Geom g, TLayout lt, const float* __restrict__ phi,
                                                       const unsigned* __restrict__ bits,
-                                                      const float2* v, float2* __restrict__ y) {
+                                                      const float2* v, float2* __restrict__ y, int tc) {
   extern __shared__ float sphi[];
   for (int i = threadIdx.x; i < g.T * g.K; i += blockDim.x) sphi[i] = phi[i];
   __syncthreads();
@@ -284,16 +286,19 @@ __global__ void __launch_bounds__(kThreads) k_expand_te(Geom g, TLayout lt, cons
   const int n = 2 * (blockIdx.x * blockDim.x + threadIdx.x);  // nz is even: both points share a row
   if (n >= N) return;
   const long long nsc = (long long)g.S * g.C;
+  const int tlo = blockIdx.z * tc, thi = min(g.T, tlo + tc);  // this CTA's echoes
   for (long long sc = blockIdx.y; sc < nsc; sc += gridDim.y) {
     const TePlace pl(g, lt, sc, n);
     float4 a[KC];
 #pragma unroll
     for (int k = 0; k < KC; ++k)
       a[k] = k < g.K ? *reinterpret_cast<const float4*>(v + pl.at(k)) : make_float4(0.f, 0.f, 0.f, 0.f);
-    float2* yb = y + sc * g.T * (long long)N + n;
-    for (int t0 = 0; t0 < g.T; t0 += 32) {
+    float2* yb = y + (sc * g.T + tlo) * (long long)N + n;
+    for (int t0 = tlo; t0 < thi; t0 += 32) {  // tc is a multiple of 32 or divides it: no chunk leaves its word
       uint2 b = *reinterpret_cast<const uint2*>(bits + (long long)(t0 >> 5) * N + n);
-      const int m = min(32, g.T - t0);
+      b.x >>= t0 & 31;
+      b.y >>= t0 & 31;
+      const int m = min(32, thi - t0);
 #pragma unroll 4
       for (int i = 0; i < m; ++i) {
         float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -373,12 +378,18 @@ cudaError_t launch_expand_te(const Geom& g, const TLayout& lt, const float* phi,
                              float2* y_te, cudaStream_t st) {
   const int N2 = g.ny * g.nz / 2;
   const long long nsc = (long long)g.S * g.C;
-  dim3 grid((N2 + kThreads - 1) / kThreads, (unsigned)(nsc < 65535 ? nsc : 65535));
+  int nsm = 0;
+  const cudaError_t e = sm_count(&nsm);
+  if (e != cudaSuccess) return e;
+  const long long ctas = (long long)((N2 + kThreads - 1) / kThreads) * nsc;
+  int tc = (g.T + 31) / 32 * 32;
+  while (tc > 8 && ctas * ((g.T + tc - 1) / tc) < 8LL * nsm) tc = tc > 32 ? 32 : tc / 2;
+  dim3 grid((N2 + kThreads - 1) / kThreads, (unsigned)(nsc < 65535 ? nsc : 65535), (g.T + tc - 1) / tc);
   const size_t sm = sizeof(float) * g.T * g.K;
   const bool wide = ((uintptr_t)y_te & 15) == 0;
   auto kern = g.K <= 4 ? (wide ? k_expand_te<4, true> : k_expand_te<4, false>)
                        : (wide ? k_expand_te<8, true> : k_expand_te<8, false>);
-  return launch_pdl(kern, grid, kThreads, sm, st, g, lt, phi, bits, v, y_te);
+  return launch_pdl(kern, grid, kThreads, sm, st, g, lt, phi, bits, v, y_te, tc);
 }
 
 }  // namespace t2sh

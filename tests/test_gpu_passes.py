@@ -54,6 +54,9 @@ def test_passes_of_four_images(T, S, ny, nz, C, M):  # noqa: F811
     (1, 192, 240, 2, 4, 4, 1),    # as few echoes as images
     (2, 60, 36, 3, 40, 3, 1),     # planar intermediate, K < 4
     (1, 30, 50, 2, 65, 6, 2),     # K > 4
+    (1, 16, 24, 1, 7, 4, 1),      # echoes shared out over CTAs: fewer than a chunk,
+    (1, 64, 48, 2, 41, 4, 1),     # chunks that end in the second word,
+    (3, 256, 160, 8, 40, 4, 1),   # chunks of 32
 ])
 def test_per_echo_and_projected_forms(T, S, ny, nz, C, Tn, K, M):  # noqa: F811
     rng, phi, mask, maps = random_problem(ny + nz + Tn, S, ny, nz, C, Tn, K, M)
