@@ -243,10 +243,12 @@ __global__ void __launch_bounds__(kFftThreads, 1) k_col_normal(Geom g, FftPlan p
   cp_async_wait<0>();
 }
 
-// Column pass.  tin/tout are [S][C][K][ny][nz] (may alias).
+// Column pass.  tin/tout are [S][C][K][ny][nz] (may alias); COL_FWD_TE writes per-echo k-space
+// [S][C][T][ny][nz] to tout.
 template <int MODE, int KC, bool R13>
 __global__ void __launch_bounds__(kFftThreads) k_col(Geom g, FftPlan py, const float2* __restrict__ tw_g,
-                                                const float* __restrict__ psi, const float2* tin, float2* tout,
+                                                const float* __restrict__ psi, const float* __restrict__ phi,
+                                                const unsigned* __restrict__ bits, const float2* tin, float2* tout,
                                                 int W) {
   extern __shared__ float2 smem[];
   const int ny = g.ny, nz = g.nz, N = ny * nz, K = g.K;
@@ -314,6 +316,34 @@ __global__ void __launch_bounds__(kFftThreads) k_col(Geom g, FftPlan py, const f
       __syncthreads();
       if (MODE == COL_FWD_PROJ) return;
       fft_lines<true, R13>(buf, ld, K * wc, py, tw);
+    } else if (MODE == COL_FWD_TE) {
+      for (int q = threadIdx.x; q < npt; q += kFftThreads) {
+        const int w = q % wc, y = q / wc;
+        const long long n = (long long)y * nz + z0 + w;
+        const float sg = g.gsign * g.inv_sqrt_n * parity_sign(y + z0 + w);
+        float2 v[KC];
+#pragma unroll
+        for (int k = 0; k < KC; ++k) v[k] = (k < K) ? cscale(buf[(k * wc + w) * ld + y], sg) : make_float2(0.f, 0.f);
+        float2* yb = tout + ((long long)(s * g.C + c) * g.T) * N + n;
+        for (int t0 = 0; t0 < g.T; t0 += 32) {
+          const unsigned word = bits[(long long)(t0 >> 5) * N + n];
+          const int m = min(32, g.T - t0);
+          for (int i = 0; i < m; ++i) {
+            float2 a = make_float2(0.f, 0.f);
+            if ((word >> i) & 1u) {
+#pragma unroll
+              for (int k = 0; k < KC; ++k)
+                if (k < K) {
+                  const float ph = __ldg(phi + (t0 + i) * K + k);
+                  a.x = fmaf(ph, v[k].x, a.x);
+                  a.y = fmaf(ph, v[k].y, a.y);
+                }
+            }
+            yb[(long long)(t0 + i) * N] = a;
+          }
+        }
+      }
+      return;
     }
   }
   // store the columns back (COL_NORMAL, COL_ADJ_DATA, COL_FWD_RAW)
@@ -385,6 +415,13 @@ TLayout t_layout(const Geom& g) {
   return lt;
 }
 
+// A x per echo on the planar layout in one pass of the columns, instead of transforming in place and writing
+// the echoes in a pass of their own: short columns (their CTAs write long enough runs) and few echoes per
+// image.  64x338, K = 4, C = 15, T = 30, 9 slices 434 us against 509, 90x512, K = 2, C = 8, T = 22, 3 slices 166
+// against 173, 48x96, K = 1, C = 11, T = 54, 2 slices 27 against 31; 64x338, K = 2, C = 7, T = 85, 10 slices 378
+// against 300; 80x160, K = 1, C = 9, T = 76 50 against 43; 512x192, K = 6, T = 16 782 against 693.
+bool fwd_te_in_one_pass(const Geom& g) { return g.K <= 4 && g.ny <= 96 && g.T * g.ny <= (g.K == 1 ? 3300 : 1280 * g.K); }
+
 cudaError_t launch_col_t(const Geom& g, const TLayout& lt, IlPass pass, const float2* tw_y, const float* psi,
                          const float2* in, float2* out, cudaStream_t st) {
   return lt.col_il ? launch_col_il(g, pass, tw_y, psi, in, out, st)
@@ -412,8 +449,8 @@ cudaError_t launch_row(const Geom& g, RowMode mode, const TLayout& lt, const Fft
 }
 
 template <int MODE, int KC, bool R13>
-static cudaError_t col_go13(const Geom& g, const FftPlan& py, const float2* tw, const float* psi,
-                            const float2* tin, float2* tout, cudaStream_t st) {
+static cudaError_t col_go13(const Geom& g, const FftPlan& py, const float2* tw, const float* psi, const float* phi,
+                            const unsigned* bits, const float2* tin, float2* tout, cudaStream_t st) {
   const int W = col_cols_per_cta(g);
   const size_t sm = sizeof(float2) * (((g.ny + 1) & ~1) + (size_t)g.K * W * (g.ny + 1));
   {
@@ -421,15 +458,15 @@ static cudaError_t col_go13(const Geom& g, const FftPlan& py, const float2* tw, 
     if (e != cudaSuccess) return e;
   }
   dim3 grid((g.nz + W - 1) / W, g.C, g.S);
-  k_col<MODE, KC, R13><<<grid, kFftThreads, sm, st>>>(g, py, tw, psi, tin, tout, W);
+  k_col<MODE, KC, R13><<<grid, kFftThreads, sm, st>>>(g, py, tw, psi, phi, bits, tin, tout, W);
   return cudaGetLastError();
 }
 
 template <int MODE, int KC>
-static cudaError_t col_go(const Geom& g, const FftPlan& py, const float2* tw, const float* psi,
-                          const float2* tin, float2* tout, cudaStream_t st) {
-  return plan_has13(py) ? col_go13<MODE, KC, true>(g, py, tw, psi, tin, tout, st)
-                        : col_go13<MODE, KC, false>(g, py, tw, psi, tin, tout, st);
+static cudaError_t col_go(const Geom& g, const FftPlan& py, const float2* tw, const float* psi, const float* phi,
+                          const unsigned* bits, const float2* tin, float2* tout, cudaStream_t st) {
+  return plan_has13(py) ? col_go13<MODE, KC, true>(g, py, tw, psi, phi, bits, tin, tout, st)
+                        : col_go13<MODE, KC, false>(g, py, tw, psi, phi, bits, tin, tout, st);
 }
 
 template <int KC, bool R13>
@@ -461,7 +498,7 @@ static cudaError_t col_normal_go(const Geom& g, const FftPlan& py, const float2*
 }
 
 cudaError_t launch_col(const Geom& g, ColMode mode, const FftPlan& py, const float2* tw_y, const float* psi,
-                       const float2* tin, float2* tout, cudaStream_t st) {
+                       const float* phi, const unsigned* bits, const float2* tin, float2* tout, cudaStream_t st) {
   const bool k4 = g.K <= 4;
   switch (mode) {
     case COL_NORMAL:
@@ -485,14 +522,17 @@ cudaError_t launch_col(const Geom& g, ColMode mode, const FftPlan& py, const flo
       const cudaError_t et = launch_col_adj_tma(g, tw_y, tin, tout, st);
       if (et != cudaErrorNotSupported) return et;
     }
-      return k4 ? col_go<COL_ADJ_DATA, 4>(g, py, tw_y, psi, tin, tout, st)
-                : col_go<COL_ADJ_DATA, 8>(g, py, tw_y, psi, tin, tout, st);
+      return k4 ? col_go<COL_ADJ_DATA, 4>(g, py, tw_y, psi, phi, bits, tin, tout, st)
+                : col_go<COL_ADJ_DATA, 8>(g, py, tw_y, psi, phi, bits, tin, tout, st);
     case COL_FWD_PROJ:
-      return k4 ? col_go<COL_FWD_PROJ, 4>(g, py, tw_y, psi, tin, tout, st)
-                : col_go<COL_FWD_PROJ, 8>(g, py, tw_y, psi, tin, tout, st);
+      return k4 ? col_go<COL_FWD_PROJ, 4>(g, py, tw_y, psi, phi, bits, tin, tout, st)
+                : col_go<COL_FWD_PROJ, 8>(g, py, tw_y, psi, phi, bits, tin, tout, st);
     case COL_FWD_RAW:
-      return k4 ? col_go<COL_FWD_RAW, 4>(g, py, tw_y, psi, tin, tout, st)
-                : col_go<COL_FWD_RAW, 8>(g, py, tw_y, psi, tin, tout, st);
+      return k4 ? col_go<COL_FWD_RAW, 4>(g, py, tw_y, psi, phi, bits, tin, tout, st)
+                : col_go<COL_FWD_RAW, 8>(g, py, tw_y, psi, phi, bits, tin, tout, st);
+    case COL_FWD_TE:
+      return k4 ? col_go<COL_FWD_TE, 4>(g, py, tw_y, psi, phi, bits, tin, tout, st)
+                : col_go<COL_FWD_TE, 8>(g, py, tw_y, psi, phi, bits, tin, tout, st);
   }
   return cudaErrorInvalidValue;
 }

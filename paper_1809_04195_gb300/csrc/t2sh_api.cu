@@ -387,7 +387,7 @@ t2sh_status normal_op(t2sh_plan_t p, const float2* x, float2* y) {
   {
     KTimer k(p, KC_COL);
     T2SH_CK(lt.W ? launch_col_t(p->g, lt, IL_NORMAL, p->tw_y, p->psi, p->t, p->t, p->st)
-               : launch_col(p->g, COL_NORMAL, p->py, p->tw_y, p->psi, p->t, p->t, p->st));
+               : launch_col(p->g, COL_NORMAL, p->py, p->tw_y, p->psi, nullptr, nullptr, p->t, p->t, p->st));
   }
   { KTimer k(p, KC_ROW_ADJ); T2SH_CK(launch_row(p->g, ROW_ADJ, lt, p->pz, p->tw_z, p->maps, nullptr, p->t, y, p->st)); }
   return T2SH_OK;
@@ -408,7 +408,7 @@ t2sh_status adjoint_data(t2sh_plan_t p, const void* y, int32_t kform, float2* x)
   {
     KTimer k(p, KC_COL);
     T2SH_CK(lt.W ? launch_col_t(p->g, lt, pass, p->tw_y, nullptr, proj, p->t, p->st)
-               : launch_col(p->g, COL_ADJ_DATA, p->py, p->tw_y, p->psi, proj, p->t, p->st));
+               : launch_col(p->g, COL_ADJ_DATA, p->py, p->tw_y, p->psi, nullptr, nullptr, proj, p->t, p->st));
   }
   { KTimer k(p, KC_ROW_ADJ); T2SH_CK(launch_row(p->g, ROW_ADJ, lt, p->pz, p->tw_z, p->maps, nullptr, p->t, x, p->st)); }
   return T2SH_OK;
@@ -644,8 +644,9 @@ t2sh_status t2sh_get_step(t2sh_plan_t p, float* step) {
 t2sh_status t2sh_forward(t2sh_plan_t p, const void* x, void* y, int32_t kform) {
   T2SH_REQ(p && x && y, "NULL argument");
   T2SH_REQ(kform == T2SH_KSPACE_TE || kform == T2SH_KSPACE_PROJ, "bad kform %d", kform);
-  const TLayout lt = t_layout(p->g);
   const bool te = kform == T2SH_KSPACE_TE;
+  const TLayout lt = t_layout(p->g);
+  const bool expand = te && (lt.W || !fwd_te_in_one_pass(p->g));
   float2* yo = static_cast<float2*>(y);
   { KTimer k(p, KC_ROW_FWD); T2SH_CK(launch_row(p->g, ROW_FWD, lt, p->pz, p->tw_z, p->maps, static_cast<const float2*>(x), p->t, nullptr, p->st)); }
   {
@@ -653,9 +654,10 @@ t2sh_status t2sh_forward(t2sh_plan_t p, const void* x, void* y, int32_t kform) {
     if (lt.W)
       T2SH_CK(launch_col_t(p->g, lt, te ? IL_FWD_RAW : IL_FWD_PROJ, p->tw_y, p->psi, p->t, te ? p->t : yo, p->st));
     else
-      T2SH_CK(launch_col(p->g, te ? COL_FWD_RAW : COL_FWD_PROJ, p->py, p->tw_y, p->psi, p->t, te ? p->t : yo, p->st));
+      T2SH_CK(launch_col(p->g, expand ? COL_FWD_RAW : te ? COL_FWD_TE : COL_FWD_PROJ, p->py, p->tw_y, p->psi, p->phi,
+                         p->bits, p->t, expand ? p->t : yo, p->st));
   }
-  if (te) {
+  if (expand) {
     KTimer k(p, KC_PROJ);
     T2SH_CK(launch_expand_te(p->g, lt, p->phi, p->bits, p->t, yo, p->st));
   }
@@ -764,7 +766,7 @@ t2sh_status iteration(t2sh_plan_t p) {
     // LLR, momentum and DFT_z(S z_{k+1}) for the next iteration (z_0 = 0: no A^H A z_0)
     if (it > 0) {
       KTimer k(p, KC_COL);
-      T2SH_CK(launch_col(p->g, COL_NORMAL, p->py, p->tw_y, p->psi, p->t, p->t, p->st));
+      T2SH_CK(launch_col(p->g, COL_NORMAL, p->py, p->tw_y, p->psi, nullptr, nullptr, p->t, p->t, p->st));
     }
     KTimer k(p, KC_BAND);
     T2SH_CK(launch_band_fused(p->g, a, p->tw_z, p->maps, p->t, p->x, p->z, p->aty, p->st));

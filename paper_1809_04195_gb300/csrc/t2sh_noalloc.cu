@@ -147,7 +147,7 @@ extern "C" t2sh_status t2sh_normal_op_noalloc(const t2sh_dims* dims, const float
   if (e == cudaSuccess) e = launch_row(g, ROW_FWD, lt, pz, tw_z, maps_s, static_cast<const float2*>(x), t, nullptr, st);
   if (e == cudaSuccess)
     e = lt.W ? launch_col_t(g, lt, IL_NORMAL, tw_y, psi, t, t, st)
-           : launch_col(g, COL_NORMAL, py, tw_y, psi, t, t, st);
+           : launch_col(g, COL_NORMAL, py, tw_y, psi, nullptr, nullptr, t, t, st);
   if (e == cudaSuccess) e = launch_row(g, ROW_ADJ, lt, pz, tw_z, maps_s, nullptr, t, static_cast<float2*>(y), st);
   if (e != cudaSuccess) {
     cudaGetLastError();

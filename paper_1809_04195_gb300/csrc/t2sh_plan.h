@@ -56,6 +56,7 @@ enum ColMode : int {
   COL_NORMAL = 0,    // DFT_y, Psi (pre-scaled by 1/N), IDFT_y                 (normal operator)
   COL_ADJ_DATA = 1,  // multiply by gsign (-1)^(ky+kz) / sqrt(N), IDFT_y          (A^H y)
   COL_FWD_PROJ = 2,  // DFT_y, multiply by gsign (-1)^(ky+kz) / sqrt(N), Psi * N  (Phi^T P A x)
+  COL_FWD_TE = 4,    // DFT_y, the same factor, P_t Phi of every echo                      (A x in one pass)
   COL_FWD_RAW = 3    // DFT_y, multiply by gsign (-1)^(ky+kz) / sqrt(N), in place  (A x before P_t Phi)
 };
 
@@ -111,8 +112,10 @@ cudaError_t launch_row(const Geom& g, RowMode mode, const TLayout& lt, const Fft
 // column pass on a chunked layout (lt.W > 0)
 cudaError_t launch_col_t(const Geom& g, const TLayout& lt, IlPass pass, const float2* tw_y, const float* psi,
                          const float2* in, float2* out, cudaStream_t st);
+// planar column pass; phi, bits: COL_FWD_TE only, which fwd_te_in_one_pass chooses
+bool fwd_te_in_one_pass(const Geom& g);
 cudaError_t launch_col(const Geom& g, ColMode mode, const FftPlan& py, const float2* tw_y, const float* psi,
-                       const float2* tin, float2* tout, cudaStream_t st);
+                       const float* phi, const unsigned* bits, const float2* tin, float2* tout, cudaStream_t st);
 struct PostArgs {
   int te[kMaxPostTe];
   int nte;

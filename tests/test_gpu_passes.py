@@ -90,6 +90,7 @@ def test_per_echo_and_projected_forms(T, S, ny, nz, C, Tn, K, M):  # noqa: F811
     (1, 300, 250, 2, 8, 1),   # eight images of 250-point rows: the three-stage passes
     (1, 512, 400, 1, 4, 1),
     (1, 250, 60, 3, 5, 1), (1, 500, 48, 2, 5, 2), (1, 450, 52, 1, 5, 1),  # 25 items of 20 threads: most threads a column CTA has
+    (1, 64, 338, 2, 4, 1), (1, 90, 512, 2, 2, 1), (1, 390, 16, 2, 2, 1),  # three radix stages: A x in one column pass, and in two
 ])
 def test_two_radix_passes(T, S, ny, nz, C, K, M):  # noqa: F811
     rng, phi, mask, maps = random_problem(ny * nz + K, S, ny, nz, C, 12, K, M)
