@@ -26,7 +26,19 @@
 #include "launch.h"
 #include "t2sh_device.cuh"
 
+#define T2SH_COL_TMA_LENGTHS(X) X(48) X(64) X(96) X(128) X(160) X(192) X(240) X(256) X(260)
+
 namespace t2sh {
+
+bool col_tma_length(int ny) {
+  switch (ny) {
+#define X(n) case n:
+    T2SH_COL_TMA_LENGTHS(X)
+#undef X
+    return true;
+    default: return false;
+  }
+}
 
 template <int N, int W>
 struct ColTma {
@@ -397,15 +409,9 @@ template <int W>
 cudaError_t col_tma_w(const Geom& g, const float2* tw_y, const float* psi, float2* t, cudaStream_t st) {
   if (g.K > 4 || g.nz % W != 0) return cudaErrorNotSupported;
   switch (g.ny) {
-    case 48: return col_tma_go<48, W>(g, tw_y, psi, t, st);
-    case 64: return col_tma_go<64, W>(g, tw_y, psi, t, st);
-    case 96: return col_tma_go<96, W>(g, tw_y, psi, t, st);
-    case 128: return col_tma_go<128, W>(g, tw_y, psi, t, st);
-    case 160: return col_tma_go<160, W>(g, tw_y, psi, t, st);
-    case 192: return col_tma_go<192, W>(g, tw_y, psi, t, st);
-    case 240: return col_tma_go<240, W>(g, tw_y, psi, t, st);
-    case 256: return col_tma_go<256, W>(g, tw_y, psi, t, st);
-    case 260: return col_tma_go<260, W>(g, tw_y, psi, t, st);
+#define X(n) case n: return col_tma_go<n, W>(g, tw_y, psi, t, st);
+    T2SH_COL_TMA_LENGTHS(X)
+#undef X
     default: return cudaErrorNotSupported;
   }
 }

@@ -12,6 +12,7 @@
 #include <algorithm>
 
 #include "t2sh_device.cuh"
+#include "two_radix.h"
 
 namespace t2sh {
 
@@ -397,15 +398,34 @@ static cudaError_t row_go(const Geom& g, const FftPlan& pz, const float2* tw, co
 // Chunked layouts serve the default column variant: the size-specialised passes of four basis
 // images where both lengths have them, the passes of k_any.cu for what they cover otherwise (the
 // two share a layout at K = 4, so one side may be specialised).  Planar: the other column
-// variants and lengths that need three radix stages.
-TLayout t_layout(const Geom& g) {
+// variants, lengths that need three radix stages, and fewer images where keep_planar says so.
+//
+// Fewer than four images on row lengths that the planar row pass has: its rows are faster than the
+// two-radix ones, its columns only at the nine lengths of k_col_tma.cu (elsewhere, and for A x at every
+// length, they are the Stockham passes), and the two-radix passes, which share a coil's columns and a band's
+// rows among fewer threads, need a launch that fills the chip, and more than one coil to spread a row's
+// set-up over.  Two-radix against planar passes, K = 1 to 3, 700 drawn calls:
+//   at the nine lengths A^H A and A^H 1.1 to 2.8 times slower, A x projected 0.5 to 1.3;
+//   at other lengths with 600 column tiles (four per SM), 1000 for A^H A with one or two images, 1500 for A^H (2500
+//   with one image), and 120 lines in all cases: 0.26 to 1.08; with fewer 0.6 to 1.8, with one coil up to 1.4, and A^H
+//   with radices of 20 and 25 up to 1.8.  180x160, K = 3, C = 10, 24 slices: A^H A 656 -> 414 us;
+//   A x per echo 0.3 to 1.05 at any length and size, but one image in small launches (1.6).
+// The tiles are those of the whole plan, so a slice's bits do not depend on the launch it is part of.
+static bool keep_planar(const Geom& g, TUse use) {
+  if (g.K >= 4 || g.nz % 8 != 0 || !row_fast_supported(g)) return false;
+  const long long tiles = (long long)g.Sp * g.C * (g.nz / 4), lines = (long long)g.Sp * g.ny * g.K;
+  if (use == USE_FWD_TE) return g.K == 1 && (tiles < 1500 || lines < 120);
+  const int least = use == USE_ADJ ? (g.K == 1 ? 2500 : 1500) : use == USE_NORMAL && g.K < 3 ? 1000 : 600;
+  if (col_tma_length(g.ny) || tiles < least || lines < 120 || g.C == 1) return true;
+  int ra = 0, rb = 0;
+  return use == USE_ADJ && (!two_radices(g.ny, kMaxRadix, false, &ra, &rb) || ra > 18 || rb > 18);
+}
+
+TLayout t_layout(const Geom& g, TUse use) {
   TLayout lt{};
-  if (g.colvar != 0) return lt;
+  if (g.colvar != 0 || keep_planar(g, use)) return lt;
   const long long nsc = (long long)g.S * g.C;
   const bool four = g.K == 4 && g.nz % 4 == 0;
-  // fewer images on lengths that the planar size-specialised passes have: those are 1.1 to 1.7
-  // times faster than the two-radix ones (256x160, C = 12, 16 slices, K = 3: 244 against 403 us)
-  if (g.K < 4 && g.nz % 8 == 0 && il_rb(g.ny) > 0 && row_fast_supported(g)) return lt;
   lt.col_il = four && il_rb(g.ny) > 0 && nsc * (std::max(g.ny, g.nz) + 1) <= 0x7fffffffLL && tma_encode_fn() != nullptr;
   lt.row_il = four && row_il_supported(g);
   if ((lt.col_il || any_col_supported(g)) && (lt.row_il || any_row_supported(g))) {
@@ -420,7 +440,9 @@ TLayout t_layout(const Geom& g) {
 // image.  64x338, K = 4, C = 15, T = 30, 9 slices 434 us against 509, 90x512, K = 2, C = 8, T = 22, 3 slices 166
 // against 173, 48x96, K = 1, C = 11, T = 54, 2 slices 27 against 31; 64x338, K = 2, C = 7, T = 85, 10 slices 378
 // against 300; 80x160, K = 1, C = 9, T = 76 50 against 43; 512x192, K = 6, T = 16 782 against 693.
-bool fwd_te_in_one_pass(const Geom& g) { return g.K <= 4 && g.ny <= 96 && g.T * g.ny <= (g.K == 1 ? 3300 : 1280 * g.K); }
+bool fwd_te_in_one_pass(const Geom& g) {
+  return g.K <= 4 && g.ny >= 48 && g.ny <= 96 && g.T * g.ny <= (g.K == 1 ? 3300 : 1280 * g.K);
+}
 
 cudaError_t launch_col_t(const Geom& g, const TLayout& lt, IlPass pass, const float2* tw_y, const float* psi,
                          const float2* in, float2* out, cudaStream_t st) {

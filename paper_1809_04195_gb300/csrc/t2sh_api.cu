@@ -382,7 +382,7 @@ enum { KC_ROW_FWD = 0, KC_ROW_ADJ = 1, KC_COL = 2, KC_LLR = 3, KC_PLAN = 4, KC_P
 namespace {
 
 t2sh_status normal_op(t2sh_plan_t p, const float2* x, float2* y) {
-  const TLayout lt = t_layout(p->g);
+  const TLayout lt = t_layout(p->g, USE_NORMAL);
   { KTimer k(p, KC_ROW_FWD); T2SH_CK(launch_row(p->g, ROW_FWD, lt, p->pz, p->tw_z, p->maps, x, p->t, nullptr, p->st)); }
   {
     KTimer k(p, KC_COL);
@@ -396,7 +396,7 @@ t2sh_status normal_op(t2sh_plan_t p, const float2* x, float2* y) {
 // A^H y for device k-space in either form, result in x.
 t2sh_status adjoint_data(t2sh_plan_t p, const void* y, int32_t kform, float2* x) {
   const float2* proj = static_cast<const float2*>(y);
-  const TLayout lt = t_layout(p->g);
+  const TLayout lt = t_layout(p->g, USE_ADJ);
   // per-echo data are projected into t itself, in the layout the column pass takes in place
   IlPass pass = IL_ADJ_PLANAR;
   if (kform == T2SH_KSPACE_TE) {
@@ -645,7 +645,7 @@ t2sh_status t2sh_forward(t2sh_plan_t p, const void* x, void* y, int32_t kform) {
   T2SH_REQ(p && x && y, "NULL argument");
   T2SH_REQ(kform == T2SH_KSPACE_TE || kform == T2SH_KSPACE_PROJ, "bad kform %d", kform);
   const bool te = kform == T2SH_KSPACE_TE;
-  const TLayout lt = t_layout(p->g);
+  const TLayout lt = t_layout(p->g, te ? USE_FWD_TE : USE_FWD_PROJ);
   const bool expand = te && (lt.W || !fwd_te_in_one_pass(p->g));
   float2* yo = static_cast<float2*>(y);
   { KTimer k(p, KC_ROW_FWD); T2SH_CK(launch_row(p->g, ROW_FWD, lt, p->pz, p->tw_z, p->maps, static_cast<const float2*>(x), p->t, nullptr, p->st)); }

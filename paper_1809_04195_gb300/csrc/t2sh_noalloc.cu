@@ -143,7 +143,7 @@ extern "C" t2sh_status t2sh_normal_op_noalloc(const t2sh_dims* dims, const float
   if (e == cudaSuccess) e = cudaMemsetAsync(red, 0, kHeader - kRedOff, st);
   if (e == cudaSuccess) e = launch_maps_prep(g, static_cast<const float2*>(maps), maps_s, red, st);
   if (e == cudaSuccess) e = launch_psi_build(g, phi, mask, psi, nullptr, red + 1, st);
-  const TLayout lt = t_layout(g);
+  const TLayout lt = t_layout(g, USE_NORMAL);
   if (e == cudaSuccess) e = launch_row(g, ROW_FWD, lt, pz, tw_z, maps_s, static_cast<const float2*>(x), t, nullptr, st);
   if (e == cudaSuccess)
     e = lt.W ? launch_col_t(g, lt, IL_NORMAL, tw_y, psi, t, t, st)

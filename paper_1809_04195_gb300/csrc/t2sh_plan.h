@@ -97,7 +97,9 @@ struct TLayout {
   int trb;              // slot of image k in row y: (k + y % trb + y / trb) % 4 (k_col_il.cuh); 0: k
   bool col_il, row_il;  // the size-specialised column / row passes serve it, else those of k_any.cu
 };
-TLayout t_layout(const Geom& g);
+// what t is made for: the layout may differ from one operator to the next
+enum TUse { USE_NORMAL, USE_ADJ, USE_FWD_PROJ, USE_FWD_TE };
+TLayout t_layout(const Geom& g, TUse use);
 // bits (nullable): the sampling pattern as bit words [ceil(T / 32)][ny][nz], bit i of word w for
 // echo 32 w + i; lam_bits: zero on entry
 cudaError_t launch_psi_build(const Geom& g, const float* phi, const uint8_t* mask, float* psi, unsigned* bits,
@@ -180,6 +182,7 @@ cudaError_t launch_llr_list(const LlrJob* jobs, int njobs, int units, bool kc8, 
 
 // size-specialised passes (k_fft_fast.cu); cudaErrorNotSupported when the shape has none
 bool row_fast_supported(const Geom& g);
+bool col_tma_length(int ny);  // lengths of the planar TMA column pass
 cudaError_t launch_row_fast(const Geom& g, RowMode mode, const float2* tw_z, const float2* maps, const float2* x,
                             float2* t, float2* out, cudaStream_t st);
 cudaError_t launch_col_normal_fast(const Geom& g, const float2* tw_y, const float* psi, float2* t, cudaStream_t st);

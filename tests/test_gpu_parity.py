@@ -289,16 +289,18 @@ def test_solve_host_io_pipelined_matches_device(T):
     assert np.allclose(host_res, dev_res, rtol=1e-6, atol=0)
 
 
-@pytest.mark.parametrize("S,ny,nz,C,M", [(4, 64, 48, 8, 1), (4, 128, 128, 8, 1), (8, 256, 160, 12, 1), (3, 60, 64, 5, 2)])
-def test_solve_host_io_matches_device_where_coils_are_split(T, S, ny, nz, C, M):
-    """Launches small enough that several CTAs share a row band's coils: the chunks of a host-buffer
-    solve add the coils in the order of the device-buffer solve, so the results are bitwise equal."""
-    rng, phi, mask, maps = random_problem(S + ny + nz, S, ny, nz, C, 12, 4, M)
-    y = crandn(rng, S, C, 4, ny, nz) * 0.05
+@pytest.mark.parametrize("S,ny,nz,C,M,K", [(4, 64, 48, 8, 1, 4), (4, 128, 128, 8, 1, 4), (8, 256, 160, 12, 1, 4), (3, 60, 64, 5, 2, 4),
+                                           (40, 60, 64, 3, 1, 2)])
+def test_solve_host_io_matches_device_whatever_the_launch(T, S, ny, nz, C, M, K):
+    """Launches small enough that several CTAs share a row band's coils, and scans whose passes are chosen
+    by the number of slices: the chunks of a host-buffer solve take the passes and the order of the sums
+    of the device-buffer solve, so the results are bitwise equal."""
+    rng, phi, mask, maps = random_problem(S + ny + nz, S, ny, nz, C, 12, K, M)
+    y = crandn(rng, S, C, K, ny, nz) * 0.05
     kw = dict(block=8, lam=0.02, iters=6, seed=4)
     with make_plan(T, phi, mask, maps, **kw) as p:
         dev_out = host(p.solve(c64(y), T.KSPACE_PROJ))
-    d = T.make_dims(ny, nz, C, 12, 4, nslices=S, nmaps=M, flags=T.HOST_IO, **kw)
+    d = T.make_dims(ny, nz, C, 12, K, nslices=S, nmaps=M, flags=T.HOST_IO, **kw)
     with T.Plan(d, phi.astype(np.float32), mask.astype(np.uint8), maps.astype(np.complex64)) as p:
         host_out = p.solve(y.astype(np.complex64), T.KSPACE_PROJ)
     assert np.array_equal(host_out.astype(np.complex128), dev_out)

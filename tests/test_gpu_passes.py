@@ -90,6 +90,9 @@ def test_per_echo_and_projected_forms(T, S, ny, nz, C, Tn, K, M):  # noqa: F811
     (1, 300, 250, 2, 8, 1),   # eight images of 250-point rows: the three-stage passes
     (1, 512, 400, 1, 4, 1),
     (1, 250, 60, 3, 5, 1), (1, 500, 48, 2, 5, 2), (1, 450, 52, 1, 5, 1),  # 25 items of 20 threads: most threads a column CTA has
+    # fewer than four images on the planar row lengths, both sides of every line of the choice of layout
+    (8, 180, 160, 5, 3, 1), (1, 180, 160, 5, 3, 1), (2, 200, 128, 3, 2, 2), (14, 64, 48, 9, 2, 1), (70, 64, 48, 6, 2, 1),
+    (40, 100, 48, 4, 3, 1), (130, 16, 48, 1, 3, 1), (2, 48, 96, 3, 1, 1), (26, 54, 64, 4, 1, 2),
     (1, 64, 338, 2, 4, 1), (1, 90, 512, 2, 2, 1), (1, 390, 16, 2, 2, 1),  # three radix stages: A x in one column pass, and in two
 ])
 def test_two_radix_passes(T, S, ny, nz, C, K, M):  # noqa: F811
