@@ -91,8 +91,9 @@ static_assert(col_threads_fit(), "every column CTA within its launch bounds");
 
 // Persistent CTAs over contiguous runs of the (column chunk, slice x coil) list, column-chunk major:
 // Psi of a chunk's columns is copied to shared memory once per run.  The next tile streams in by
-// cp.async while the current one is transformed.
-template <int KC>
+// cp.async while the current one is transformed.  FWD: the passes that begin with the forward transform;
+// the others take k-space (compiled apart, so that neither costs the other registers).
+template <int KC, bool FWD>
 __global__ void __launch_bounds__(kColThreads, KC == 4 ? 3 : 2)
     k_col_any(Geom g, AnyCol a, const float2* __restrict__ tw_g, const float* __restrict__ psi, const float2* in,
               float2* out, int nsc, int ntiles) {
@@ -101,11 +102,10 @@ __global__ void __launch_bounds__(kColThreads, KC == 4 ? 3 : 2)
   const int wl = W == 4 ? 2 : 1;
   const long long NN = (long long)N * nz;
   const int rowlen = K * nz;  // values of one row of t
-  const bool fwd = a.mode == IL_NORMAL || a.mode == IL_FWD_PROJ || a.mode == IL_FWD_RAW;
   float2* tw = smem;  // [N]
   float2* bufs = smem + ((N + 1) & ~1);
   const int ts = (RA * QS + 1) & ~1;
-  int* ftab = reinterpret_cast<int*>(bufs + (fwd ? 2 : 1) * ts);  // position -> place << 10 | frequency
+  int* ftab = reinterpret_cast<int*>(bufs + (FWD ? 2 : 1) * ts);  // position -> place << 10 | frequency
   float* ps = reinterpret_cast<float*>(ftab + N);                 // [entry][position][w]
   for (int i = threadIdx.x; i < N; i += blockDim.x) {
     const int k1 = i / RB, k2 = i - k1 * RB;
@@ -137,16 +137,16 @@ __global__ void __launch_bounds__(kColThreads, KC == 4 ? 3 : 2)
   };
   pdl_wait();
   pdl_trigger();
-  if (fwd && lo < hi) issue(lo, bufs);
+  if (FWD && lo < hi) issue(lo, bufs);
   cp_async_commit();
   int have = -1;  // column chunk whose Psi is in shared memory
   for (int tile = lo; tile < hi; ++tile) {
     const int zt = tile / nsc, sc = tile - zt * nsc, z0 = zt * W;
     const long long tbase = (long long)sc * N * rowlen + (long long)zt * LK;
-    float2* buf = bufs + (fwd ? ((tile - lo) & 1) * ts : 0);
+    float2* buf = bufs + (FWD ? ((tile - lo) & 1) * ts : 0);
     cp_async_wait<0>();
     __syncthreads();  // tables and this tile are here; the previous tile is done
-    if (fwd) {
+    if constexpr (FWD) {
       if (tile + 1 < hi) issue(tile + 1, bufs + ((tile + 1 - lo) & 1) * ts);
       cp_async_commit();
       if (a.psi_sm && have != zt) {
@@ -157,15 +157,28 @@ __global__ void __launch_bounds__(kColThreads, KC == 4 ? 3 : 2)
         have = zt;  // read after at least two barriers
       }
     } else {  // k-space, centred and scaled, to the places where stage B leaves it
-      for (int p = item0; act && p < N; p += nitem) {
-        const int f = ftab[p] & 1023, k = e >> wl, w = e & (W - 1);
-        const float2 v = a.mode == IL_ADJ ? in[tbase + (long long)f * rowlen + e]
-                                          : in[((long long)sc * K + k) * NN + (long long)f * nz + z0 + w];
-        buf[(ftab[p] >> 10) + e] = cscale(v, scale * parity_sign(f + w));  // z0 is even
+      // More than four images: eight loads in flight per thread (the compiler keeps one behind the other's
+      // shared-memory store, which the array could alias): A^H from projected k-space, 240x128, K = 5, C = 15,
+      // 16 slices 925 -> 539 us.  Up to four images, with more items per round: 240x108, K = 2 35 -> 49 us.
+      constexpr int B = KC == 4 ? 1 : 8;
+      const int k = e >> wl, w = e & (W - 1);
+      const float2* src = a.mode == IL_ADJ ? in + tbase + e : in + ((long long)sc * K + k) * NN + z0 + w;
+      const int fstep = a.mode == IL_ADJ ? rowlen : nz;
+      for (int p = item0; act && p < N; p += B * nitem) {
+        float2 v[B];
+        int ft[B];
+#pragma unroll
+        for (int u = 0; u < B; ++u) {
+          ft[u] = p + u * nitem < N ? ftab[p + u * nitem] : -1;
+          if (ft[u] >= 0) v[u] = src[(ft[u] & 1023) * fstep];
+        }
+#pragma unroll
+        for (int u = 0; u < B; ++u)
+          if (ft[u] >= 0) buf[(ft[u] >> 10) + e] = cscale(v[u], scale * parity_sign((ft[u] & 1023) + w));  // z0 is even
       }
       __syncthreads();
     }
-    if (fwd) {
+    if constexpr (FWD) {
       for (int j = item0; act && j < RB; j += nitem) {
         switch (RA) {
 #define X(R) case R: any_stage<R, false, false, false>(buf, j * LK + e, QS, tw, 0); break;
@@ -458,15 +471,15 @@ cudaError_t launch_col_any(const Geom& g, int W, IlPass pass, const float2* tw_y
   if (!col_any_plan(g, W, pass, &a, &sm)) return cudaErrorNotSupported;
   const int threads = col_threads(g.K * W, std::max(a.RA, a.RB));
   const long long nsc = (long long)g.S * g.C, ntiles = nsc * (g.nz / W);
-  const void* kern = g.K <= 4 ? (const void*)k_col_any<4> : (const void*)k_col_any<8>;
+  const bool fwd = pass == IL_NORMAL || pass == IL_FWD_PROJ || pass == IL_FWD_RAW;
+  auto kern = g.K <= 4 ? (fwd ? k_col_any<4, true> : k_col_any<4, false>) : (fwd ? k_col_any<8, true> : k_col_any<8, false>);
   int nsm = 0, per = 0;
-  cudaError_t e = smem_optin(kern, 220 * 1024);
+  cudaError_t e = smem_optin((const void*)kern, 220 * 1024);
   if (e == cudaSuccess) e = sm_count(&nsm);
-  if (e == cudaSuccess) e = ctas_per_sm(kern, threads, sm, &per);
+  if (e == cudaSuccess) e = ctas_per_sm((const void*)kern, threads, sm, &per);
   if (e != cudaSuccess) return e;
   const int grid = (int)std::min<long long>(ntiles, (long long)nsm * per);
-  return launch_pdl(g.K <= 4 ? k_col_any<4> : k_col_any<8>, dim3(grid), threads, sm, st, g, a, tw_y, psi, in, out,
-                    (int)nsc, (int)ntiles);
+  return launch_pdl(kern, dim3(grid), threads, sm, st, g, a, tw_y, psi, in, out, (int)nsc, (int)ntiles);
 }
 
 template <int MODE, int MC>
