@@ -53,13 +53,16 @@ __device__ __forceinline__ float cta_quotient(const double* num, const double* d
 }
 #define CG_INDEX(i) (2 * ((long long)(blockIdx.x * kCgPerThread + (i)) * kCgThreads + threadIdx.x))
 
+// None of these kernels triggers early: the row pass that follows would pile up on the SMs that empty first
+// (one slice of 240x240, K = 3, C = 16: ADMM 616 us with the triggers, 481 without; 560 launched one after
+// the other).  32 slices of 192x192, C = 16: 6.86 ms both ways.
+
 // r = aty + rho (v - u) - w - rho x  (w = A^H A x);  p = r;  rr[s] += |r|^2
 __global__ void __launch_bounds__(kCgThreads) k_cg_init(long long L, const float2* x, const float2* w,
                                                        const float2* aty, const float2* v, const float2* u,
                                                        float rho, float2* __restrict__ r, float2* __restrict__ p,
                                                        double* rr) {
   pdl_wait();
-  pdl_trigger();
   const long long base = (long long)blockIdx.y * L;
   float4 xa[kCgPerThread], wa[kCgPerThread], ya[kCgPerThread], va[kCgPerThread], ua[kCgPerThread];
 #pragma unroll
@@ -92,7 +95,6 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_init(long long L, const float
 __global__ void __launch_bounds__(kCgThreads) k_cg_dot(long long L, const float2* p, const float2* w, float rho,
                                                       double* pq) {
   pdl_wait();
-  pdl_trigger();
   const long long base = (long long)blockIdx.y * L;
   float4 pa[kCgPerThread], wa[kCgPerThread];
 #pragma unroll
@@ -118,7 +120,6 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_step(long long L, float2* x, 
                                                        const double* rr, const double* pq,
                                                        double* rr_new) {
   pdl_wait();
-  pdl_trigger();
   const int s = blockIdx.y;
   const long long base = (long long)s * L;
   float4 pa[kCgPerThread], wa[kCgPerThread], xa[kCgPerThread], ra[kCgPerThread];
@@ -158,7 +159,6 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_dir(long long L, const float2
                                                       const double* rr, const double* rr_new,
                                                       double* pq, double* rr_next) {
   pdl_wait();
-  pdl_trigger();
   const int s = blockIdx.y;
   const long long base = (long long)s * L;
   float4 ra[kCgPerThread], pa[kCgPerThread];
