@@ -317,11 +317,18 @@ __device__ __forceinline__ void row_t_fwd(const float2* ex, int xs, const float2
     for (int q = 0; q < R; ++q) t[any_off(i + q * zs, wl, LK)] = v[q];
   }
 }
-template <int R>
-__device__ __forceinline__ void row_t_adj(float2* ex, int xs, int i, const float2* t, int zs, int wl, int LK, bool on) {
+// (the loads are issued before the barrier `sync`, which every thread takes: A^H A of 50 slices of 100x160,
+// K = 6, M = 2 784 -> 760 us; not those of radix 25, which the registers do not hold across it; in: the thread
+// has an item)
+template <int R, typename Sync>
+__device__ __forceinline__ void row_t_adj(float2* ex, int xs, int i, const float2* t, int zs, int wl, int LK, bool on,
+                                          bool in, Sync sync) {
+  if constexpr (R > 20) sync();
   float2 v[R];
 #pragma unroll
   for (int q = 0; q < R; ++q) v[q] = on ? t[any_off(i + q * zs, wl, LK)] : make_float2(0.f, 0.f);
+  if constexpr (R <= 20) sync();
+  if (!in) return;
   dft_r<R, true>(v);
 #pragma unroll
   for (int q = 0; q < R; ++q) ex[q * xs] = v[q];
@@ -371,10 +378,13 @@ __global__ void __launch_bounds__(kRowThreads, MC == 1 ? 3 : 2)
       val[m][q] = MODE == ROW_FWD && on_i && q < RI ? x[img + (long long)m * K * NN + q * RT] : make_float2(0.f, 0.f);
   for (int c = 0; c < g.C; ++c) {
     const int buf = c & 1;
-    cp_async_wait<0>();
-    __syncthreads();  // coil c's maps are here, and nobody is in the previous coil any more
-    if (c + 1 < g.C) issue(c + 1, buf ^ 1);
-    cp_async_commit();
+    auto next_coil = [&] {
+      cp_async_wait<0>();
+      __syncthreads();  // coil c's maps are here, and nobody is in the previous coil any more
+      if (c + 1 < g.C) issue(c + 1, buf ^ 1);
+      cp_async_commit();
+    };
+    if (MODE == ROW_FWD) next_coil();
     const float2* mrow = mst + (buf * MC * rows + r) * N + item;
     if (MODE == ROW_FWD) {
       if (in_i) {
@@ -393,12 +403,10 @@ __global__ void __launch_bounds__(kRowThreads, MC == 1 ? 3 : 2)
         }
       }
     } else {
-      if (in_t) {
-        switch (RT) {
-#define X(R) case R: row_t_adj<R>(ex_t, nl, item, tp, RI, wl, LK, on_t); break;
-          T2SH_RADICES(X)
+      switch (RT) {
+#define X(R) case R: row_t_adj<R>(ex_t, nl, item, tp, RI, wl, LK, on_t, in_t, next_coil); break;
+        T2SH_RADICES(X)
 #undef X
-        }
       }
       __syncthreads();
       if (in_i) {
