@@ -53,9 +53,9 @@ __device__ __forceinline__ float cta_quotient(const double* num, const double* d
 }
 #define CG_INDEX(i) (2 * ((long long)(blockIdx.x * kCgPerThread + (i)) * kCgThreads + threadIdx.x))
 
-// None of these kernels triggers early: the row pass that follows would pile up on the SMs that empty first
-// (one slice of 240x240, K = 3, C = 16: ADMM 616 us with the triggers, 481 without; 560 launched one after
-// the other).  32 slices of 192x192, C = 16: 6.86 ms both ways.
+// These kernels trigger when a CTA's vectors are stored, not at their start: the row pass that follows would
+// pile up on the SMs that empty first (one slice of 240x240, K = 3, C = 16: ADMM 616 us with early triggers, 481
+// with late ones; 560 launched one after the other).  32 slices of 192x192, C = 16: 6.86 ms every way.
 
 // r = aty + rho (v - u) - w - rho x  (w = A^H A x);  p = r;  rr[s] += |r|^2
 __global__ void __launch_bounds__(kCgThreads) k_cg_init(long long L, const float2* x, const float2* w,
@@ -88,6 +88,7 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_init(long long L, const float
       acc += dot4(ra, ra);
     }
   }
+  pdl_trigger();
   block_add((double)acc, rr + blockIdx.y);
 }
 
@@ -111,6 +112,7 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_dot(long long L, const float2
     if (CG_INDEX(i) < L)
       acc += pa[i].x * (wa[i].x + rho * pa[i].x) + pa[i].y * (wa[i].y + rho * pa[i].y) +
              pa[i].z * (wa[i].z + rho * pa[i].z) + pa[i].w * (wa[i].w + rho * pa[i].w);
+  pdl_trigger();
   block_add((double)acc, pq + blockIdx.y);
 }
 
@@ -150,6 +152,7 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_step(long long L, float2* x, 
       acc += dot4(ra[i], ra[i]);
     }
   }
+  pdl_trigger();
   block_add((double)acc, rr_new + s);
 }
 
@@ -182,6 +185,7 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_dir(long long L, const float2
       st4(p, base + e, pa[i]);
     }
   }
+  pdl_trigger();
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     pq[s] = 0.0;
     rr_next[s] = 0.0;
